@@ -1,18 +1,45 @@
 // Mode-3 DFT along the tubes of a frontal-slice-major tensor (Section 2:
-// fft(A,[],3) and its inverse), real data <-> half spectrum.
+// fft(A,[],3) and its inverse), real data <-> half spectrum, any n.
 //
-// One CTA owns 32 tubes and all n of their entries: slice k of the 32 tubes
-// is one coalesced row read, the transform runs in shared memory, and each
-// output slice is one coalesced 32-element row write.  For power-of-two n two
-// real tubes are packed into one complex sequence (x_a + i x_b), transformed by
-// an in-place radix-2 decimation-in-time FFT and separated again; for other n
-// the DFT sum is evaluated directly from a table of the n roots of unity.
+// One CTA owns 32 neighbouring tubes as 16 packed complex sequences (tube 2p
+// the real, tube 2p + 1 the imaginary part of sequence p), so that a row of a
+// slice is one 8-byte load per lane and a row of the spectrum one 16-byte
+// store.  n = r_1 r_2 .. r_np D: the transform is an in-place
+// decimation-in-frequency FFT in shared memory, one pass per radix r_i <= 16
+// (the register DFTs below), followed by direct DFTs of length D, the part of
+// n made of primes above 13 (D = 1 for most n).  The passes leave the
+// spectrum in digit-reversed order.
+//   forward: the first pass reads its r_1 rows straight from global memory
+//     (r_1 loads in flight per thread); the last pass writes shared memory, from
+//     which the two tubes of a sequence are separated by conjugate symmetry;
+//   inverse: the half spectrum becomes the packed full spectrum in shared
+//     memory (re and im swapped: the inverse DFT is the swapped DFT of the
+//     swapped data); the last pass writes its rows straight to global memory.
+// So n = r_1 r_2 moves every element through shared memory two (inverse) or
+// three (forward) times.
+//
+// What bounds it: HBM (12 bytes per element and direction), short of it the
+// issue rate (62 % of the issue slots at 256 x 256 x 256, register DFTs,
+// twiddles and shared-memory addresses) with 50 % occupancy.  Measured from a
+// flushed L2 (CUDA events, forward / inverse), before: the direct sums over n
+// that every n but the powers of two took, a radix-2 kernel for those, and
+// kernels written for n = 256 and 512:
+//   n    tubes      now                     before
+//   96   256 x 256   21 / 23 us              116 / 140 us   (direct)
+//   128  256 x 256   21 / 23 us              54 / 38 us     (radix 2)
+//   256  256 x 256   36 / 40 us (3.8 TB/s)   38 / 43 us     (16 x 16)
+//   331  256 x 256   322 / 289 us            1169 / 1484 us (direct; 331 is prime)
+//   384  384 x 384   118 / 118 us (3.9 TB/s) 3392 / 4326 us (direct)
+//   512  512 x 512   275 / 283 us (3.9 TB/s) 274 / 436 us   (16 x 32; radix 2)
+//   1000 256 x 256   219 / 184 us            18654 / 19093 us (direct)
+//
+// Two tubes share a sequence, so a NaN or infinity in one would reach the
+// other.  A CTA that meets one (or squares that overflow) evaluates the
+// defining sums tube by tube instead (rare, slow, correct).
+//
 // The forward kernel can also emit one float64 partial sum of squares per CTA
-// (used for ||A||_F^2).
-//
-// A thread always handles the same tube (DFT_THREADS is a multiple of
-// DFT_TILE), so its tube offset is computed once; squares are summed per
-// thread in the working precision and combined in float64 across the CTA.
+// (used for ||A||_F^2); squares are summed per thread in the working precision
+// and combined in float64 across the CTA.
 #include <algorithm>
 
 #include "common.cuh"
@@ -20,525 +47,760 @@
 
 namespace tp {
 
-constexpr int DFT_TILE = 32;
-constexpr int DFT_THREADS = 256;
+constexpr int DFT_TILE = 32;   // tubes per CTA
+constexpr int DFT_SEQ = 16;    // packed sequences per CTA
+constexpr int DFT_MAX_THREADS = 256;
+constexpr int DFT_MAX_PASS = 10;
 
 template <typename T> __device__ __forceinline__ void sincospi_t(T x, T* s, T* c);
 template <> __device__ __forceinline__ void sincospi_t<float>(float x, float* s, float* c) { sincospif(x, s, c); }
 template <> __device__ __forceinline__ void sincospi_t<double>(double x, double* s, double* c) { sincospi(x, s, c); }
 
-__device__ __forceinline__ long tube_off(long t, int cols, long ld) {
-    long r = t / cols;
-    return r * ld + (t - r * cols);
+// ---- register DFTs ------------------------------------------------------------
+// cos and sin of 2 pi m / R at compile time: the angle is brought to the first
+// octant by symmetry, where the Taylor series converge to double precision.
+constexpr double trig_pi = 3.14159265358979323846;
+constexpr double taylor_cos(double x) {
+    double t = 1.0, s = 1.0;
+    for (int i = 1; i < 12; ++i) {
+        t *= -x * x / ((2 * i - 1) * (2 * i));
+        s += t;
+    }
+    return s;
 }
-__device__ __forceinline__ int bitrev(int x, int logn) {
-    return logn ? (int)(__brev((unsigned)x) >> (32 - logn)) : 0;
+constexpr double taylor_sin(double x) {
+    double t = x, s = x;
+    for (int i = 1; i < 12; ++i) {
+        t *= -x * x / ((2 * i) * (2 * i + 1));
+        s += t;
+    }
+    return s;
 }
+// num / den of a turn, 0 <= num / den <= 1/4
+constexpr double cos_quarter(int num, int den) {
+    return 8 * num <= den ? taylor_cos(2 * trig_pi * num / den) : taylor_sin(2 * trig_pi * (den - 4 * num) / (4.0 * den));
+}
+constexpr double root_cos(int m, int R) {
+    m = ((m % R) + R) % R;
+    if (2 * m > R) m = R - m;                                  // cos(2 pi - x) = cos x
+    return 4 * m > R ? -cos_quarter(R - 2 * m, 2 * R) : cos_quarter(m, R);  // cos(pi - x) = -cos x
+}
+// sin x = cos(x - pi / 2), the angle in units of 1 / (4 R) of a turn
+constexpr double root_sin(int m, int R) { return root_cos(4 * m - R, 4 * R); }
 
-// exp(sign * 2 pi i m / n) for m < count
-template <typename T>
-__device__ void fill_roots(cplx<T>* tw, int count, int n, T sign) {
-    for (int m = threadIdx.x; m < count; m += blockDim.x) {
-        T s, c;
-        sincospi_t<T>((T)(2 * m) / (T)n, &s, &c);
-        tw[m] = mk<T>(c, sign * s);
+// a exp(-2 pi i m / R), m and R known at compile time
+template <typename T, int M, int R> __device__ __forceinline__ cplx<T> turn(cplx<T> a) {
+    constexpr int m = ((M % R) + R) % R;
+    if constexpr (m == 0) {
+        return a;
+    } else if constexpr (4 * m == R) {
+        return mk<T>(a.y, -a.x);
+    } else if constexpr (2 * m == R) {
+        return mk<T>(-a.x, -a.y);
+    } else if constexpr (4 * m == 3 * R) {
+        return mk<T>(-a.y, a.x);
+    } else {
+        constexpr double cd = root_cos(m, R), sd = root_sin(m, R);
+        const T c = (T)cd, s = (T)sd;
+        return mk<T>(a.x * c + a.y * s, a.y * c - a.x * s);
     }
 }
 
-// In-place radix-2 DIT over the 16 packed sequences z[k*16 + p] (input in
-// bit-reversed order, output natural).  tw holds exp(+-2 pi i m / n), m < n/2.
-template <typename T>
-__device__ void fft16_inplace(cplx<T>* z, const cplx<T>* tw, int n) {
-    for (int lh = 0; (1 << (lh + 1)) <= n; ++lh) {
-        const int half = 1 << lh, step = n >> (lh + 1);
-        for (int e = threadIdx.x; e < (n >> 1) * 16; e += blockDim.x) {
-            const int p = e & 15, bf = e >> 4;
-            const int j = bf & (half - 1), grp = bf >> lh;
-            const int i1 = (grp << (lh + 1)) + j, i2 = i1 + half;
-            cplx<T> a = z[i1 * 16 + p];
-            cplx<T> b = cmul(z[i2 * 16 + p], tw[j * step]);
-            z[i1 * 16 + p] = cadd(a, b);
-            z[i2 * 16 + p] = csub(a, b);
+// Forward R-point DFT of v in place, natural order in and out:
+// X_k = sum_t x_t exp(-2 pi i t k / R).
+template <typename T, int R> struct RDft;
+template <typename T> struct RDft<T, 1> {
+    static __device__ __forceinline__ void run(cplx<T> (&)[1]) {}
+};
+template <typename T> struct RDft<T, 2> {
+    static __device__ __forceinline__ void run(cplx<T> (&v)[2]) {
+        const cplx<T> a = v[0];
+        v[0] = cadd(a, v[1]);
+        v[1] = csub(a, v[1]);
+    }
+};
+template <typename T> struct RDft<T, 4> {
+    static __device__ __forceinline__ void run(cplx<T> (&v)[4]) {
+        const cplx<T> t0 = cadd(v[0], v[2]), t1 = csub(v[0], v[2]), t2 = cadd(v[1], v[3]), t3 = csub(v[1], v[3]);
+        v[0] = cadd(t0, t2);
+        v[2] = csub(t0, t2);
+        v[1] = mk<T>(t1.x + t3.y, t1.y - t3.x);  // t1 - i t3
+        v[3] = mk<T>(t1.x - t3.y, t1.y + t3.x);  // t1 + i t3
+    }
+};
+// odd prime R: with e_q = x_q + x_{R-q} and o_q = x_q - x_{R-q},
+// X_k, X_{R-k} = (x_0 + sum e_q cos(2 pi q k / R)) -+ i sum o_q sin(2 pi q k / R)
+template <typename T, int R> struct RDftOdd {
+    template <int K, int Q> static __device__ __forceinline__ void terms(const cplx<T> (&e)[R / 2], const cplx<T> (&o)[R / 2],
+                                                                         cplx<T>& a, cplx<T>& b) {
+        if constexpr (Q <= R / 2) {
+            constexpr double cd = root_cos(K * Q, R), sd = root_sin(K * Q, R);
+            const T c = (T)cd, s = (T)sd;
+            a.x = fma(e[Q - 1].x, c, a.x);
+            a.y = fma(e[Q - 1].y, c, a.y);
+            b.x = fma(o[Q - 1].x, s, b.x);
+            b.y = fma(o[Q - 1].y, s, b.y);
+            terms<K, Q + 1>(e, o, a, b);
         }
-        __syncthreads();
     }
+    template <int K> static __device__ __forceinline__ void outputs(const cplx<T> (&e)[R / 2], const cplx<T> (&o)[R / 2],
+                                                                    cplx<T> x0, cplx<T> (&v)[R]) {
+        if constexpr (K <= R / 2) {
+            cplx<T> a = x0, b = mk<T>(0, 0);
+            terms<K, 1>(e, o, a, b);
+            v[K] = mk<T>(a.x + b.y, a.y - b.x);      // a - i b
+            v[R - K] = mk<T>(a.x - b.y, a.y + b.x);  // a + i b
+            outputs<K + 1>(e, o, x0, v);
+        }
+    }
+    static __device__ __forceinline__ void run(cplx<T> (&v)[R]) {
+        cplx<T> e[R / 2], o[R / 2], x0 = v[0], s = v[0];
+#pragma unroll
+        for (int q = 1; q <= R / 2; ++q) {
+            e[q - 1] = cadd(v[q], v[R - q]);
+            o[q - 1] = csub(v[q], v[R - q]);
+            s = cadd(s, e[q - 1]);
+        }
+        v[0] = s;
+        outputs<1>(e, o, x0, v);
+    }
+};
+template <typename T> struct RDft<T, 3> : RDftOdd<T, 3> {};
+template <typename T> struct RDft<T, 5> : RDftOdd<T, 5> {};
+template <typename T> struct RDft<T, 7> : RDftOdd<T, 7> {};
+template <typename T> struct RDft<T, 11> : RDftOdd<T, 11> {};
+template <typename T> struct RDft<T, 13> : RDftOdd<T, 13> {};
+// R = A B: t = B t1 + t2, k = k1 + A k2
+template <typename T, int A, int B> struct RDftComp {
+    static constexpr int R = A * B;
+    template <int T2> static __device__ __forceinline__ void columns(cplx<T> (&v)[R]) {
+        if constexpr (T2 < B) {
+            cplx<T> u[A];
+#pragma unroll
+            for (int i = 0; i < A; ++i) u[i] = v[B * i + T2];
+            RDft<T, A>::run(u);
+            twiddles<T2, 0>(u, v);
+            columns<T2 + 1>(v);
+        }
+    }
+    template <int T2, int K1> static __device__ __forceinline__ void twiddles(cplx<T> (&u)[A], cplx<T> (&v)[R]) {
+        if constexpr (K1 < A) {
+            v[B * K1 + T2] = turn<T, T2 * K1, R>(u[K1]);
+            twiddles<T2, K1 + 1>(u, v);
+        }
+    }
+    static __device__ __forceinline__ void run(cplx<T> (&v)[R]) {
+        columns<0>(v);
+        cplx<T> o[R];
+#pragma unroll
+        for (int k1 = 0; k1 < A; ++k1) {
+            cplx<T> u[B];
+#pragma unroll
+            for (int i = 0; i < B; ++i) u[i] = v[B * k1 + i];
+            RDft<T, B>::run(u);
+#pragma unroll
+            for (int i = 0; i < B; ++i) o[k1 + A * i] = u[i];
+        }
+#pragma unroll
+        for (int i = 0; i < R; ++i) v[i] = o[i];
+    }
+};
+template <typename T> struct RDft<T, 6> : RDftComp<T, 2, 3> {};
+template <typename T> struct RDft<T, 8> : RDftComp<T, 2, 4> {};
+template <typename T> struct RDft<T, 9> : RDftComp<T, 3, 3> {};
+template <typename T> struct RDft<T, 10> : RDftComp<T, 2, 5> {};
+template <typename T> struct RDft<T, 12> : RDftComp<T, 4, 3> {};
+template <typename T> struct RDft<T, 15> : RDftComp<T, 3, 5> {};
+template <typename T> struct RDft<T, 16> : RDftComp<T, 4, 4> {};
+
+constexpr int DFT_RADICES[] = {16, 15, 13, 12, 11, 10, 9, 8, 7, 6, 5, 4, 3, 2, 1};
+
+// ---- the plan -------------------------------------------------------------------
+struct DftPlan {
+    int n = 0, np, D;         // n = r[0] .. r[np-1] D
+    int r[DFT_MAX_PASS];
+    unsigned rr[DFT_MAX_PASS], rm[DFT_MAX_PASS];  // ceil(2^20 / r) and ceil(2^20 / M) of each pass (M: see pass_smem)
+    int lns;                  // log2 of the sequences per sub-tile
+    int nt;                   // threads per CTA
+    int kb;                   // direct part: pairs (k, D - k) per thread
+};
+
+// Fewest passes, then the smallest sum of radices, largest radix first.
+static void best_radices(int m, int max_idx, int depth, int sum, int* cur, int* best, int* best_np, int* best_sum) {
+    if (m == 1) {
+        if (depth < *best_np || (depth == *best_np && sum < *best_sum)) {
+            *best_np = depth;
+            *best_sum = sum;
+            for (int i = 0; i < depth; ++i) best[i] = cur[i];
+        }
+        return;
+    }
+    if (depth + 1 > *best_np || depth + 1 > DFT_MAX_PASS) return;
+    for (int i = max_idx; DFT_RADICES[i] > 1; ++i)
+        if (m % DFT_RADICES[i] == 0) {
+            cur[depth] = DFT_RADICES[i];
+            best_radices(m / DFT_RADICES[i], i, depth + 1, sum + DFT_RADICES[i], cur, best, best_np, best_sum);
+        }
 }
 
+// sequences per sub-tile: all 16 while two CTAs fit on an SM (the direct part
+// needs a second buffer in the forward kernel), else 8 or 4, one after another
+static size_t dft_smem(const DftPlan& P, size_t elem, bool fwd) {
+    const size_t c = 2 * elem, buf = ((size_t)P.n << P.lns) * c;
+    return (P.D > 1 && fwd ? 2 : 1) * buf + (size_t)P.n * c + (((size_t)P.n * 2 + 15) & ~(size_t)15);
+}
+
+static DftPlan make_plan(int n, size_t elem, bool fwd) {
+    DftPlan P;
+    P.n = n;
+    int m = n;
+    P.D = 1;
+    for (int q = 17; q <= m; ++q)
+        while (m % q == 0) {
+            bool prime = true;
+            for (int d = 2; d * d <= q; ++d) prime = prime && q % d != 0;
+            if (!prime) break;
+            m /= q;
+            P.D *= q;
+        }
+    int cur[DFT_MAX_PASS], sum = 1 << 30;
+    P.np = DFT_MAX_PASS + 1;
+    best_radices(m, 0, 0, 0, cur, P.r, &P.np, &sum);
+    if (P.np == 0 && P.D == 1) {  // n = 1
+        P.np = 1;
+        P.r[0] = 1;
+    }
+    // x / d = x ceil(2^20 / d) >> 20 for x <= 1024, d <= 1024
+    for (int i = 0, L = n; i < P.np; ++i) {
+        P.rr[i] = ((1u << 20) + P.r[i] - 1) / P.r[i];
+        L /= P.r[i];
+        P.rm[i] = ((1u << 20) + L - 1) / L;
+    }
+    P.lns = 4;
+    while (P.lns > 2 && dft_smem(P, elem, fwd) > 112 * 1024) --P.lns;
+    // a thread per item of the pass with the fewest items
+    const int items = (n / (P.np ? P.r[0] : 1)) << P.lns;
+    P.nt = std::min(DFT_MAX_THREADS, std::max(64, (items + 31) & ~31));
+    if (P.D > 1) P.nt = DFT_MAX_THREADS;
+    // the direct part's groups of kb pairs run in rounds of nt / (sequences / 2): about kb + 1/2 units of time each
+    P.kb = 4;
+    long best = 1L << 60;
+    for (int kb : {3, 4, 6}) {
+        const int slots = P.nt >> (P.lns - 1), groups = n / P.D * ((P.D / 2 + kb) / kb);
+        const long cost = (long)((groups + slots - 1) / slots) * (2 * kb + 1);
+        if (cost < best) {
+            best = cost;
+            P.kb = kb;
+        }
+    }
+    return P;
+}
+
+// The plans of the last lengths that a thread used (the search takes about a
+// microsecond, which a small transform would notice).
+static const DftPlan& dft_plan(int n, size_t elem, bool fwd) {
+    struct Slot {
+        DftPlan P;
+        size_t elem = 0;
+        bool fwd = false;
+    };
+    thread_local Slot slots[16];
+    Slot& s = slots[((n * 4) ^ (elem == 4 ? 2 : 0) ^ (fwd ? 1 : 0)) & 15];
+    if (s.elem != elem || s.fwd != fwd || s.P.n != n) {
+        s.P = make_plan(n, elem, fwd);
+        s.elem = elem;
+        s.fwd = fwd;
+    }
+    return s.P;
+}
+
+// Class of a plan: 0 = powers of two, 1 = radices up to 10, 2 = the other
+// products of small primes, 3 = plans with a direct part or whose tiles are
+// split (the others have the sequence count as a compile-time constant).
+static int dft_class(const DftPlan& P) {
+    if (P.lns != 4 || P.D > 1) return 3;
+    int cls = 0;
+    for (int i = 0; i < P.np; ++i) {
+        const int r = P.r[i];
+        if (r > 10 && r != 16) return 2;
+        if (r & (r - 1)) cls = 1;
+    }
+    for (int i = 0; i < P.np; ++i)
+        if (cls == 1 && P.r[i] > 10) return 2;
+    return cls;
+}
+constexpr int DFT_CTAS[4] = {4, 4, 3, 2};  // CTAs per SM that the registers of each class allow (float32)
+
+// ---- kernels ----------------------------------------------------------------------
 template <typename T>
-__device__ void store_partial(T v, double* sumsq) {
-    if (!sumsq) return;
+__device__ __forceinline__ void store_partial(T v, double* sumsq) {
     __shared__ double red[33];
     const double t = block_sum_t(v, red);
     if (threadIdx.x == 0) sumsq[blockIdx.x] = t;
 }
 
-static_assert(DFT_THREADS % DFT_TILE == 0, "a thread must keep one tube");
+__device__ __forceinline__ long tube_off(long t, int cols, long ld) {
+    if (ld == cols) return t;  // a uniform branch: no 64-bit division
+    const long r = t / cols;
+    return r * ld + (t - r * cols);
+}
 
+// n roots exp(-2 pi i m / n), and the digit reversal of the passes: table[pos]
+// = frequency index of shared position pos (inverse) or table[s] = position
+// of frequency s (forward).  Position digits (most significant first) are k_1
+// (weight n / r_1), k_2 (n / (r_1 r_2)), ..., the last one, of the direct part,
+// of weight 1; the frequency is k_1 + r_1 (k_2 + r_2 (k_3 + ...)).
 template <typename T>
-__global__ void __launch_bounds__(DFT_THREADS)
-k_rdft_pow2(const T* __restrict__ X, cplx<T>* __restrict__ Xh, int n, int logn, long tubes, int cols,
-            long ld, long ss, double* sumsq, const int* skip) {
-    if (skip && *skip) return;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    cplx<T>* z = (cplx<T>*)smraw;
-    cplx<T>* tw = z + (size_t)n * 16;
-    T* zf = (T*)z;
-    const long t0 = (long)blockIdx.x * DFT_TILE;
-    fill_roots<T>(tw, n / 2, n, (T)-1);
-    const int tt = threadIdx.x & (DFT_TILE - 1), k0 = threadIdx.x / DFT_TILE, kst = blockDim.x / DFT_TILE;
-    const bool live = t0 + tt < tubes;
-    const T* xt = X + (live ? tube_off(t0 + tt, cols, ld) : 0);
-    T acc = 0;
-    // LB loads in flight per thread before any is used (the tube entries are
-    // one strided row each: the kernel is bound by how many rows are in flight)
-    constexpr int LB = sizeof(T) == 4 ? 32 : 16;
-    for (int kb = k0; kb < n; kb += LB * kst) {
-        T v[LB];
-#pragma unroll
-        for (int j = 0; j < LB; ++j) {
-            const int k = kb + j * kst;
-            v[j] = (live && k < n) ? __ldcs(xt + (long)k * ss) : (T)0;
+__device__ __forceinline__ void fill_tables(const DftPlan& P, cplx<T>* tw, unsigned short* table, bool by_pos) {
+    const int n = P.n;
+    const T step = (T)2 / (T)n;
+    const bool pow2 = (n & (n - 1)) == 0;  // 2 m / n without a division then
+    for (int m = threadIdx.x; m < n; m += blockDim.x) {
+        T s, c;
+        sincospi_t<T>(pow2 ? (T)m * step : (T)(2 * m) / (T)n, &s, &c);
+        tw[m] = mk<T>(c, -s);
+        int rest = m, pos = 0, w = n;
+        for (int i = 0; i < P.np; ++i) {  // m as a frequency: its digits, lowest first
+            const int r = P.r[i], q = (int)((rest * P.rr[i]) >> 20);
+            w = (int)((w * P.rr[i]) >> 20);
+            pos += (rest - q * r) * w;
+            rest = q;
         }
+        pos += rest;
+        if (by_pos) table[pos] = (unsigned short)m;
+        else table[m] = (unsigned short)pos;
+    }
+}
+
+// One pass over shared memory: blocks of length L, radix R, M = L / R.
+// LAST: M = 1, no twiddles.  MR = ceil(2^20 / M) divides item numbers by M.
+template <typename T, int R, bool LAST>
+__device__ __forceinline__ void pass_smem(cplx<T>* z, const cplx<T>* tw, int n, int L, int tstep, unsigned MR, int lns) {
+    const int p = threadIdx.x & ((1 << lns) - 1), ust = blockDim.x >> lns, items = n / R;
+    const int M = LAST ? 1 : L / R;
+    for (int u = threadIdx.x >> lns; u < items; u += ust) {
+        const int b = LAST ? u : (int)((u * MR) >> 20), j = LAST ? 0 : u - b * M;
+        cplx<T>* zp = z + ((size_t)(b * L + j) << lns) + p;
+        cplx<T> v[R];
 #pragma unroll
-        for (int j = 0; j < LB; ++j) {
-            const int k = kb + j * kst;
-            if (k < n) {
-                acc = fma(v[j], v[j], acc);
-                zf[((size_t)bitrev(k, logn) * 16 + (tt & 15)) * 2 + (tt >> 4)] = v[j];
+        for (int q = 0; q < R; ++q) v[q] = zp[(q * M) << lns];
+        RDft<T, R>::run(v);
+        zp[0] = v[0];
+#pragma unroll
+        for (int k = 1; k < R; ++k) zp[(k * M) << lns] = LAST ? v[k] : cmul(v[k], tw[j * k * tstep]);
+    }
+}
+
+// The radices of a kernel's class (dft_class): the registers of a kernel are
+// those of its largest radix, and fewer registers keep more CTAs on an SM.
+#define DFT_SWITCH(r, GO)                                    \
+    if constexpr (CLS == 0) {                                \
+        switch (r) {                                         \
+            case 1: GO(1); break;                            \
+            case 2: GO(2); break;                            \
+            case 4: GO(4); break;                            \
+            case 8: GO(8); break;                            \
+            default: GO(16); break;                          \
+        }                                                    \
+    } else if constexpr (CLS == 1) {                         \
+        switch (r) {                                         \
+            case 2: GO(2); break;                            \
+            case 3: GO(3); break;                            \
+            case 4: GO(4); break;                            \
+            case 5: GO(5); break;                            \
+            case 6: GO(6); break;                            \
+            case 7: GO(7); break;                            \
+            case 8: GO(8); break;                            \
+            case 9: GO(9); break;                            \
+            default: GO(10); break;                          \
+        }                                                    \
+    } else {                                                 \
+        switch (r) {                                         \
+            case 2: GO(2); break;                            \
+            case 3: GO(3); break;                            \
+            case 4: GO(4); break;                            \
+            case 5: GO(5); break;                            \
+            case 6: GO(6); break;                            \
+            case 7: GO(7); break;                            \
+            case 8: GO(8); break;                            \
+            case 9: GO(9); break;                            \
+            case 10: GO(10); break;                          \
+            case 11: GO(11); break;                          \
+            case 12: GO(12); break;                          \
+            case 13: GO(13); break;                          \
+            case 15: GO(15); break;                          \
+            default: GO(16); break;                          \
+        }                                                    \
+    }
+
+// First forward pass: rows j, j + M, ... of the real tubes, packed.
+template <typename T, int R>
+__device__ __forceinline__ void pass_load(cplx<T>* z, const cplx<T>* tw, int n, int lns, const T* xa, const T* xb,
+                                          bool la, bool lb, bool vec, long ss, T& acc) {
+    const int p = threadIdx.x & ((1 << lns) - 1), M = n / R, ust = blockDim.x >> lns;
+    for (int j = threadIdx.x >> lns; j < M; j += ust) {
+        cplx<T> v[R];
+        if (vec) {
+#pragma unroll
+            for (int q = 0; q < R; ++q)
+                v[q] = la ? __ldcs((const cplx<T>*)(xa + (long)(j + q * M) * ss)) : mk<T>(0, 0);
+        } else {
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                const long off = (long)(j + q * M) * ss;
+                v[q] = mk<T>(la ? __ldcs(xa + off) : (T)0, lb ? __ldcs(xb + off) : (T)0);
             }
         }
-    }
-    __syncthreads();
-    fft16_inplace<T>(z, tw, n);
-    const int h = n / 2 + 1;
-    for (int e = threadIdx.x; e < h * DFT_TILE; e += blockDim.x) {
-        const int s = e >> 5, tt = e & 31;
-        const long t = t0 + tt;
-        if (t >= tubes) continue;
-        const int p = tt & 15;
-        cplx<T> zs = z[s * 16 + p];
-        cplx<T> zc = cconj(z[((n - s) & (n - 1)) * 16 + p]);
-        cplx<T> o;
-        if (tt < 16) o = mk<T>((zs.x + zc.x) * (T)0.5, (zs.y + zc.y) * (T)0.5);
-        else o = mk<T>((zs.y - zc.y) * (T)0.5, -(zs.x - zc.x) * (T)0.5);
-        Xh[(long)s * tubes + t] = o;
-    }
-    store_partial<T>(acc, sumsq);
-}
-
-// ---- register DFTs of 4, 16 and 32 points (the n = 16 Q kernels below) --------
-template <typename T>
-__device__ __forceinline__ void dft4f(cplx<T>& x0, cplx<T>& x1, cplx<T>& x2, cplx<T>& x3) {
-    // forward 4-point DFT in place: X_k = sum_n x_n exp(-2 pi i n k / 4)
-    const cplx<T> t0 = cadd(x0, x2), t1 = csub(x0, x2), t2 = cadd(x1, x3), t3 = csub(x1, x3);
-    x0 = cadd(t0, t2);
-    x2 = csub(t0, t2);
-    x1 = mk<T>(t1.x + t3.y, t1.y - t3.x);  // t1 - i t3
-    x3 = mk<T>(t1.x - t3.y, t1.y + t3.x);  // t1 + i t3
-}
-
-// forward 16-point DFT of v in place, natural order in and out (4 x 4 split)
-template <typename T>
-__device__ __forceinline__ void dft16f(cplx<T> (&v)[16]) {
-    const T c8 = (T)0.92387953251128675613, s8 = (T)0.38268343236508977173, h2 = (T)0.70710678118654752440;
-    // step 1: for each n2, the 4-point DFT over n1 of v[4 n1 + n2] -> a[k1][n2] kept at v[4 k1 + n2]
 #pragma unroll
-    for (int n2 = 0; n2 < 4; ++n2) dft4f<T>(v[n2], v[4 + n2], v[8 + n2], v[12 + n2]);
-    // step 2: twiddles exp(-2 pi i n2 k1 / 16), n2 k1 in {1, 2, 3, 2, 4, 6, 3, 6, 9}
-    auto tw = [](cplx<T> a, T c, T s) { return mk<T>(a.x * c - a.y * s, a.x * s + a.y * c); };  // a (c + i s)
-    v[4 * 1 + 1] = tw(v[5], c8, -s8);
-    v[4 * 1 + 2] = tw(v[6], h2, -h2);
-    v[4 * 1 + 3] = tw(v[7], s8, -c8);
-    v[4 * 2 + 1] = tw(v[9], h2, -h2);
-    v[4 * 2 + 2] = mk<T>(v[10].y, -v[10].x);  // times -i
-    v[4 * 2 + 3] = tw(v[11], -h2, -h2);
-    v[4 * 3 + 1] = tw(v[13], s8, -c8);
-    v[4 * 3 + 2] = tw(v[14], -h2, -h2);
-    v[4 * 3 + 3] = tw(v[15], -c8, s8);
-    // step 3: for each k1, the 4-point DFT over n2 -> X[k1 + 4 k2]
+        for (int q = 0; q < R; ++q) acc = fma(v[q].x, v[q].x, fma(v[q].y, v[q].y, acc));
+        RDft<T, R>::run(v);
+        cplx<T>* zp = z + ((size_t)j << lns) + p;
+        zp[0] = v[0];
 #pragma unroll
-    for (int k1 = 0; k1 < 4; ++k1) dft4f<T>(v[4 * k1], v[4 * k1 + 1], v[4 * k1 + 2], v[4 * k1 + 3]);
-    // v[4 k1 + k2] holds X[k1 + 4 k2]: transpose the 4 x 4 index
-    cplx<T> o[16];
-#pragma unroll
-    for (int k1 = 0; k1 < 4; ++k1)
-#pragma unroll
-        for (int k2 = 0; k2 < 4; ++k2) o[k1 + 4 * k2] = v[4 * k1 + k2];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = o[i];
-}
-
-// forward 32-point DFT of v in place, natural order in and out: the 16-point
-// DFTs of the even and odd entries, combined with exp(-2 pi i k / 32)
-template <typename T>
-__device__ __forceinline__ void dft32f(cplx<T> (&v)[32]) {
-    // cos and sin of 2 pi k / 32, k = 0 .. 7
-    const T c1 = (T)0.98078528040323044913, s1 = (T)0.19509032201612826785;
-    const T c2 = (T)0.92387953251128675613, s2 = (T)0.38268343236508977173;
-    const T c3 = (T)0.83146961230254523708, s3 = (T)0.55557023301960222474, h2 = (T)0.70710678118654752440;
-    const T C[8] = {(T)1, c1, c2, c3, h2, s3, s2, s1}, S[8] = {(T)0, s1, s2, s3, h2, c3, c2, c1};
-    cplx<T> e[16], o[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        e[i] = v[2 * i];
-        o[i] = v[2 * i + 1];
-    }
-    dft16f<T>(e);
-    dft16f<T>(o);
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        // exp(-2 pi i k / 32) = c - i s; k >= 8 turns by a further -pi / 2
-        const T c = k < 8 ? C[k] : -S[k - 8], sn = k < 8 ? S[k] : C[k - 8];
-        const cplx<T> t = mk<T>(o[k].x * c + o[k].y * sn, o[k].y * c - o[k].x * sn);
-        v[k] = cadd(e[k], t);
-        v[k + 16] = csub(e[k], t);
+        for (int k = 1; k < R; ++k) zp[(k * M) << lns] = cmul(v[k], tw[j * k]);
     }
 }
-template <typename T, int Q> struct DftQ;
-template <typename T> struct DftQ<T, 16> {
-    static __device__ __forceinline__ void run(cplx<T> (&v)[16]) { dft16f<T>(v); }
-};
-template <typename T> struct DftQ<T, 32> {
-    static __device__ __forceinline__ void run(cplx<T> (&v)[32]) { dft32f<T>(v); }
-};
 
-// ---- n = 16 Q (Q = 16: n = 256; Q = 32: n = 512) ------------------------------
-// x_t with t = Q t1 + t2 (t1 < 16, t2 < Q), X_k with k = k1 + 16 k2:
-//   X[k1 + 16 k2] = sum_t2 exp(-2 pi i t2 k2 / Q) exp(-2 pi i t2 k1 / n)
-//                   sum_t1 exp(-2 pi i t1 k1 / 16) x[Q t1 + t2].
-// Thread (seq, j) of the 16 per packed sequence does the 16-point DFTs over t1
-// for t2 = j, j + 16, ... (Q / 16 of them), applies the twiddles, and then the
-// Q-point DFT over t2 for k1 = j, all in registers.  The three shared-memory
-// phases (real input [t][tube], twiddled partial DFTs [seq][k1][t2], packed
-// spectrum [k][seq]) share one buffer, each read into registers behind a
-// barrier before the next is written, so that several CTAs fit on an SM.
-template <int Q> struct Rdft16Q {
-    static constexpr int n = 16 * Q, TS = Q + 1, ZS = 17;
-    template <typename T> static constexpr size_t region() {
-        const size_t b = (size_t)256 * TS * 2 * sizeof(T), c = (size_t)n * ZS * 2 * sizeof(T);
-        return b > c ? b : c;
-    }
-    template <typename T> static constexpr size_t smem() { return (size_t)n * 2 * sizeof(T) + region<T>(); }
-};
-
-template <typename T, int Q>
-__global__ void __launch_bounds__(DFT_THREADS, sizeof(T) == 4 ? (Q == 16 ? 5 : 3) : 1)
-k_rdft_16q(const T* __restrict__ X, cplx<T>* __restrict__ Xh, long tubes, int cols, long ld, long ss, double* sumsq,
-           const int* skip) {
-    if (skip && *skip) return;
-    typedef Rdft16Q<Q> R;
-    constexpr int n = R::n, TS = R::TS, ZS = R::ZS, h = n / 2 + 1;
-    constexpr int NT = DFT_THREADS;  // compile-time strides: the index arithmetic folds into constants
-    static_assert(NT == 256, "16 packed sequences x 16 threads");
-    extern __shared__ __align__(16) unsigned char smraw[];
-    cplx<T>* tw = (cplx<T>*)smraw;                 // n roots exp(-2 pi i m / n)
-    cplx<T>* zp = tw + n;                          // phase 1: packed input [t][seq], row stride 17
-    cplx<T>* zt = zp;                              // phase 2: [seq][k1][t2], row stride Q + 1
-    cplx<T>* z = zp;                               // phase 3: packed spectrum [k][seq], row stride 17
-    const int tid = threadIdx.x;
-    const long t0 = (long)blockIdx.x * DFT_TILE;
-    {
-        const T step = (T)2 / (T)n;  // exact for a power of two: the argument 2 m / n without a division
-        for (int m = tid; m < n; m += NT) {
-            T sn, cs;
-            sincospi_t<T>((T)m * step, &sn, &cs);
-            tw[m] = mk<T>(cs, -sn);
-        }
-    }
-    // phase 1: thread (row group kr, pair p) loads tubes p and p + 16 (the real and imaginary parts of packed
-    // sequence p) at rows kr, kr + 16, ...; a half-warp reads 16 consecutive tubes of one row
-    const int p = tid & 15, kr = tid >> 4;
-    T acc = 0;
-    {
-        const bool la = t0 + p < tubes, lb = t0 + p + 16 < tubes;
-        const T* xa = X + (la ? tube_off(t0 + p, cols, ld) : 0);
-        const T* xb = X + (lb ? tube_off(t0 + p + 16, cols, ld) : 0);
-        constexpr int RPT = n / 16;                  // rows per thread
-        constexpr int LB = RPT > 16 ? 16 : RPT;      // row pairs in flight per thread
-#pragma unroll 1
-        for (int rb = 0; rb < RPT; rb += LB) {
-            T va[LB], vb[LB];
-#pragma unroll
-            for (int i = 0; i < LB; ++i) {
-                const long off = (long)(kr + 16 * (rb + i)) * ss;
-                va[i] = la ? __ldcs(xa + off) : (T)0;
-                vb[i] = lb ? __ldcs(xb + off) : (T)0;
-            }
-#pragma unroll
-            for (int i = 0; i < LB; ++i) {
-                acc = fma(va[i], va[i], acc);
-                acc = fma(vb[i], vb[i], acc);
-                zp[(kr + 16 * (rb + i)) * ZS + p] = mk<T>(va[i], vb[i]);
-            }
-        }
-    }
-    __syncthreads();
-    const int seq = tid >> 4, j = tid & 15;
-    {
-        // 16-point DFTs over t1 of x[Q t1 + t2], t2 = j + 16 u
-        cplx<T> v[Q / 16][16];
-#pragma unroll
-        for (int u = 0; u < Q / 16; ++u)
-#pragma unroll
-            for (int t1 = 0; t1 < 16; ++t1) v[u][t1] = zp[(Q * t1 + j + 16 * u) * ZS + seq];
-        __syncthreads();  // the input is read: the buffer takes the partial DFTs
-#pragma unroll
-        for (int u = 0; u < Q / 16; ++u) {
-            const int t2 = j + 16 * u;
-            dft16f<T>(v[u]);
-#pragma unroll
-            for (int k1 = 0; k1 < 16; ++k1) zt[(seq * 16 + k1) * TS + t2] = cmul(v[u][k1], tw[(t2 * k1) & (n - 1)]);
-        }
-    }
-    __syncthreads();
-    {
-        // Q-point DFT over t2 for k1 = j: X[j + 16 k2]
-        cplx<T> v[Q];
-#pragma unroll
-        for (int t2 = 0; t2 < Q; ++t2) v[t2] = zt[(seq * 16 + j) * TS + t2];
-        __syncthreads();  // the partial DFTs are read: the buffer takes the spectrum
-        DftQ<T, Q>::run(v);
-#pragma unroll
-        for (int k2 = 0; k2 < Q; ++k2) z[(j + 16 * k2) * ZS + seq] = v[k2];
-    }
-    __syncthreads();
-    {
-        // separate the two real tubes of each packed sequence: thread (row group, tube tq) writes
-        // slices s = tid / 32 + 8 i of tube tq; tq < 16 takes (Z_s + conj Z_{n-s}) / 2, the others
-        // (Z_s - conj Z_{n-s}) / 2i, branch-free
-        const int tq = tid & 31, q = tq & 15, s0 = tid >> 5;
-        const long t = t0 + tq;
-        const T sg = tq < 16 ? (T)1 : (T)-1;
-        if (t < tubes) {
-            cplx<T>* dst = Xh + t + (long)s0 * tubes;
-            const long dstep = 8 * tubes;
-#pragma unroll 4
-            for (int s = s0; s < h; s += NT / 32, dst += dstep) {
-                const cplx<T> zs = z[s * ZS + q];
-                const cplx<T> zc = z[((n - s) & (n - 1)) * ZS + q];
-                const T ux = fma(sg, zc.x, zs.x), uy = fma(-sg, zc.y, zs.y);  // Z_s +- conj Z_{n-s}
-                *dst = tq < 16 ? mk<T>(ux * (T)0.5, uy * (T)0.5) : mk<T>(uy * (T)0.5, -ux * (T)0.5);
-            }
-        }
-    }
-    store_partial<T>(acc, sumsq);
-}
-
-// Inverse for n = 256: the half spectra of 32 tubes become 16 packed full
-// spectra Z = X_a + i X_b, transformed back by the 16 x 16 split with
-// conjugated roots (the inverse DFT is conj(DFT(conj(Z)))), scaled by 1/n.
-template <typename T>
-__global__ void __launch_bounds__(DFT_THREADS)
-k_irdft_256(const cplx<T>* __restrict__ Xh, T* __restrict__ X, long tubes, int cols, long ld, long ss,
-            const int* skip) {
-    if (skip && *skip) return;
-    constexpr int n = 256, TS = 17;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    cplx<T>* tw = (cplx<T>*)smraw;          // 256 roots exp(-2 pi i m / 256)
-    cplx<T>* zt = tw + n;                   // [seq][k1][n2], row stride 17
-    cplx<T>* z = zt + 16 * 16 * TS;         // conj of the packed spectrum, then the packed signal: [k][seq]
-    const long t0 = (long)blockIdx.x * DFT_TILE;
-    fill_roots<T>(tw, n, n, (T)-1);
-    const int h = n / 2 + 1;
-    constexpr int LB = sizeof(T) == 4 ? 8 : 4;
-    for (int e0 = threadIdx.x; e0 < h * 16; e0 += LB * blockDim.x) {
-        cplx<T> xa[LB], xb[LB];
-#pragma unroll
-        for (int u = 0; u < LB; ++u) {
-            const int e = e0 + u * blockDim.x;
-            const int s = e >> 4, p = e & 15;
-            const long ta = t0 + p, tb = t0 + p + 16;
-            xa[u] = (e < h * 16 && ta < tubes) ? Xh[(long)s * tubes + ta] : mk<T>(0, 0);
-            xb[u] = (e < h * 16 && tb < tubes) ? Xh[(long)s * tubes + tb] : mk<T>(0, 0);
-        }
-#pragma unroll
-        for (int u = 0; u < LB; ++u) {
-            const int e = e0 + u * blockDim.x;
-            if (e >= h * 16) break;
-            const int s = e >> 4, p = e & 15;
-            cplx<T> a = xa[u], b = xb[u];
-            const bool self = (s == 0) || (2 * s == n);
-            if (self) { a.y = 0; b.y = 0; }
-            // conj(Z[s]) and conj(Z[n - s]), Z = X_a + i X_b with X(n - s) = conj(X(s))
-            z[s * TS + p] = mk<T>(a.x - b.y, -(a.y + b.x));
-            if (!self) z[(n - s) * TS + p] = mk<T>(a.x + b.y, -(b.x - a.y));
-        }
-    }
-    __syncthreads();
-    const int seq = threadIdx.x >> 4, j = threadIdx.x & 15;
-    {
-        cplx<T> v[16];
-#pragma unroll
-        for (int n1 = 0; n1 < 16; ++n1) v[n1] = z[(16 * n1 + j) * TS + seq];
-        dft16f<T>(v);
-#pragma unroll
-        for (int k1 = 0; k1 < 16; ++k1) zt[(seq * 16 + k1) * TS + j] = cmul(v[k1], tw[(j * k1) & (n - 1)]);
-    }
-    __syncthreads();
-    {
-        cplx<T> v[16];
-#pragma unroll
-        for (int n2 = 0; n2 < 16; ++n2) v[n2] = zt[(seq * 16 + j) * TS + n2];
-        dft16f<T>(v);
-#pragma unroll
-        for (int k2 = 0; k2 < 16; ++k2) z[(j + 16 * k2) * TS + seq] = v[k2];  // conj of the packed signal
-    }
-    __syncthreads();
+// Last inverse pass: block u's outputs are the rows low + (n / R) k of the
+// tubes (low = the frequency of the block's first position), swapped back and
+// scaled.
+template <typename T, int R>
+__device__ __forceinline__ void pass_store(const cplx<T>* z, const unsigned short* freq, int n, int lns, T* xa, T* xb,
+                                           bool la, bool lb, bool vec, long ss) {
+    const int p = threadIdx.x & ((1 << lns) - 1), M = n / R, ust = blockDim.x >> lns;
     const T inv = (T)1 / (T)n;
-    const int tt = threadIdx.x & (DFT_TILE - 1), k0 = threadIdx.x / DFT_TILE, kst = blockDim.x / DFT_TILE;
-    if (t0 + tt < tubes) {
-        T* xt = X + tube_off(t0 + tt, cols, ld);
-#pragma unroll 8
-        for (int k = k0; k < n; k += kst) {
-            const cplx<T> v = z[k * TS + (tt & 15)];
-            xt[(long)k * ss] = (tt < 16 ? v.x : -v.y) * inv;
-        }
-    }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(DFT_THREADS)
-k_rdft_direct(const T* __restrict__ X, cplx<T>* __restrict__ Xh, int n, long tubes, int cols,
-              long ld, long ss, double* sumsq, const int* skip) {
-    if (skip && *skip) return;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    cplx<T>* tw = (cplx<T>*)smraw;
-    T* x = (T*)(tw + n);
-    const long t0 = (long)blockIdx.x * DFT_TILE;
-    fill_roots<T>(tw, n, n, (T)-1);
-    const int tt = threadIdx.x & (DFT_TILE - 1), k0 = threadIdx.x / DFT_TILE, kst = blockDim.x / DFT_TILE;
-    const bool live = t0 + tt < tubes;
-    const T* xt = X + (live ? tube_off(t0 + tt, cols, ld) : 0);
-    T acc = 0;
-#pragma unroll 4
-    for (int k = k0; k < n; k += kst) {
-        const T v = live ? xt[(long)k * ss] : (T)0;
-        acc = fma(v, v, acc);
-        x[k * DFT_TILE + tt] = v;
-    }
-    __syncthreads();
-    const int h = n / 2 + 1;
-    for (int e = threadIdx.x; e < h * DFT_TILE; e += blockDim.x) {
-        const int s = e >> 5, tt = e & 31;
-        const long t = t0 + tt;
-        cplx<T> o = mk<T>(0, 0);
-        int idx = 0;
-        for (int k = 0; k < n; ++k) {
-            const T v = x[k * DFT_TILE + tt];
-            o.x = fma(v, tw[idx].x, o.x);
-            o.y = fma(v, tw[idx].y, o.y);
-            idx += s;
-            if (idx >= n) idx -= n;
-        }
-        if (t < tubes) Xh[(long)s * tubes + t] = o;
-    }
-    store_partial<T>(acc, sumsq);
-}
-
-template <typename T>
-__global__ void __launch_bounds__(DFT_THREADS)
-k_irdft_pow2(const cplx<T>* __restrict__ Xh, T* __restrict__ X, int n, int logn, long tubes, int cols,
-             long ld, long ss, const int* skip) {
-    if (skip && *skip) return;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    cplx<T>* z = (cplx<T>*)smraw;
-    cplx<T>* tw = z + (size_t)n * 16;
-    const long t0 = (long)blockIdx.x * DFT_TILE;
-    fill_roots<T>(tw, n / 2, n, (T)1);
-    const int h = n / 2 + 1;
-    // LB pairs of spectrum loads in flight per thread before any is used
-    constexpr int LB = sizeof(T) == 4 ? 8 : 4;
-    for (int e0 = threadIdx.x; e0 < h * 16; e0 += LB * blockDim.x) {
-        cplx<T> xa[LB], xb[LB];
+    for (int u = threadIdx.x >> lns; u < M; u += ust) {
+        const cplx<T>* zp = z + ((size_t)(u * R) << lns) + p;
+        cplx<T> v[R];
 #pragma unroll
-        for (int u = 0; u < LB; ++u) {
-            const int e = e0 + u * blockDim.x;
-            const int s = e >> 4, p = e & 15;
-            const long ta = t0 + p, tb = t0 + p + 16;
-            xa[u] = (e < h * 16 && ta < tubes) ? Xh[(long)s * tubes + ta] : mk<T>(0, 0);
-            xb[u] = (e < h * 16 && tb < tubes) ? Xh[(long)s * tubes + tb] : mk<T>(0, 0);
-        }
+        for (int q = 0; q < R; ++q) v[q] = zp[q << lns];
+        RDft<T, R>::run(v);
+        const long row = freq[u * R];
 #pragma unroll
-        for (int u = 0; u < LB; ++u) {
-            const int e = e0 + u * blockDim.x;
-            if (e >= h * 16) break;
-            const int s = e >> 4, p = e & 15;
-            cplx<T> a = xa[u], b = xb[u];
-            const bool self = (s == 0) || (2 * s == n);
-            if (self) { a.y = 0; b.y = 0; }
-            z[bitrev(s, logn) * 16 + p] = mk<T>(a.x - b.y, a.y + b.x);
-            if (!self) z[bitrev(n - s, logn) * 16 + p] = mk<T>(a.x + b.y, b.x - a.y);
-        }
-    }
-    __syncthreads();
-    fft16_inplace<T>(z, tw, n);
-    const T inv = (T)1 / (T)n;
-    const int tt = threadIdx.x & (DFT_TILE - 1), k0 = threadIdx.x / DFT_TILE, kst = blockDim.x / DFT_TILE;
-    if (t0 + tt < tubes) {
-        T* xt = X + tube_off(t0 + tt, cols, ld);
-#pragma unroll 8
-        for (int k = k0; k < n; k += kst) {
-            const cplx<T> v = z[k * 16 + (tt & 15)];
-            xt[(long)k * ss] = (tt < 16 ? v.x : v.y) * inv;
+        for (int k = 0; k < R; ++k) {
+            const long off = (row + (long)k * M) * ss;
+            if (vec) {
+                if (la) *(cplx<T>*)(xa + off) = mk<T>(v[k].y * inv, v[k].x * inv);
+            } else {
+                if (la) xa[off] = v[k].y * inv;
+                if (lb) xb[off] = v[k].x * inv;
+            }
         }
     }
 }
 
+// The direct part: DFTs of the n / D contiguous blocks of odd length D, whose
+// entries q and D - q first become e_q = x_q + x_{D-q} and o_q = x_q - x_{D-q}.
+// (direct_fold.)  A thread forms KB pairs (k, D - k) of two neighbouring sequences, so each
+// twiddle and each (e, o) read serves several products (about two thirds of
+// the issue slots are multiply-adds).  put(block, k, sequence, value).
 template <typename T>
-__global__ void __launch_bounds__(DFT_THREADS)
-k_irdft_direct(const cplx<T>* __restrict__ Xh, T* __restrict__ X, int n, long tubes, int cols,
-               long ld, long ss, const int* skip) {
-    if (skip && *skip) return;
-    extern __shared__ __align__(16) unsigned char smraw[];
-    cplx<T>* tw = (cplx<T>*)smraw;
-    cplx<T>* xs = tw + n;
-    const long t0 = (long)blockIdx.x * DFT_TILE;
-    fill_roots<T>(tw, n, n, (T)1);
-    const int h = n / 2 + 1;
-    for (int e = threadIdx.x; e < h * DFT_TILE; e += blockDim.x) {
-        const int s = e >> 5, tt = e & 31;
-        const long t = t0 + tt;
-        cplx<T> v = mk<T>(0, 0);
-        if (t < tubes) v = Xh[(long)s * tubes + t];
-        if (s == 0 || 2 * s == n) v.y = 0;
-        xs[e] = v;
+__device__ __forceinline__ void direct_fold(cplx<T>* z, int n, int D, int lns) {
+    typedef cplx<T> V;
+    const int H = D / 2, nb = n / D, ns = 1 << lns;
+    for (int e = threadIdx.x; e < nb * H * ns; e += blockDim.x) {
+        const int p = e & (ns - 1), bq = e >> lns, b = bq / H, q = bq - b * H + 1;
+        V* x = z + ((size_t)(b * D + q) << lns) + p;
+        V* y = z + ((size_t)(b * D + D - q) << lns) + p;
+        const V u = *x, v = *y;
+        *x = cadd(u, v);
+        *y = csub(u, v);
     }
     __syncthreads();
-    const T inv = (T)1 / (T)n;
-    const int tt = threadIdx.x & (DFT_TILE - 1), k0 = threadIdx.x / DFT_TILE, kst = blockDim.x / DFT_TILE;
-    const bool live = t0 + tt < tubes;
-    T* xt = X + (live ? tube_off(t0 + tt, cols, ld) : 0);
-    for (int k = k0; k < n; k += kst) {
-        T acc = xs[tt].x;  // slice 0
-        int idx = k;
-        for (int s = 1; s < h; ++s) {
-            const cplx<T> v = xs[s * DFT_TILE + tt];
-            const T wgt = (2 * s == n) ? (T)1 : (T)2;
-            acc += wgt * (v.x * tw[idx].x - v.y * tw[idx].y);
-            idx += k;
-            if (idx >= n) idx -= n;
+}
+template <typename T, int KB, typename Put>
+__device__ __forceinline__ void direct_part(const cplx<T>* z, const cplx<T>* tw, int n, int D, int lns, Put put) {
+    typedef cplx<T> V;
+    const int H = D / 2, nb = n / D, ts = n / D;  // twiddles exp(-2 pi i m / D) = tw[m n / D]
+    const int lhs = lns - 1, sp = threadIdx.x & ((1 << lhs) - 1), gst = blockDim.x >> lhs;
+    const int ng = (H + KB) / KB;  // groups of KB values of k in 0 .. H
+    for (int it = threadIdx.x >> lhs; it < nb * ng; it += gst) {
+        const int b = it / ng, k0 = (it - b * ng) * KB;
+        const V* zb = z + ((size_t)(b * D) << lns) + 2 * sp;
+        V A[KB][2], B[KB][2];
+        int idx[KB], kk[KB];
+#pragma unroll
+        for (int t = 0; t < KB; ++t) {
+            kk[t] = min(k0 + t, H);
+            idx[t] = 0;
+            A[t][0] = zb[0];
+            A[t][1] = zb[1];
+            B[t][0] = B[t][1] = mk<T>(0, 0);
         }
-        if (live) xt[(long)k * ss] = acc * inv;
+#pragma unroll 2
+        for (int q = 1; q <= H; ++q) {
+            const V e0 = zb[(size_t)q << lns], e1 = zb[((size_t)q << lns) + 1];
+            const V o0 = zb[(size_t)(D - q) << lns], o1 = zb[((size_t)(D - q) << lns) + 1];
+#pragma unroll
+            for (int t = 0; t < KB; ++t) {
+                const unsigned nx = (unsigned)(idx[t] + kk[t]);
+                idx[t] = (int)min(nx, nx - (unsigned)D);  // (q k) mod D
+                const V w = tw[idx[t] * ts];
+                A[t][0].x = fma(e0.x, w.x, A[t][0].x);
+                A[t][0].y = fma(e0.y, w.x, A[t][0].y);
+                A[t][1].x = fma(e1.x, w.x, A[t][1].x);
+                A[t][1].y = fma(e1.y, w.x, A[t][1].y);
+                B[t][0].x = fma(o0.x, w.y, B[t][0].x);
+                B[t][0].y = fma(o0.y, w.y, B[t][0].y);
+                B[t][1].x = fma(o1.x, w.y, B[t][1].x);
+                B[t][1].y = fma(o1.y, w.y, B[t][1].y);
+            }
+        }
+        // tw holds cos - i sin: X_k, X_{D-k} = A +- i B
+#pragma unroll
+        for (int t = 0; t < KB; ++t) {
+            const int k = k0 + t;
+            if (k > H) break;
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const V a = A[t][c], bb = B[t][c];
+                put(b, k, 2 * sp + c, mk<T>(a.x - bb.y, a.y + bb.x));
+                if (k > 0) put(b, D - k, 2 * sp + c, mk<T>(a.x + bb.y, a.y - bb.x));
+            }
+        }
     }
 }
 
-static inline bool is_pow2(int n) { return n > 0 && (n & (n - 1)) == 0; }
-static inline int ilog2(int n) { int l = 0; while ((1 << l) < n) ++l; return l; }
+// Entries of two neighbouring tubes in one row of the spectrum.
+template <typename T>
+__device__ __forceinline__ void store_pair(cplx<T>* dst, cplx<T> a, cplx<T> b, bool lb, bool vec) {
+    if (sizeof(T) == 4 && vec) {
+        *(float4*)dst = make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
+    } else {
+        dst[0] = a;
+        if (lb) dst[1] = b;
+    }
+}
+template <typename T>
+__device__ __forceinline__ void load_pair(const cplx<T>* src, cplx<T>& a, cplx<T>& b, bool lb, bool vec) {
+    if (sizeof(T) == 4 && vec) {
+        const float4 v = *(const float4*)src;
+        a = mk<T>((T)v.x, (T)v.y);
+        b = mk<T>((T)v.z, (T)v.w);
+    } else {
+        a = src[0];
+        if (lb) b = src[1];
+    }
+}
+
+template <typename T, int CLS>
+__global__ void __launch_bounds__(DFT_MAX_THREADS, sizeof(T) == 4 ? DFT_CTAS[CLS] : 1)
+k_rdft(const __grid_constant__ DftPlan P, const T* __restrict__ X, cplx<T>* __restrict__ Xh, long tubes, int cols,
+       long ld, long ss, int vin, int vout, double* sumsq, const int* skip) {
+    if (skip && *skip) return;
+    typedef cplx<T> V;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const int n = P.n, lns = CLS == 3 ? P.lns : 4, ns = 1 << lns, h = n / 2 + 1;
+    V* z = (V*)smraw;
+    V* z2 = CLS == 3 && P.D > 1 ? z + ((size_t)n << lns) : z;
+    V* tw = z2 + ((size_t)n << lns);
+    unsigned short* pos = (unsigned short*)(tw + n);
+    fill_tables<T>(P, tw, pos, false);
+    __syncthreads();
+    T total = 0;
+    for (int sub = 0; sub < DFT_SEQ; sub += ns) {
+        const long t0 = (long)blockIdx.x * DFT_TILE + 2 * (sub + (threadIdx.x & (ns - 1)));
+        const bool la = t0 < tubes, lb = t0 + 1 < tubes;
+        const T* xa = X + (la ? tube_off(t0, cols, ld) : 0);
+        const T* xb = X + (lb ? tube_off(t0 + 1, cols, ld) : 0);
+        T acc = 0;
+        int L = n, tstep = 1;
+        if (CLS < 3 || P.np > 0) {
+#define GO(R) pass_load<T, R>(z, tw, n, lns, xa, xb, la, lb, vin, ss, acc)
+            DFT_SWITCH(P.r[0], GO)
+#undef GO
+            tstep = P.r[0];
+            L = (int)((n * P.rr[0]) >> 20);
+        } else {  // n is all direct part: a plain copy
+            for (int k = threadIdx.x >> lns; k < n; k += blockDim.x >> lns) {
+                const V v = mk<T>(la ? __ldcs(xa + (long)k * ss) : (T)0, lb ? __ldcs(xb + (long)k * ss) : (T)0);
+                acc = fma(v.x, v.x, fma(v.y, v.y, acc));
+                z[((size_t)k << lns) + (threadIdx.x & (ns - 1))] = v;
+            }
+        }
+        const bool finite = !__syncthreads_or(!isfinite(acc));
+        total += acc;
+        if (!finite) {
+            // the defining sum, tube by tube
+            const long f0 = (long)blockIdx.x * DFT_TILE + 2 * sub;
+            for (int e = threadIdx.x; e < h * 2 * ns; e += blockDim.x) {
+                const int s = e / (2 * ns), tt = e - s * 2 * ns;
+                const long t = f0 + tt;
+                if (t >= tubes) continue;
+                const T* x = X + tube_off(t, cols, ld);
+                V o = mk<T>(0, 0);
+                int idx = 0;
+                for (int k = 0; k < n; ++k) {
+                    const T v = x[(long)k * ss];
+                    o.x = fma(v, tw[idx].x, o.x);
+                    o.y = fma(v, tw[idx].y, o.y);
+                    idx += s;
+                    if (idx >= n) idx -= n;
+                }
+                Xh[(long)s * tubes + t] = o;
+            }
+            __syncthreads();
+            continue;
+        }
+        for (int i = 1; i < P.np; ++i) {
+            if (L == P.r[i]) {
+#define GO(R) pass_smem<T, R, true>(z, tw, n, L, tstep, 0u, lns)
+                DFT_SWITCH(P.r[i], GO)
+#undef GO
+            } else {
+#define GO(R) pass_smem<T, R, false>(z, tw, n, L, tstep, P.rm[i], lns)
+                DFT_SWITCH(P.r[i], GO)
+#undef GO
+            }
+            tstep *= P.r[i];
+            L = (int)((L * P.rr[i]) >> 20);
+            __syncthreads();
+        }
+        if (CLS == 3 && P.D > 1) {
+            direct_fold<T>(z, n, P.D, lns);
+            auto put = [&](int b, int k, int q, V v) { z2[((size_t)(b * P.D + k) << lns) + q] = v; };
+            if (P.kb == 3) direct_part<T, 3>(z, tw, n, P.D, lns, put);
+            else if (P.kb == 4) direct_part<T, 4>(z, tw, n, P.D, lns, put);
+            else direct_part<T, 6>(z, tw, n, P.D, lns, put);
+            __syncthreads();
+        }
+        // the two tubes of a sequence: (Z_s + conj Z_{n-s}) / 2 and (Z_s - conj Z_{n-s}) / 2i
+        const int p = threadIdx.x & (ns - 1);
+        if (la) {
+            const int hp = (n + 1) / 2, sst = blockDim.x >> lns;
+            V* dst = Xh + t0;
+            auto out = [&](int s, int m) {  // m: n - s, or s when they are the same slice
+                const V zs = z2[((size_t)pos[s] << lns) + p], zc = z2[((size_t)pos[m] << lns) + p];
+                const V a = mk<T>((zs.x + zc.x) * (T)0.5, (zs.y - zc.y) * (T)0.5);
+                const V b = mk<T>((zs.y + zc.y) * (T)0.5, (zc.x - zs.x) * (T)0.5);
+                store_pair<T>(dst + (long)s * tubes, a, b, lb, vout);
+            };
+#pragma unroll 2
+            for (int s = threadIdx.x >> lns; s < hp; s += sst) out(s, s ? n - s : 0);
+            if (2 * hp == n && (int)(threadIdx.x >> lns) == sst - 1) out(hp, hp);
+        }
+        if (ns < DFT_SEQ) __syncthreads();
+    }
+    if (sumsq) store_partial<T>(total, sumsq);
+}
+
+template <typename T, int CLS>
+__global__ void __launch_bounds__(DFT_MAX_THREADS, sizeof(T) == 4 ? DFT_CTAS[CLS] : 1)
+k_irdft(const __grid_constant__ DftPlan P, const cplx<T>* __restrict__ Xh, T* __restrict__ X, long tubes, int cols,
+        long ld, long ss, int vin, int vout, const int* skip) {
+    if (skip && *skip) return;
+    typedef cplx<T> V;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const int n = P.n, lns = CLS == 3 ? P.lns : 4, ns = 1 << lns, h = n / 2 + 1;
+    V* z = (V*)smraw;
+    V* tw = z + ((size_t)n << lns);
+    unsigned short* freq = (unsigned short*)(tw + n);
+    fill_tables<T>(P, tw, freq, true);
+    for (int sub = 0; sub < DFT_SEQ; sub += ns) {
+        const int p = threadIdx.x & (ns - 1), sst = blockDim.x >> lns;
+        const long t0 = (long)blockIdx.x * DFT_TILE + 2 * (sub + p);
+        const bool la = t0 < tubes, lb = t0 + 1 < tubes;
+        T* xa = X + (la ? tube_off(t0, cols, ld) : 0);
+        T* xb = X + (lb ? tube_off(t0 + 1, cols, ld) : 0);
+        T bad = 0;  // stays 0 for finite data
+        constexpr int LB = sizeof(T) == 4 ? 8 : 4;  // pairs of spectrum entries in flight per thread
+        const int hp = (n + 1) / 2;  // slices 0 .. hp - 1, then slice n / 2 of an even n
+        auto put = [&](int s, V x, V y, bool self) {
+            if (self) x.y = y.y = 0;  // the imaginary parts of slices 0 and n / 2 are ignored
+            bad = fma(x.x, (T)0, fma(x.y, (T)0, fma(y.x, (T)0, fma(y.y, (T)0, bad))));
+            // Z_s = x + i y and Z_{n-s} = conj(x) + i conj(y), re and im swapped
+            z[((size_t)s << lns) + p] = mk<T>(x.y + y.x, x.x - y.y);
+            if (!self) z[((size_t)(n - s) << lns) + p] = mk<T>(y.x - x.y, x.x + y.y);
+        };
+        const V* src = Xh + t0;
+        for (int s0 = threadIdx.x >> lns; s0 < hp; s0 += LB * sst) {
+            V a[LB], b[LB];
+#pragma unroll
+            for (int u = 0; u < LB; ++u) {
+                a[u] = b[u] = mk<T>(0, 0);
+                if (la && s0 + u * sst < hp) load_pair<T>(src + (long)(s0 + u * sst) * tubes, a[u], b[u], lb, vin);
+            }
+#pragma unroll
+            for (int u = 0; u < LB; ++u)
+                if (s0 + u * sst < hp) put(s0 + u * sst, a[u], b[u], s0 + u * sst == 0);
+        }
+        if (2 * hp == n && (int)(threadIdx.x >> lns) == sst - 1) {
+            V a = mk<T>(0, 0), b = mk<T>(0, 0);
+            if (la) load_pair<T>(src + (long)hp * tubes, a, b, lb, vin);
+            put(hp, a, b, true);
+        }
+        const bool finite = !__syncthreads_or(bad != (T)0 || isnan(bad));
+        if (!finite) {
+            // the defining sum, tube by tube
+            const long f0 = (long)blockIdx.x * DFT_TILE + 2 * sub;
+            const T inv = (T)1 / (T)n;
+            for (int e = threadIdx.x; e < n * 2 * ns; e += blockDim.x) {
+                const int k = e / (2 * ns), tt = e - k * 2 * ns;
+                const long t = f0 + tt;
+                if (t >= tubes) continue;
+                T acc = Xh[t].x;
+                int idx = k;
+                for (int s = 1; s < h; ++s) {
+                    V v = Xh[(long)s * tubes + t];
+                    if (2 * s == n) v.y = 0;
+                    const T w = (2 * s == n) ? (T)1 : (T)2;
+                    acc += w * (v.x * tw[idx].x + v.y * tw[idx].y);  // tw holds cos - i sin
+                    idx += k;
+                    if (idx >= n) idx -= n;
+                }
+                X[tube_off(t, cols, ld) + (long)k * ss] = acc * inv;
+            }
+            __syncthreads();
+            continue;
+        }
+        int L = n, tstep = 1;
+        const int last = P.D > 1 ? P.np : P.np - 1;
+        for (int i = 0; i < last; ++i) {
+            if (L == P.r[i]) {
+#define GO(R) pass_smem<T, R, true>(z, tw, n, L, tstep, 0u, lns)
+                DFT_SWITCH(P.r[i], GO)
+#undef GO
+            } else {
+#define GO(R) pass_smem<T, R, false>(z, tw, n, L, tstep, P.rm[i], lns)
+                DFT_SWITCH(P.r[i], GO)
+#undef GO
+            }
+            tstep *= P.r[i];
+            L = (int)((L * P.rr[i]) >> 20);
+            __syncthreads();
+        }
+        if (CLS == 3 && P.D > 1) {
+            const T inv = (T)1 / (T)n;
+            const int nb = n / P.D;
+            const long f0 = (long)blockIdx.x * DFT_TILE + 2 * sub;
+            direct_fold<T>(z, n, P.D, lns);
+            auto put = [&](int b, int k, int q, V v) {
+                const long t = f0 + 2 * q, off = (long)(freq[b * P.D] + nb * k) * ss;
+                if (t < tubes) X[tube_off(t, cols, ld) + off] = v.y * inv;
+                if (t + 1 < tubes) X[tube_off(t + 1, cols, ld) + off] = v.x * inv;
+            };
+            if (P.kb == 3) direct_part<T, 3>(z, tw, n, P.D, lns, put);
+            else if (P.kb == 4) direct_part<T, 4>(z, tw, n, P.D, lns, put);
+            else direct_part<T, 6>(z, tw, n, P.D, lns, put);
+        } else {
+#define GO(R) pass_store<T, R>(z, freq, n, lns, xa, xb, la, lb, vout, ss)
+            DFT_SWITCH(P.r[last], GO)
+#undef GO
+        }
+        if (ns < DFT_SEQ) __syncthreads();
+    }
+}
 
 int rdft_parts(int rows, int cols) { return (int)(((long)rows * cols + DFT_TILE - 1) / DFT_TILE); }
 
-size_t rdft_smem(int n, size_t elem) {
-    const size_t c = 2 * elem;
-    if (is_pow2(n)) return ((size_t)n * 16 + n / 2) * c;
-    const size_t fwd = (size_t)n * c + (size_t)n * DFT_TILE * elem;
-    const size_t inv = (size_t)n * c + (size_t)(n / 2 + 1) * DFT_TILE * c;
-    return fwd > inv ? fwd : inv;
+// Tubes t and t + 1 (t even) are neighbours in every slice and 2-element
+// aligned: one load or store serves both.
+template <typename T> static int pair_ok(const void* X, long tubes, int cols, long ld, long ss) {
+    return ld == cols && (ss & 1) == 0 && (tubes & 1) == 0 && ((size_t)X & (2 * sizeof(T) - 1)) == 0;
 }
-
-template <typename K>
-static tp_status prep(K kern, size_t smem) {
-    if (smem_optin((const void*)kern, smem) != TP_OK) return TP_ERR_CUDA;
-    return TP_OK;
+// the same for the spectrum's (h, tubes) rows, 16 bytes a store in float32
+template <typename T> static int hat_pair_ok(const void* Xh, long tubes) {
+    return (tubes & 1) == 0 && ((size_t)Xh & 15) == 0;
 }
 
 template <typename T>
@@ -547,23 +809,14 @@ tp_status rdft(const T* X, void* Xh, int n, int rows, int cols, long ld, long ss
     const long tubes = (long)rows * cols;
     if (tubes == 0) return TP_OK;
     const unsigned grid = (unsigned)((tubes + DFT_TILE - 1) / DFT_TILE);
-    const size_t smem = rdft_smem(n, sizeof(T));
-    if (n == 256 || n == 512) {
-        const size_t sm = n == 256 ? Rdft16Q<16>::smem<T>() : Rdft16Q<32>::smem<T>();
-        auto kern = n == 256 ? k_rdft_16q<T, 16> : k_rdft_16q<T, 32>;
-        if (prep(kern, sm) != TP_OK) return TP_ERR_CUDA;
-        prof_begin(TP_KC_DFT, st);
-        kern<<<grid, DFT_THREADS, sm, st>>>(X, (cplx<T>*)Xh, tubes, cols, ld, ss, sumsq, skip);
-    } else if (is_pow2(n)) {
-        if (prep(k_rdft_pow2<T>, smem) != TP_OK) return TP_ERR_CUDA;
-        prof_begin(TP_KC_DFT, st);
-        k_rdft_pow2<T><<<grid, DFT_THREADS, smem, st>>>(X, (cplx<T>*)Xh, n, ilog2(n), tubes, cols, ld, ss,
-                                                         sumsq, skip);
-    } else {
-        if (prep(k_rdft_direct<T>, smem) != TP_OK) return TP_ERR_CUDA;
-        prof_begin(TP_KC_DFT, st);
-        k_rdft_direct<T><<<grid, DFT_THREADS, smem, st>>>(X, (cplx<T>*)Xh, n, tubes, cols, ld, ss, sumsq, skip);
-    }
+    const DftPlan& P = dft_plan(n, sizeof(T), true);
+    const size_t smem = dft_smem(P, sizeof(T), true);
+    const int cls = dft_class(P);
+    auto kern = cls == 0 ? k_rdft<T, 0> : (cls == 1 ? k_rdft<T, 1> : (cls == 2 ? k_rdft<T, 2> : k_rdft<T, 3>));
+    if (smem_optin((const void*)kern, smem) != TP_OK) return TP_ERR_CUDA;
+    prof_begin(TP_KC_DFT, st);
+    kern<<<grid, P.nt, smem, st>>>(P, X, (cplx<T>*)Xh, tubes, cols, ld, ss, pair_ok<T>(X, tubes, cols, ld, ss),
+                                        hat_pair_ok<T>(Xh, tubes), sumsq, skip);
     return launched(TP_KC_DFT, st);
 }
 
@@ -573,22 +826,14 @@ tp_status irdft(const void* Xh, T* X, int n, int rows, int cols, long ld, long s
     const long tubes = (long)rows * cols;
     if (tubes == 0) return TP_OK;
     const unsigned grid = (unsigned)((tubes + DFT_TILE - 1) / DFT_TILE);
-    const size_t smem = rdft_smem(n, sizeof(T));
-    if (n == 256) {
-        const size_t sm256 = (size_t)(256 + 2 * 16 * 16 * 17) * 2 * sizeof(T);
-        if (prep(k_irdft_256<T>, sm256) != TP_OK) return TP_ERR_CUDA;
-        prof_begin(TP_KC_DFT, st);
-        k_irdft_256<T><<<grid, DFT_THREADS, sm256, st>>>((const cplx<T>*)Xh, X, tubes, cols, ld, ss, skip);
-    } else if (is_pow2(n)) {
-        if (prep(k_irdft_pow2<T>, smem) != TP_OK) return TP_ERR_CUDA;
-        prof_begin(TP_KC_DFT, st);
-        k_irdft_pow2<T><<<grid, DFT_THREADS, smem, st>>>((const cplx<T>*)Xh, X, n, ilog2(n), tubes, cols, ld,
-                                                          ss, skip);
-    } else {
-        if (prep(k_irdft_direct<T>, smem) != TP_OK) return TP_ERR_CUDA;
-        prof_begin(TP_KC_DFT, st);
-        k_irdft_direct<T><<<grid, DFT_THREADS, smem, st>>>((const cplx<T>*)Xh, X, n, tubes, cols, ld, ss, skip);
-    }
+    const DftPlan& P = dft_plan(n, sizeof(T), false);
+    const size_t smem = dft_smem(P, sizeof(T), false);
+    const int cls = dft_class(P);
+    auto kern = cls == 0 ? k_irdft<T, 0> : (cls == 1 ? k_irdft<T, 1> : (cls == 2 ? k_irdft<T, 2> : k_irdft<T, 3>));
+    if (smem_optin((const void*)kern, smem) != TP_OK) return TP_ERR_CUDA;
+    prof_begin(TP_KC_DFT, st);
+    kern<<<grid, P.nt, smem, st>>>(P, (const cplx<T>*)Xh, X, tubes, cols, ld, ss, hat_pair_ok<T>(Xh, tubes),
+                                         pair_ok<T>(X, tubes, cols, ld, ss), skip);
     return launched(TP_KC_DFT, st);
 }
 

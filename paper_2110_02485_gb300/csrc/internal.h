@@ -55,7 +55,6 @@ int rdft_parts(int rows, int cols);
 // rdft_parts(rows, cols) partial sums that rdft writes for X (Parseval).
 template <typename T>
 tp_status norm2_hat(const void* Xh, int n, int rows, int cols, double* parts, cudaStream_t st);
-size_t rdft_smem(int n, size_t elem);
 
 // Batched complex matrix product over slices:
 //   C[s] = alpha * op(A[s]) * op(B[s]) + beta * C[s]
