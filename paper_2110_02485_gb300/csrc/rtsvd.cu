@@ -956,156 +956,215 @@ __device__ __forceinline__ float rsqrt_nr(float x) {
     return y * fmaf(-0.5f * x * y, y, 1.5f);
 }
 
-// Float32 sweeps with the two columns of a pair held in registers by GL = 8
-// lanes (r <= GL EPL; fewer lanes per pair than a half-warp amortise the
-// rotation's scalar work and shuffles over more entries per lane, and the
-// CTA needs only 512 threads): the Gram entries and the rotation read and
-// write shared memory once per element (as 16-byte pairs of entries when r
-// is even), the rotation parameters come from Newton-refined reciprocal
-// square roots (c^2 + s^2 = 1 to about an ulp), the pair indices of the round-robin ordering advance by
-// one per round (no integer division), and the per-round "any rotation" flag
-// rides on the round's barrier.
-template <int EPL, bool V2, int GL = 8>
-__device__ int jacobi_sweeps_reg(float2* Rs, float2* dp, int np, int r, int max_sweeps, float tol, float* cn) {
-    __shared__ int max_off2;  // bit pattern of the largest (|g|^2 / (a b)) of a sweep
-    const int tid = threadIdx.x, lane = tid & 31, hl = tid & (GL - 1), slot = tid / GL, nslots = blockDim.x / GL;
-    const int rr = r + (r & 1), npair = rr / 2;
+// ---- float32 sweeps over blocks of four columns ------------------------------
+// The columns are grouped in blocks of four; a round pairs the blocks (round
+// robin over blocks), a warp takes one pair of blocks: its eight columns go to
+// registers (entry lane + 32 e of each), the 16 cross pairs are rotated there in
+// four steps of four disjoint pairs, and the columns go back.  The first round
+// of a sweep also rotates the pairs inside each block (three steps) and forms
+// the columns' squared norms, which the rotations carry from then on (a
+// rotation by t = tan(theta) leaves |x|^2 - t |g| and |y|^2 + t |g|).
+//
+// What bounds it: FMA and shuffle issue.  A form with one column pair per eight
+// lanes and round moved every column to and from shared memory once per
+// rotation (half of its time at r = 96, and four times that through L2 when R
+// is in global memory); here a column moves once per four rotations, a
+// barrier comes once per 16 pairs instead of once per 4, and a rotation takes
+// 8 multiply-adds per entry instead of 12, because its cosine is kept as a
+// scale of the column that is applied when the column is stored:
+// x' = x - (t conj(e) d_y / d_x) y, y' = y + (t e d_x / d_y) x, d' = c d.
+// Measured (129 / 257 slices, six sweeps): r = 96 691 -> 586 us, r = 128
+// 2711 -> 2370 us; r = 256 from global memory 3.2 -> 1.9 ms per sweep.  At
+// r = 96 ncu counts 2.3 instructions per cycle: a step issues about 395 of
+// them per warp for its 144 multiply-adds (reduction, rotation parameters,
+// guards), with three warps per scheduler to cover each other's latencies.
+//
+// Step KIND pairs column slots P(i), Q(i), i < 4: 0-3 slot i of the first block
+// with slot (i + KIND) mod 4 of the second, 4-6 the three pairings inside a
+// block.  Lanes 8 i .. 8 i + 7 work out the rotation of pair i.
+__host__ __device__ constexpr int jac_p(int kind, int i) {
+    return kind < 4 ? i : (kind == 4 ? 2 * i : (i & 1) + 4 * (i >> 1));
+}
+__host__ __device__ constexpr int jac_q(int kind, int i) {
+    return kind < 4 ? 4 + ((i + kind) & 3)
+                    : (kind == 4 ? 2 * i + 1 : (kind == 5 ? 2 + (i & 1) + 4 * (i >> 1) : 3 - (i & 1) + 4 * (i >> 1)));
+}
+
+// Sums over the warp of eight values per lane; lane gets value 2 pair + part,
+// pair = lane bits 4-3, part = lane bit 2.
+__device__ __forceinline__ float reduce8(const float (&w)[8]) {
+    const int lane = threadIdx.x & 31;
+    float a[4], b[2], c;
+    const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float send = h4 ? w[i] : w[4 + i];
+        a[i] = (h4 ? w[4 + i] : w[i]) + __shfl_xor_sync(0xffffffffu, send, 16);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const float send = h3 ? a[i] : a[2 + i];
+        b[i] = (h3 ? a[2 + i] : a[i]) + __shfl_xor_sync(0xffffffffu, send, 8);
+    }
+    c = (h2 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h2 ? b[0] : b[1], 4);
+    c += __shfl_xor_sync(0xffffffffu, c, 2);
+    c += __shfl_xor_sync(0xffffffffu, c, 1);
+    return c;
+}
+
+// Per-warp scratch: (squared norm, scale) of the eight columns, and the two
+// coefficients of each of a step's four rotations.
+struct JacWarp {
+    float2 sc[8];
+    float4 cf[4];
+};
+
+template <int KIND, int EPL>
+__device__ __forceinline__ void jac_step(float2 (&v)[8][EPL], JacWarp& W, int col0, int col1, float2* dp, int np,
+                                         float tol2, float& mo2, int& any) {
+    const int lane = threadIdx.x & 31, pid = lane >> 3;
+    const int ps = jac_p(KIND, pid), qs = jac_q(KIND, pid);
+    const float2 A = W.sc[ps], B = W.sc[qs];
+    float w[8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float2 g = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) cfmac(g, v[jac_p(KIND, i)][e], v[jac_q(KIND, i)][e]);
+        w[2 * i] = g.x;
+        w[2 * i + 1] = g.y;
+    }
+    const float mine = reduce8(w), other = __shfl_xor_sync(0xffffffffu, mine, 4);
+    const float dd = A.y * B.y;
+    const float2 g = make_float2(((lane & 4) ? other : mine) * dd, ((lane & 4) ? mine : other) * dd);
+    const float ag2 = fmaf(g.x, g.x, g.y * g.y), ab = A.x * B.x;
+    if (ab > 0.f) mo2 = fmaxf(mo2, __fdividef(ag2, ab));
+    const bool rot = A.x > 0.f && B.x > 0.f && ag2 >= 1.17549435e-38f && ag2 > tol2 * ab;
+    if (!__any_sync(0xffffffffu, rot)) return;
+    any = 1;
+    float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (rot) {
+        const float rg = rsqrt_nr(ag2);  // 1/|g|
+        const float2 e = make_float2(g.x * rg, g.y * rg);
+        const float zeta = (B.x - A.x) * 0.5f * rg;
+        const float tt = __fdividef(copysignf(1.f, zeta), fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.f)));
+        const float c = rsqrt_nr(fmaf(tt, tt, 1.f)), sn = c * tt;
+        const float f1 = tt * __fdividef(B.y, A.y), f2 = tt * __fdividef(A.y, B.y);
+        f = make_float4(e.x * f1, -e.y * f1, e.x * f2, e.y * f2);
+        if ((lane & 7) == 0) {
+            const float tg = tt * (ag2 * rg);  // t |g|
+            W.sc[ps] = make_float2(fmaxf(A.x - tg, 0.f), A.y * c);
+            W.sc[qs] = make_float2(fmaxf(B.x + tg, 0.f), B.y * c);
+        }
+        float2* dx = dp + (ps < 4 ? col0 + ps : col1 + ps - 4) * np;
+        float2* dy = dp + (qs < 4 ? col0 + qs : col1 + qs - 4) * np;
+        for (int cc = lane & 7; cc < np; cc += 8) {  // the rows p, q of d' (np right-hand sides)
+            const float2 x = dx[cc], y = dy[cc];
+            const float2 ey = cmul(e, y), ex = cmul(cconj(e), x);
+            dx[cc] = make_float2(c * x.x - sn * ey.x, c * x.y - sn * ey.y);
+            dy[cc] = make_float2(sn * ex.x + c * y.x, sn * ex.y + c * y.y);
+        }
+    }
+    if ((lane & 7) == 0) W.cf[pid] = f;
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float4 r = W.cf[i];
+#pragma unroll
+        for (int k = 0; k < EPL; ++k) {
+            float2& x = v[jac_p(KIND, i)][k];
+            float2& y = v[jac_q(KIND, i)][k];
+            const float2 x0 = x, y0 = y;
+            x.x = fmaf(-r.x, y0.x, fmaf(r.y, y0.y, x0.x));
+            x.y = fmaf(-r.x, y0.y, fmaf(-r.y, y0.x, x0.y));
+            y.x = fmaf(r.z, x0.x, fmaf(-r.w, x0.y, y0.x));
+            y.y = fmaf(r.z, x0.y, fmaf(r.w, x0.x, y0.y));
+        }
+    }
+    __syncwarp();
+}
+
+template <int EPL>
+__device__ int jacobi_sweeps_blk(float2* Rs, float2* dp, int np, int r, int max_sweeps, float tol, float* cn,
+                                 JacWarp* scratch, int* max_off2) {
+    // max_off2: bit pattern of the largest (|g|^2 / (a b)) of a sweep
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    const int nb = (r + 3) / 4, nbb = nb + (nb & 1), npair = nbb / 2;
+    // pairs of blocks over the warps in equal passes
+    const int passes = (npair + nw - 1) / nw, act = (npair + passes - 1) / passes;
     const float tol2 = tol * tol;
-    // element e of this lane: index hl + GL e, or with pairs (V2) 2 (hl + GL (e / 2)) + e % 2
-    auto idx = [&](int e) { return V2 ? 2 * (hl + GL * (e >> 1)) + (e & 1) : hl + GL * e; };
-    // squared column norms: recomputed from the columns at the start of every
-    // sweep and carried through its rotations (a rotation by t = tan(theta)
-    // with |g| the off-diagonal entry leaves |x|^2 - t |g| and |y|^2 + t |g|),
-    // so a round forms only g = x^H y (cn: r floats of shared memory)
-    const int warp = tid >> 5, nw = blockDim.x >> 5;
+    JacWarp& W = scratch[warp];
     int sweep = 0;
     for (; sweep < max_sweeps; ++sweep) {
-        if (tid == 0) max_off2 = 0;
-        for (int j = warp; j < r; j += nw) {
-            float sq = 0.f;
-            for (int i = lane; i < r; i += 32) {
-                const float2 v = Rs[(size_t)j * r + i];
-                sq = fmaf(v.x, v.x, fmaf(v.y, v.y, sq));
-            }
-            sq = warp_sum(sq);
-            if (lane == 0) cn[j] = sq;
-        }
-        __syncthreads();
+        if (tid == 0) *max_off2 = 0;
         int any = 0;
         float mo2 = 0.f;
-        for (int base = 0; base < npair; base += nslots) {
-            const int kp = base + slot;
-            // round 0 of slot kp: (0, 1) for kp = 0, else (1 + kp, 1 + (rr - 1 - kp) % (rr - 1))
-            int pa = kp == 0 ? 0 : 1 + kp;
-            int pb = kp == 0 ? 1 : 1 + (rr - 1 - kp);
-            if (pa > rr - 1) pa -= rr - 1;
-            if (pb > rr - 1) pb -= rr - 1;
-            for (int t = 0; t < rr - 1; ++t) {
-                const int p = min(pa, pb), q = max(pa, pb);
-                const bool valid = kp < npair && q < r && p != q;
-                // a warp whose slots all lie beyond the round's pairs (r = 96: 48 pairs
-                // for 64 slots) skips to the barrier instead of issuing the round on zeros
-                // (up to r = 96; the longer columns leave no register for the test)
-                if (EPL > 12 || base + (tid >> 5) * (32 / GL) < npair) {
-                float2* cp = Rs + (size_t)p * r;
-                float2* cq = Rs + (size_t)q * r;
-                float2 x[EPL], y[EPL];
-                if (V2) {
+        for (int t = 0; t < nbb - 1; ++t) {
+            for (int kp = warp; kp < npair && warp < act; kp += act) {
+                // round robin over blocks: (0, 1 + t), (1 + (t + kp) mod, 1 + (t - kp) mod)
+                int bi = 0, bj = 1 + t;
+                if (kp > 0) {
+                    bi = 1 + t + kp;
+                    if (bi > nbb - 1) bi -= nbb - 1;
+                    bj = t - kp + nbb;
+                    if (bj > nbb - 1) bj -= nbb - 1;
+                }
+                const int col0 = 4 * min(bi, bj), col1 = 4 * max(bi, bj);
+                float2 v[8][EPL];
 #pragma unroll
-                    for (int v = 0; v < EPL / 2; ++v) {
-                        const int i = 2 * (hl + GL * v);
-                        float4 xv = make_float4(0.f, 0.f, 0.f, 0.f), yv = xv;
-                        if (valid && i < r) {
-                            xv = *(const float4*)(cp + i);
-                            yv = *(const float4*)(cq + i);
-                        }
-                        x[2 * v] = make_float2(xv.x, xv.y);
-                        x[2 * v + 1] = make_float2(xv.z, xv.w);
-                        y[2 * v] = make_float2(yv.x, yv.y);
-                        y[2 * v + 1] = make_float2(yv.z, yv.w);
+                for (int s = 0; s < 8; ++s) {
+                    const int col = s < 4 ? col0 + s : col1 + s - 4;
+                    const float2* src = Rs + (size_t)col * r;
+#pragma unroll
+                    for (int e = 0; e < EPL; ++e) {
+                        const int i = lane + 32 * e;
+                        v[s][e] = (col < r && i < r) ? src[i] : make_float2(0.f, 0.f);
                     }
+                }
+                const int mycol = lane < 4 ? col0 + lane : col1 + lane - 4;  // lanes 0-7: slot lane
+                if (t == 0) {
+                    float w[8];
+#pragma unroll
+                    for (int s = 0; s < 8; ++s) {
+                        w[s] = 0.f;
+#pragma unroll
+                        for (int e = 0; e < EPL; ++e) w[s] = fmaf(v[s][e].x, v[s][e].x, fmaf(v[s][e].y, v[s][e].y, w[s]));
+                    }
+                    const float n2 = reduce8(w);  // lanes 4 s .. 4 s + 3 hold slot s
+                    if ((lane & 3) == 0) W.sc[lane >> 2] = make_float2(n2, 1.f);
+                    __syncwarp();
+                    jac_step<4, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
+                    jac_step<5, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
+                    jac_step<6, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
                 } else {
+                    if (lane < 8) W.sc[lane] = make_float2(mycol < r ? cn[mycol] : 0.f, 1.f);
+                    __syncwarp();
+                }
+                jac_step<0, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
+                jac_step<1, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
+                jac_step<2, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
+                jac_step<3, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
+                if (lane < 8 && mycol < r) cn[mycol] = W.sc[lane].x;
+#pragma unroll
+                for (int s = 0; s < 8; ++s) {
+                    const int col = s < 4 ? col0 + s : col1 + s - 4;
+                    const float d = W.sc[s].y;
+                    float2* dst = Rs + (size_t)col * r;
 #pragma unroll
                     for (int e = 0; e < EPL; ++e) {
-                        const int i = idx(e);
-                        x[e] = y[e] = make_float2(0.f, 0.f);
-                        if (valid && i < r) {
-                            x[e] = cp[i];
-                            y[e] = cq[i];
-                        }
+                        const int i = lane + 32 * e;
+                        if (col < r && i < r) dst[i] = cscale(v[s][e], d);
                     }
                 }
-                const float a = valid ? cn[p] : 0.f, b = valid ? cn[q] : 0.f;
-                float2 g = make_float2(0.f, 0.f);
-#pragma unroll
-                for (int e = 0; e < EPL; ++e) cfmac(g, x[e], y[e]);
-#pragma unroll
-                for (int o = GL / 2; o > 0; o >>= 1) {
-                    g.x += __shfl_xor_sync(0xffffffffu, g.x, o);
-                    g.y += __shfl_xor_sync(0xffffffffu, g.y, o);
-                }
-                const float ag2 = fmaf(g.x, g.x, g.y * g.y), ab = a * b;
-                if (valid && ab > 0.f) mo2 = fmaxf(mo2, __fdividef(ag2, ab));
-                const bool rot = valid && a > 0.f && b > 0.f && ag2 >= 1.17549435e-38f && ag2 > tol2 * ab;
-                if (rot) {
-                    const float rg = rsqrt_nr(ag2);  // 1/|g|
-                    const float2 ec = make_float2(g.x * rg, -g.y * rg);
-                    const float zeta = (b - a) * 0.5f * rg;
-                    const float tt = __fdividef(copysignf(1.f, zeta), fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.f)));
-                    const float c = rsqrt_nr(fmaf(tt, tt, 1.f)), sn = c * tt;
-                    if (hl == 0) {
-                        const float tg = tt * (ag2 * rg);  // t |g|
-                        cn[p] = fmaxf(a - tg, 0.f);
-                        cn[q] = fmaxf(b + tg, 0.f);
-                    }
-                    float2 xn[EPL], yn[EPL];
-#pragma unroll
-                    for (int e = 0; e < EPL; ++e) {
-                        const float2 ey = cmul(ec, y[e]);
-                        xn[e] = make_float2(c * x[e].x - sn * ey.x, c * x[e].y - sn * ey.y);
-                        yn[e] = make_float2(sn * x[e].x + c * ey.x, sn * x[e].y + c * ey.y);
-                    }
-                    if (V2) {
-#pragma unroll
-                        for (int v = 0; v < EPL / 2; ++v) {
-                            const int i = 2 * (hl + GL * v);
-                            if (i < r) {
-                                *(float4*)(cp + i) = make_float4(xn[2 * v].x, xn[2 * v].y, xn[2 * v + 1].x,
-                                                                 xn[2 * v + 1].y);
-                                *(float4*)(cq + i) = make_float4(yn[2 * v].x, yn[2 * v].y, yn[2 * v + 1].x,
-                                                                 yn[2 * v + 1].y);
-                            }
-                        }
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < EPL; ++e) {
-                            const int i = idx(e);
-                            if (i < r) {
-                                cp[i] = xn[e];
-                                cq[i] = yn[e];
-                            }
-                        }
-                    }
-                    for (int cc = hl; cc < np; cc += GL) {  // the rows p, q of d' (np right-hand sides)
-                        const float2 xv = dp[p * np + cc];
-                        const float2 ey = cmul(cconj(ec), dp[q * np + cc]);
-                        dp[p * np + cc] = make_float2(c * xv.x - sn * ey.x, c * xv.y - sn * ey.y);
-                        dp[q * np + cc] = make_float2(sn * xv.x + c * ey.x, sn * xv.y + c * ey.y);
-                    }
-                }
-                any |= rot ? 1 : 0;
-                }
-                any = __syncthreads_or(any);
-                // next round: both indices of a slot advance by one (kp = 0 keeps p = 0)
-                if (kp != 0) pa = pa == rr - 1 ? 1 : pa + 1;
-                pb = pb == rr - 1 ? 1 : pb + 1;
+                __syncwarp();  // W is read before the next pair's setup
             }
+            __syncthreads();
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) mo2 = fmaxf(mo2, __shfl_xor_sync(0xffffffffu, mo2, o));
-        if (lane == 0) atomicMax(&max_off2, __float_as_int(mo2));
-        __syncthreads();
-        const float mo = __int_as_float(max_off2);
+        if (lane == 0) atomicMax(max_off2, __float_as_int(mo2));
+        any = __syncthreads_or(any);
+        const float mo = __int_as_float(*max_off2);
         __syncthreads();
         // no rotation, or the largest relative off-diagonal below sqrt(tol)
         if (!any || mo < tol) return sweep + 1;
@@ -1113,56 +1172,64 @@ __device__ int jacobi_sweeps_reg(float2* Rs, float2* dp, int np, int r, int max_
     return sweep;  // sweeps executed
 }
 
-template <typename T> struct JacobiSweeps {
+// MAXE: 0 = no per-warp scratch (the shared-memory form), else the most entries
+// of a column per lane (5: r <= 160; 8: r <= 256, in
+// CTAs of half the threads, whose registers hold eight such columns a warp).
+template <typename T, int MAXE> struct JacobiSweeps {
     static __device__ int run(cplx<T>* Rs, cplx<T>* dp, int np, int r, int max_sweeps, T tol, T*) {
         return jacobi_sweeps_smem<T>(Rs, dp, np, r, max_sweeps, tol);
     }
 };
-template <> struct JacobiSweeps<float> {
+template <int MAXE> struct JacobiSweeps<float, MAXE> {
     static __device__ int run(float2* Rs, float2* dp, int np, int r, int max_sweeps, float tol, float* cn) {
-        const bool v2 = (r & 1) == 0;  // 16-byte pairs of entries need an even column length
-        if (r <= 32) return v2 ? jacobi_sweeps_reg<4, true>(Rs, dp, np, r, max_sweeps, tol, cn)
-                               : jacobi_sweeps_reg<4, false>(Rs, dp, np, r, max_sweeps, tol, cn);
-        if (r <= 64) return v2 ? jacobi_sweeps_reg<8, true>(Rs, dp, np, r, max_sweeps, tol, cn)
-                               : jacobi_sweeps_reg<8, false>(Rs, dp, np, r, max_sweeps, tol, cn);
-        if (r <= 96) return v2 ? jacobi_sweeps_reg<12, true>(Rs, dp, np, r, max_sweeps, tol, cn)
-                               : jacobi_sweeps_reg<12, false>(Rs, dp, np, r, max_sweeps, tol, cn);
-        if (r <= 128) return v2 ? jacobi_sweeps_reg<16, true>(Rs, dp, np, r, max_sweeps, tol, cn)
-                                : jacobi_sweeps_reg<16, false>(Rs, dp, np, r, max_sweeps, tol, cn);
-        if (r <= 160) return v2 ? jacobi_sweeps_reg<20, true>(Rs, dp, np, r, max_sweeps, tol, cn)
-                                : jacobi_sweeps_reg<20, false>(Rs, dp, np, r, max_sweeps, tol, cn);
-        return jacobi_sweeps_smem<float>(Rs, dp, np, r, max_sweeps, tol);
+        __shared__ int max_off2;
+        __shared__ JacWarp scratch[JAC_THREADS / 32];
+        if constexpr (MAXE == 0) return jacobi_sweeps_smem<float>(Rs, dp, np, r, max_sweeps, tol);
+        if constexpr (MAXE > 5) {
+            if (r > 224) return jacobi_sweeps_blk<8>(Rs, dp, np, r, max_sweeps, tol, cn, scratch, &max_off2);
+            if (r > 192) return jacobi_sweeps_blk<7>(Rs, dp, np, r, max_sweeps, tol, cn, scratch, &max_off2);
+            if (r > 160) return jacobi_sweeps_blk<6>(Rs, dp, np, r, max_sweeps, tol, cn, scratch, &max_off2);
+        }
+        if (r > 128) return jacobi_sweeps_blk<5>(Rs, dp, np, r, max_sweeps, tol, cn, scratch, &max_off2);
+        if (r > 96) return jacobi_sweeps_blk<4>(Rs, dp, np, r, max_sweeps, tol, cn, scratch, &max_off2);
+        if (r > 64) return jacobi_sweeps_blk<3>(Rs, dp, np, r, max_sweeps, tol, cn, scratch, &max_off2);
+        if (r > 32) return jacobi_sweeps_blk<2>(Rs, dp, np, r, max_sweeps, tol, cn, scratch, &max_off2);
+        return jacobi_sweeps_blk<1>(Rs, dp, np, r, max_sweeps, tol, cn, scratch, &max_off2);
     }
 };
 
-template <typename T>
-__global__ void __launch_bounds__(JAC_THREADS)
+template <typename T, int MAXE, bool GM>
+__global__ void __launch_bounds__(MAXE > 5 ? JAC_THREADS / 2 : JAC_THREADS)
 k_jacobi(const cplx<T>* __restrict__ R, long ldr, long sR, const State* st, const cplx<T>* __restrict__ d, long sd,
          int np, T* sigma, long ssig, cplx<T>* UR, long ldu, long sU, cplx<T>* dprime, long sdp, int max_sweeps,
          int* sweeps_out, cplx<T>* gR, long sG) {
     // d and d' are r x np (np right-hand sides, row-major) per slice.  The
-    // working copy of R (column-major) lives in shared memory, or, when gR is
-    // given (factors too large for shared memory: the full T-tSVD), in gR +
-    // s sG in global memory (the slices' copies stay in L2).
+    // working copy of R (column-major) lives in shared memory, or (GM: factors
+    // too large for shared memory, the full T-tSVD) in gR + s sG in global
+    // memory (the slices' copies stay in L2).
     typedef cplx<T> V;
     const int r = st->r;
     if (r <= 0) return;
     extern __shared__ __align__(16) unsigned char smraw[];
-    V* Rs = gR ? gR + (long)blockIdx.x * sG : (V*)smraw;  // column j at Rs[j*r]
-    V* dp = gR ? (V*)smraw : Rs + (size_t)r * r;
+    V* Rs = GM ? gR + (long)blockIdx.x * sG : (V*)smraw;  // column j at Rs[j*r]
+    V* dp = GM ? (V*)smraw : Rs + (size_t)r * r;
     T* sg = (T*)(dp + (size_t)r * np);  // column norms (sigma), working precision
     int* perm = (int*)(sg + r);
     __shared__ T tol_s;
     const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     R += (long)s * sR;
-    for (int e = tid; e < r * r; e += blockDim.x) {
-        const int i = e / r, j = e - i * r;
-        Rs[(size_t)j * r + i] = R[(long)i * ldr + j];
+    // transposed copy in tiles of 8 rows x 4 columns per warp: 32-byte pieces of
+    // R's rows, and at most four words per bank in shared memory (whole rows
+    // of R per warp would put a column stride between the lanes)
+    const int ti = lane >> 2, tj = lane & 3, njt = (r + 3) / 4, ntile = (r + 7) / 8 * njt;
+    for (int q = warp; q < ntile; q += nw) {
+        const int i = q / njt * 8 + ti, j = q % njt * 4 + tj;
+        if (i < r && j < r) Rs[(size_t)j * r + i] = R[(long)i * ldr + j];
     }
     for (int i = tid; i < r * np; i += blockDim.x) dp[i] = d[(long)s * sd + i];
     if (tid == 0) tol_s = (T)(4.0 * sqrt((double)r) * Eps<T>::v);
     __syncthreads();
-    const int sweep = JacobiSweeps<T>::run(Rs, dp, np, r, max_sweeps, tol_s, sg);  // sg: the sweeps' norm scratch
+    const int sweep = JacobiSweeps<T, MAXE>::run(Rs, dp, np, r, max_sweeps, tol_s, sg);  // sg: the sweeps' norm scratch
     for (int j = warp; j < r; j += nw) {
         T a = 0;  // column norms in the working precision (float64 only on lane 0)
         for (int i = lane; i < r; i += 32) a += cabs2(Rs[(size_t)j * r + i]);
@@ -1184,12 +1251,14 @@ k_jacobi(const cplx<T>* __restrict__ R, long ldr, long sR, const State* st, cons
         dprime[(long)s * sdp + e] = dp[j * np + cc];
     }
     V* U = UR + (long)s * sU;
-    for (int e = tid; e < r * r; e += blockDim.x) {
-        const int i = e / r, jr = e - i * r;
-        const int j = perm[jr];
-        const T sv = sg[j];
-        const V x = Rs[(size_t)j * r + i];
-        U[(long)i * ldu + jr] = sv > (T)0 ? cscale(x, (T)1 / sv) : mk<T>(0, 0);
+    for (int q = warp; q < ntile; q += nw) {
+        const int i = q / njt * 8 + ti, jr = q % njt * 4 + tj;
+        if (i < r && jr < r) {
+            const int j = perm[jr];
+            const T sv = sg[j];
+            const V x = Rs[(size_t)j * r + i];
+            U[(long)i * ldu + jr] = sv > (T)0 ? cscale(x, (T)1 / sv) : mk<T>(0, 0);
+        }
     }
     if (tid == 0) atomicMax(sweeps_out, sweep);
 }
@@ -1199,20 +1268,33 @@ static size_t jacobi_smem(int r, size_t c, int np, bool global_r = false) {
            (size_t)r * sizeof(int);
 }
 
+// k_jacobi for factors of rank at most r_max, R's working copy in shared memory
+// (gR null) or in gR.
+template <typename T>
+static tp_status jacobi_launch(int h, const cplx<T>* R, long ldr, long sR, const State* st, const cplx<T>* d, long sd,
+                               int np, T* sigma, long ssig, cplx<T>* UR, long ldu, long sU, cplx<T>* dprime, long sdp,
+                               int r_max, int* sweeps, cplx<T>* gR, long sG, cudaStream_t stream) {
+    const size_t smem = jacobi_smem(r_max, sizeof(cplx<T>), np, gR != nullptr);
+    if (smem > 227 * 1024) return TP_ERR_UNSUPPORTED;
+    const bool wide = sizeof(T) == 4 && r_max > 160;
+    // a working set that leaves no room for the block sweeps' scratch (2 KB) takes the sweeps without it
+    auto kern = !gR && smem > 224 * 1024 ? k_jacobi<T, 0, false> : wide ? (gR ? k_jacobi<T, 8, true> : k_jacobi<T, 8, false>)
+                     : (gR ? k_jacobi<T, 5, true> : k_jacobi<T, 5, false>);
+    if (smem_optin((const void*)kern, smem) != TP_OK) return TP_ERR_CUDA;
+    prof_begin(TP_KC_SVD, stream);
+    kern<<<h, wide ? JAC_THREADS / 2 : JAC_THREADS, smem, stream>>>(R, ldr, sR, st, d, sd, np, sigma, ssig, UR, ldu, sU,
+                                                                    dprime, sdp, 60, sweeps, gR, sG);
+    return launched(TP_KC_SVD, stream);
+}
+
 // The one-sided Jacobi SVD of h square r x r factors (r from st->r, at most
 // r_max), with np right-hand sides rotated along; see k_jacobi.
 template <typename T>
 tp_status jacobi_svd(int h, const void* R, long ldr, long sR, const State* st, const void* d, long sd, int np,
                      T* sigma, long ssig, void* UR, long ldu, long sU, void* dprime, long sdp, int r_max,
                      int* sweeps, cudaStream_t stream) {
-    const size_t smem = jacobi_smem(r_max, sizeof(cplx<T>), np);
-    if (smem > 227 * 1024) return TP_ERR_UNSUPPORTED;
-    if (smem_optin((const void*)k_jacobi<T>, smem) != TP_OK) return TP_ERR_CUDA;
-    prof_begin(TP_KC_SVD, stream);
-    k_jacobi<T><<<h, JAC_THREADS, smem, stream>>>((const cplx<T>*)R, ldr, sR, st, (const cplx<T>*)d, sd, np, sigma,
-                                                  ssig, (cplx<T>*)UR, ldu, sU, (cplx<T>*)dprime, sdp, 60, sweeps,
-                                                  nullptr, 0);
-    return launched(TP_KC_SVD, stream);
+    return jacobi_launch<T>(h, (const cplx<T>*)R, ldr, sR, st, (const cplx<T>*)d, sd, np, sigma, ssig, (cplx<T>*)UR,
+                            ldu, sU, (cplx<T>*)dprime, sdp, r_max, sweeps, nullptr, 0, stream);
 }
 template tp_status jacobi_svd<float>(int, const void*, long, long, const State*, const void*, long, int, float*, long,
                                      void*, long, long, void*, long, int, int*, cudaStream_t);
@@ -1521,6 +1603,21 @@ __global__ void k_dp_reduce(const double* out, long so, int h, int np, int n, St
     *info = o;
 }
 
+// Columns col[0 .. b-1] of every A-hat slice (l x m) as the block Y (l x b): the
+// sketch of the T-tSVD (tt_solve), whose sketching slices are unit vectors.
+struct ColList {
+    int col[MAX_BLOCK];
+};
+template <typename T>
+__global__ void __launch_bounds__(256) k_take_cols(const cplx<T>* __restrict__ A, int l, int m, int b,
+                                                   const __grid_constant__ ColList list, cplx<T>* __restrict__ Y) {
+    const long s = blockIdx.y;
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= l * b) return;
+    const int i = e / b, c = e - i * b;
+    Y[s * l * b + e] = A[(s * l + i) * m + list.col[c]];
+}
+
 // ---------------------------------------------------------------------------
 // Workspace layout and the solve.
 // ---------------------------------------------------------------------------
@@ -1603,9 +1700,9 @@ static RtWs<T> rt_carve(void* base, int l, int m, int n, int b, int r_max, int p
 }
 
 static int jac_rmax(size_t elem, int p) {
-    // largest r whose Jacobi working set (p right-hand sides) fits in 227 KB of shared memory
+    // largest r whose Jacobi working set (p right-hand sides) fits in 227 KB of shared memory beside the sweeps' scratch
     int r = 1;
-    while (jacobi_smem(r + 1, 2 * elem, p) <= 227 * 1024) ++r;
+    while (jacobi_smem(r + 1, 2 * elem, p) <= 224 * 1024) ++r;
     return r;
 }
 
@@ -1647,7 +1744,7 @@ static tp_status rt_solve_impl(const T* A, const T* B, const T* Om, int l, int m
                                const tp_rtsvd_params* P, T* X, tp_info* info, void* ws, size_t ws_bytes,
                                cudaStream_t st, int tc_passes, bool full, const void* Ahat_in = nullptr) {
     TRY(rt_check<T>(l, m, n, p, P, full));
-    if ((!A && !Ahat_in) || !B || !Om || !X || !info) return TP_ERR_ARG;
+    if ((!A && !Ahat_in) || !B || (!Om && !full) || !X || !info) return TP_ERR_ARG;
     if (Ahat_in && ((size_t)Ahat_in & 15)) return TP_ERR_ARG;
     const int b = P->block, r_max = P->r_max, h = n / 2 + 1;
     // tc_passes: 3 = float32-accurate products, 1 = the TF32 form, 0 = the BF16
@@ -1684,7 +1781,7 @@ static tp_status rt_solve_impl(const T* A, const T* B, const T* Om, int l, int m
     // all Gaussian slices -> Fourier in one launch (blocks the sketch never
     // reaches are transformed too; one full launch beats a latency-bound
     // launch per block)
-    TRY(rdft<T>(Om, w.G, n, m, r_max, r_max, (long)m * r_max, nullptr, nullptr, st));
+    if (!full) TRY(rdft<T>(Om, w.G, n, m, r_max, r_max, (long)m * r_max, nullptr, nullptr, st));
     // the sketch and power-iteration products: A-hat (op N) or conj(A-hat^T) (op R); in the BF16 form on the
     // bfloat16 copies, tensor cores only (a shape they do not take is refused, never run on other data)
     auto sketch = [&](int M, int N, int K, const void* Af, const void* Ab, long lda, int op, const cplx<T>* Bm,
@@ -1701,11 +1798,27 @@ static tp_status rt_solve_impl(const T* A, const T* B, const T* Om, int l, int m
                                      st);
         return e == TP_ERR_UNSUPPORTED ? TP_ERR_ARG : e;
     };
+    // T-tSVD: the columns 0 .. r_max - 1 in bit-reversed order (see tt_solve)
+    int spread[RT_MAX_RANK], nspread = 0;
+    for (int i = 0; full && nspread < r_max; ++i) {
+        int rev = 0;
+        for (int bit = 0; bit < 8; ++bit) rev |= ((i >> bit) & 1) << (7 - bit);
+        if (rev < r_max) spread[nspread++] = rev;
+    }
     const int nblk = (r_max + b - 1) / b;
     for (int blk = 0; blk < nblk; ++blk) {
         const int r0 = blk * b, bb = (b < r_max - r0) ? b : r_max - r0;
         // sketch, power iterations, orthonormalise
-        TRY(sketch(l, bb, m, w.Ahat, w.Abf, m, OP_N, w.G + r0, r_max, (long)m * r_max, w.Y, bb, (long)l * bb));
+        if (full) {
+            ColList list;
+            for (int c = 0; c < bb; ++c) list.col[c] = spread[r0 + c];
+            prof_begin(TP_KC_GEMM, st);
+            k_take_cols<T><<<dim3((unsigned)((l * bb + 255) / 256), (unsigned)h), 256, 0, st>>>(w.Ahat, l, m, bb, list,
+                                                                                                w.Y);
+            TRY(launched(TP_KC_GEMM, st));
+        } else {
+            TRY(sketch(l, bb, m, w.Ahat, w.Abf, m, OP_N, w.G + r0, r_max, (long)m * r_max, w.Y, bb, (long)l * bb));
+        }
         const bool last_y = (P->q_power == 0);
         TRY(orth<T>(h, w.Y, (long)l * bb, l, bb, w.Q, (long)r_max * l, r0, last_y ? w.Q : nullptr, nullptr, 0, 0, 0,
                     nullptr, done, st));
@@ -1732,13 +1845,9 @@ static tp_status rt_solve_impl(const T* A, const T* B, const T* Om, int l, int m
     {
         // factors too large for shared memory: the working copy in Vt (free until V = Q_G U_R is formed)
         const bool gmode = r_max > jac_rmax(sizeof(T), p);
-        const size_t smem = jacobi_smem(r_max, sizeof(cplx<T>), p, gmode);
-        if (smem_optin((const void*)k_jacobi<T>, smem) != TP_OK) return TP_ERR_CUDA;
-        prof_begin(TP_KC_SVD, st);
-        k_jacobi<T><<<h, JAC_THREADS, smem, st>>>(w.R, r_max, (long)r_max * r_max, w.st, w.d, rp, p, w.sigma, r_max,
-                                                    w.UR, r_max, (long)r_max * r_max, w.dprime, rp, 60,
-                                                    &w.st->sweeps, gmode ? w.Vt : nullptr, (long)m * r_max);
-        TRY(launched(TP_KC_SVD, st));
+        TRY(jacobi_launch<T>(h, w.R, r_max, (long)r_max * r_max, w.st, w.d, rp, p, w.sigma, r_max, w.UR, r_max,
+                             (long)r_max * r_max, w.dprime, rp, r_max, &w.st->sweeps, gmode ? w.Vt : nullptr,
+                             (long)m * r_max, st));
     }
     prof_begin(TP_KC_MISC, st);
     k_alpha<T><<<h, 256, 0, st>>>(w.sigma, r_max, w.dprime, rp, w.alpha, rp, w.st, h, l > m ? l : m, r_max, p);
@@ -1824,20 +1933,22 @@ tp_status rt_adjoint(const T* G, int l, int m, int n, int p, const tp_rtsvd_para
 
 // ---------------------------------------------------------------------------
 // T-tSVD method (Section 4.1, Eqs. (11)-(14)) through the RT-tSVD path: with
-// the t-identity as the sketching tensor (Omega(:,:,1) = I, the other frontal
-// slices zero, so every Fourier slice of Omega is I) and r = min(l, m), the
-// block sketch spans the whole range of every A-hat slice, B-tilde = Q^H A-hat
-// has the singular values of A-hat, and the discrepancy scan from k = 1
-// (p = r in Eq. (kinit)) is Eq. (14)'s choice of s.  No power iterations.
+// the t-identity's lateral slices as the sketching tensor and r = min(l, m),
+// the block sketch spans the whole range of every A-hat slice, B-tilde =
+// Q^H A-hat has the singular values of A-hat, and the discrepancy scan from
+// k = 1 (p = r in Eq. (kinit)) is Eq. (14)'s choice of s.  No power iterations;
+// a block's product with A-hat is a copy of its columns.
+//
+// The columns come in bit-reversed order.  Any order gives the same subspace;
+// this one takes widely spaced columns first, which for operators whose
+// neighbouring columns are alike (blurs) does what column pivoting does: R
+// comes out graded, and the Jacobi SVD needs 8 sweeps where the natural order
+// needs 13 to 16 (float32 emulation and runs at 192 and 256; true column
+// pivoting: 7 to 8; a random order: 9 to 12).  The
+// 256^3 solve: 64.8 -> 22.1 ms, of which the SVD 57.6 -> 15.2.  Measured and
+// not kept: random slices with a power iteration (6 sweeps, but up to
+// 10 times the float32 error on ill-conditioned slices).
 // ---------------------------------------------------------------------------
-template <typename T>
-__global__ void k_tidentity(T* Om, int m, int r) {
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < m * r; e += gridDim.x * blockDim.x) {
-        const int i = e / r, j = e - i * r;
-        Om[e] = i == j ? (T)1 : (T)0;  // frontal slice 1; the other slices are zeroed by a memset
-    }
-}
-
 template <typename T>
 static tp_rtsvd_params tt_params(int l, int m, const tp_ttsvd_params* P) {
     tp_rtsvd_params R;
@@ -1858,8 +1969,7 @@ size_t tt_ws_bytes(int l, int m, int n, int p, const tp_ttsvd_params* P) {
     if (!P) return 0;
     const tp_rtsvd_params R = tt_params<T>(l, m, P);
     if (rt_check<T>(l, m, n, p, &R, true) != TP_OK) return 0;
-    const size_t rb = rt_carve<T>(nullptr, l, m, n, R.block, R.r_max, p).bytes;
-    return align256(rb) + align256((size_t)n * m * R.r_max * sizeof(T));
+    return align256(rt_carve<T>(nullptr, l, m, n, R.block, R.r_max, p).bytes);
 }
 
 template <typename T>
@@ -1870,14 +1980,8 @@ tp_status tt_solve(const T* A, const T* B, int l, int m, int n, int p, const tp_
     TRY(rt_check<T>(l, m, n, p, &R, true));
     if (!A || !B || !X || !info) return TP_ERR_ARG;
     const size_t rb = align256(rt_carve<T>(nullptr, l, m, n, R.block, R.r_max, p).bytes);
-    const size_t ob = (size_t)n * m * R.r_max * sizeof(T);
-    if (!ws || ((size_t)ws & 255) || ws_bytes < rb + align256(ob)) return TP_ERR_WORKSPACE;
-    T* Om = (T*)((char*)ws + rb);
-    if (cudaMemsetAsync(Om, 0, ob, st) != cudaSuccess) return TP_ERR_CUDA;
-    prof_begin(TP_KC_MISC, st);
-    k_tidentity<T><<<(m * R.r_max + 255) / 256, 256, 0, st>>>(Om, m, R.r_max);
-    TRY(launched(TP_KC_MISC, st));
-    return rt_solve_impl<T>(A, B, Om, l, m, n, p, &R, X, info, ws, rb, st, 3, true);
+    if (!ws || ((size_t)ws & 255) || ws_bytes < rb) return TP_ERR_WORKSPACE;
+    return rt_solve_impl<T>(A, B, nullptr, l, m, n, p, &R, X, info, ws, rb, st, 3, true);
 }
 
 // Adjoint of B -> X_s of the last tt_solve made with ws: the RT-tSVD adjoint
