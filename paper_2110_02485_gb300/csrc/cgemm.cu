@@ -150,6 +150,7 @@ k_cgemm(int M, int N, int K, const int* dM, const int* dN, const int* dK, cplx<T
 // R): a warp per row of C, the lanes striding the reduction (coalesced rows of
 // A), a warp sum per column.  Rows past the run-time count are not written.
 constexpr int ROWDOT_NB = 4;
+constexpr long CG_SMS = 152;  // SMs of a GB300
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_rowdot(int M, int N, int K, const int* dM, const int* dN, const int* dK, cplx<T> alpha,
@@ -184,6 +185,51 @@ k_rowdot(int M, int N, int K, const int* dM, const int* dN, const int* dK, cplx<
     }
     if (lane == 0)
         for (int c = 0; c < Ne; ++c) C[s * sC + (long)row * ldc + c] = cmul(alpha, acc[c]);
+}
+
+// Products with at most four right-hand columns and A read by columns (op T or
+// C): a CTA takes 32 columns of A, a warp every eighth row, so a warp reads 32
+// neighbouring entries of a row; the warps' sums meet in shared memory in a
+// fixed order.  One pass over A; the tiled form computes 16 columns of which
+// up to 15 are padding (float64, 32 x 32 by 1, 17 slices: 39 -> 4.5 us).
+constexpr int COLDOT_W = 8;
+template <typename T>
+__global__ void __launch_bounds__(32 * COLDOT_W)
+k_coldot(int M, int N, int K, const int* dM, const int* dN, const int* dK, cplx<T> alpha,
+         const cplx<T>* __restrict__ A, long lda, long sA, int conjA, const cplx<T>* __restrict__ B, long ldb,
+         long sB, cplx<T>* __restrict__ C, long ldc, long sC, const int* skip) {
+    typedef cplx<T> V;
+    if (skip && *skip) return;
+    int Me = M, Ne = N, Ke = K;
+    if (dM) Me = min(Me, *dM);
+    if (dN) Ne = min(Ne, *dN);
+    if (dK) Ke = min(Ke, *dK);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, col = blockIdx.x * 32 + lane;
+    if ((int)blockIdx.x * 32 >= Me) return;
+    __shared__ V part[ROWDOT_NB][COLDOT_W][33];
+    const long s = blockIdx.y;
+    const V* a = A + s * sA + col;
+    B += s * sB;
+    V acc[ROWDOT_NB];
+#pragma unroll
+    for (int c = 0; c < ROWDOT_NB; ++c) acc[c] = mk<T>(0, 0);
+    if (col < Me)
+#pragma unroll 4
+        for (int k = warp; k < Ke; k += COLDOT_W) {
+            V x = a[(long)k * lda];
+            if (conjA) x.y = -x.y;
+#pragma unroll
+            for (int c = 0; c < ROWDOT_NB; ++c)
+                if (c < Ne) cfma(acc[c], x, B[(long)k * ldb + c]);
+        }
+#pragma unroll
+    for (int c = 0; c < ROWDOT_NB; ++c) part[c][warp][lane] = acc[c];
+    __syncthreads();
+    if (warp < Ne && col < Me) {  // at most ROWDOT_NB <= COLDOT_W columns: a warp each
+        V t = part[warp][0][lane];
+        for (int w = 1; w < COLDOT_W; ++w) t = cadd(t, part[warp][w][lane]);
+        C[s * sC + (long)col * ldc + warp] = cmul(alpha, t);
+    }
 }
 
 template <typename T, int BM, int BN, int BK, int TM, int TN>
@@ -223,9 +269,32 @@ tp_status cgemm(int batch, int M, int N, int K, const int* dM, const int* dN, co
                                           (const cplx<T>*)B, ldb, sB, (cplx<T>*)C, ldc, sC, skip);
         return launched(TP_KC_GEMM, st);
     }
+    if (N <= ROWDOT_NB && (opA == OP_T || opA == OP_C) && opB == OP_N && beta_re == 0.0 && beta_im == 0.0) {
+        dim3 grid((unsigned)((M + 31) / 32), (unsigned)batch);
+        prof_begin(TP_KC_GEMM, st);
+        k_coldot<T><<<grid, 32 * COLDOT_W, 0, st>>>(M, N, K, dM, dN, dK, al, (const cplx<T>*)A, lda, sA,
+                                                    opA == OP_C ? 1 : 0, (const cplx<T>*)B, ldb, sB, (cplx<T>*)C, ldc,
+                                                    sC, skip);
+        return launched(TP_KC_GEMM, st);
+    }
+    // Tiles: 128 x 16 or 64 x 64, or, where those would leave SMs idle (the tiles of
+    // all slices fewer than the SMs; small slices are also mostly padding in
+    // them, which float64 pays for in full), 32 x 16 and 32 x 32, and 16 x 16
+    // while even those are fewer.  Float64, 32 x 32 by 32, 17 slices: 126 -> 11 us.
+    const long tiles128 = (long)((M + 127) / 128) * batch, tiles64 = (long)((M + 63) / 64) * ((N + 63) / 64) * batch;
+    const long tiles32 = (long)((M + 31) / 32) * ((N + 31) / 32) * batch;
+    if (N <= 16 && tiles128 < CG_SMS)
+        return launch<T, 32, 16, (sizeof(T) == 4 ? 16 : 8), 2, 1>(batch, M, N, K, dM, dN, dK, al, A, lda, sA, opA, B,
+                                                                  ldb, sB, opB, be, C, ldc, sC, skip, st);
     if (N <= 16)
         return launch<T, 128, 16, (sizeof(T) == 4 ? 16 : 8), 4, 2>(batch, M, N, K, dM, dN, dK, al, A, lda, sA, opA,
                                                                     B, ldb, sB, opB, be, C, ldc, sC, skip, st);
+    if (tiles32 < CG_SMS)
+        return launch<T, 16, 16, (sizeof(T) == 4 ? 16 : 8), 1, 1>(batch, M, N, K, dM, dN, dK, al, A, lda, sA, opA, B,
+                                                                  ldb, sB, opB, be, C, ldc, sC, skip, st);
+    if (tiles64 < CG_SMS)
+        return launch<T, 32, 32, (sizeof(T) == 4 ? 16 : 8), 2, 2>(batch, M, N, K, dM, dN, dK, al, A, lda, sA, opA, B,
+                                                                  ldb, sB, opB, be, C, ldc, sC, skip, st);
     return launch<T, 64, 64, (sizeof(T) == 4 ? 16 : 8), 4, 4>(batch, M, N, K, dM, dN, dK, al, A, lda, sA, opA, B,
                                                                ldb, sB, opB, be, C, ldc, sC, skip, st);
 }
