@@ -14,6 +14,7 @@
 #include <algorithm>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
+#include <limits.h>
 #include <math.h>
 
 #include "common.cuh"
@@ -22,6 +23,7 @@
 namespace tp {
 
 constexpr int JAC_THREADS = 512;
+constexpr int RT_MAX_RANK = 256;  // sketch rank (the small SVD of rank above jac_rmax runs from global memory)
 constexpr int MAX_BLOCK = 32;
 
 // ---------------------------------------------------------------------------
@@ -52,7 +54,17 @@ template <> __device__ __forceinline__ float rsqrt_t<float>(float x) {
     const float y = rsqrtf(x);
     return y * fmaf(-0.5f * x * y, y, 1.5f);
 }
-template <> __device__ __forceinline__ double rsqrt_t<double>(double x) { return 1.0 / sqrt(x); }
+// 1/sqrt(x), x positive and normal: two Newton steps on the hardware's
+// approximation (its relative error is below 2^-20, theirs below 2^-52)
+__device__ __forceinline__ double rsqrt_nr64(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    y = y * fma(-0.5 * x * y, y, 1.5);
+    return y * fma(-0.5 * x * y, y, 1.5);
+}
+template <> __device__ __forceinline__ double rsqrt_t<double>(double x) {
+    return x > 1e-290 && x < 1e290 ? rsqrt_nr64(x) : 1.0 / sqrt(x);
+}
 
 // Cholesky factor of a 16 x 16 Hermitian Gram matrix (upper triangle of G in
 // shared memory) by the first 160 threads (warps 0-4, named barrier 1): thread
@@ -545,15 +557,16 @@ k_orth(cplx<T>* Y, long sY, int L, int b, const cplx<T>* Qb, long sQ, int r_prev
                         cfmac(acc1[j], b0, y0);
                     }
                 }
-                const int col = (BB == 32) ? lane : (lane >> 1);
+                constexpr int GL = 32 / BB;  // lanes that hold a column's sum
+                const int col = lane / GL;
                 const V t0 = warp_reduce_scatter<V, BB>(acc0);
-                if ((BB == 32 || (lane & 1) == 0)) Cp[(size_t)i0 * BB + col] = t0;
+                if (lane % GL == 0) Cp[(size_t)i0 * BB + col] = t0;
                 const V t1 = warp_reduce_scatter<V, BB>(acc1);
-                if (two && (BB == 32 || (lane & 1) == 0)) Cp[(size_t)(i0 + 1) * BB + col] = t1;
+                if (two && lane % GL == 0) Cp[(size_t)(i0 + 1) * BB + col] = t1;
             }
             __syncthreads();
-            constexpr int CPG = BB / ORTH2_GROUPS;
-            for (int e = tid; e < L * ORTH2_GROUPS; e += blockDim.x) {
+            constexpr int NGR = BB < ORTH2_GROUPS ? BB : ORTH2_GROUPS, CPG = BB / NGR;
+            for (int e = tid; e < L * NGR; e += blockDim.x) {
                 const int g = e / L, row = e - g * L;
                 V acc[CPG];
 #pragma unroll
@@ -606,7 +619,8 @@ k_orth(cplx<T>* Y, long sY, int L, int b, const cplx<T>* Qb, long sQ, int r_prev
             orth_coef_mma<false>((const float2*)Ys, LP, (const float2*)Ys, L, LP, 16, (float2*)G, part);
         } else {
             constexpr int NE = BB * (BB + 1) / 2;
-            const int nch = (int)blockDim.x / NE > 1 ? (int)blockDim.x / NE : 1;
+            // chunks of at least four rows, at most 32 (their sums are added one after another)
+            const int nch = max(1, min((int)blockDim.x / NE, min(32, L / 4)));
             const int rpc = (L + nch - 1) / nch;
             for (int it = tid; it < NE * nch; it += blockDim.x) {
                 const int c = it / NE, e = it - c * NE;
@@ -644,7 +658,7 @@ k_orth(cplx<T>* Y, long sY, int L, int b, const cplx<T>* Qb, long sQ, int r_prev
             shift = (T)(11.0 * ((double)L * b + (double)b * (b + 1)) * Eps<T>::v) * y2;
             if (lane == 0) s_shift = shift;
         }
-        if (BB == 16 && sizeof(T) == 4) {
+        if (BB == 16) {
             if (tid < 160) {
                 bar_chol();  // s_shift
                 chol16_par<T>(G, Rk, invd, b, s_shift, pass == 0, &need_shift, &passes);
@@ -684,9 +698,8 @@ k_orth(cplx<T>* Y, long sY, int L, int b, const cplx<T>* Qb, long sQ, int r_prev
                     if (lane == 0) invd[k] = id;
                     __syncwarp();
                     // trailing update G[i][jj] -= conj(R[k][i]) R[k][jj], k < i <= jj:
-                    // a half-warp (BB = 16) or a warp (BB = 32) per row i, lane
-                    // offset jj - i (no integer division)
-                    constexpr int RW = BB == 16 ? 16 : 32;
+                    // BB lanes per row i, lane offset jj - i (no integer division)
+                    constexpr int RW = BB <= 16 ? BB : 32;
                     const int rsub = lane / RW, jo = lane % RW;
                     for (int i = k + 1 + rsub; i < BB; i += 32 / RW) {
                         const int jj = i + jo;
@@ -782,13 +795,22 @@ k_orth(cplx<T>* Y, long sY, int L, int b, const cplx<T>* Qb, long sQ, int r_prev
     }
 }
 
-static size_t orth_smem(int L, int b, int r_prev, size_t c) {
-    const size_t BB = b <= 16 ? 16 : 32;
-    const size_t part = c == 8 ? (BB == 16 ? orth_part_bytes<float, 16>() : orth_part_bytes<float, 32>())
-                               : (BB == 16 ? orth_part_bytes<double, 16>() : orth_part_bytes<double, 32>());
-    const size_t gram = c == 8 ? (BB == 16 ? orth_gram_elems<float, 16>() : orth_gram_elems<float, 32>())
-                               : (BB == 16 ? orth_gram_elems<double, 16>() : orth_gram_elems<double, 32>());
-    return ((size_t)BB * (L + 1) + 2 * (size_t)r_prev * BB + 4 * BB * BB + gram) * c + part;
+// Columns a kernel carries for a block of b.  Float64 does a multiply-add per 64
+// of float32, so its padding columns cost what live ones do: b = 1 and b <= 4
+// have kernels of their own there (block of one, L = 32, 17 slices: 65 -> 8 us
+// a launch).  Float32 blocks of up to 16 columns take the 16 columns of the
+// tensor-core tiles.
+template <typename T> static int orth_cols(int b) {
+    if (sizeof(T) == 8 && b <= 4) return b == 1 ? 1 : 4;
+    return b <= 16 ? 16 : 32;
+}
+
+template <typename T> static size_t orth_smem(int L, int b, int r_prev) {
+    const int BB = orth_cols<T>(b);
+    const size_t part = BB == 16 ? orth_part_bytes<T, 16>() : 0;
+    const size_t gram = BB == 1 ? orth_gram_elems<T, 1>() : (BB == 4 ? orth_gram_elems<T, 4>() :
+                        (BB == 16 ? orth_gram_elems<T, 16>() : orth_gram_elems<T, 32>()));
+    return ((size_t)BB * (L + 1) + 2 * (size_t)r_prev * BB + 4 * BB * BB + gram) * sizeof(cplx<T>) + part;
 }
 
 template <typename T>
@@ -796,8 +818,10 @@ static tp_status orth(int h, cplx<T>* Y, long sY, int L, int b, const cplx<T>* Q
                       cplx<T>* Qout, cplx<T>* R, long ldr, long sR, int r_rows, double* normsq, const int* skip,
                       cudaStream_t st, State* eta = nullptr, int n_dft = 0, int r_new = 0) {
     const int final_pass = (Qout != nullptr || R != nullptr) ? 1 : 0;
-    const size_t smem = orth_smem(L, b, r_prev, sizeof(cplx<T>));
+    const size_t smem = orth_smem<T>(L, b, r_prev);
     auto kern = b <= 16 ? k_orth<T, 16> : k_orth<T, 32>;
+    if constexpr (sizeof(T) == 8)
+        if (b <= 4) kern = b == 1 ? k_orth<T, 1> : k_orth<T, 4>;
     const int nt = b <= 16 ? OrthThreads<T, 16>::v : OrthThreads<T, 32>::v;
     if (smem_optin((const void*)kern, smem) != TP_OK) return TP_ERR_CUDA;
     prof_begin(TP_KC_ORTH, st);
@@ -946,6 +970,154 @@ __device__ int jacobi_sweeps_smem(cplx<T>* Rs, cplx<T>* dp, int np, int r, int m
         __syncthreads();
         if (rc == 0 || mo < stop_off) return sweep + 1;
     }
+    return sweep;  // sweeps executed
+}
+
+// Float64 sweeps.  A float64 instruction costs the issue time of 64 float32 ones,
+// so a round (r / 2 disjoint pairs) runs in three phases that keep the count
+// down: 16 lanes per pair form g = x^H y alone (4 multiply-adds per entry; the
+// squared norms are carried through the rotations as in the float32 form);
+// one lane per pair works out the rotations, 32 pairs to a warp, with
+// Newton-refined reciprocals instead of divisions and square roots; 16 lanes
+// per pair apply them at 8 multiply-adds per entry (the cosines are kept as
+// scales of the columns, folded in at every sweep's start).  The form before
+// had every lane of a pair do the scalar work and form both norms in every
+// round: 4.9 ms for a 32^3
+// T-tSVD, 1.3 ms now.  R is scaled by a power of two to entries of
+// at most 1, so that |g|^2 and the products of norms stay in range.
+struct JacPair64 {
+    double2 g, f2, se;  // g, then the coefficient of y in x' (phase 2 replaces it); of x in y'; s e
+    double c;
+};
+constexpr int JAC64_PAIRS = RT_MAX_RANK / 2;
+
+// 1/x, x positive and normal, in the same way as rsqrt_nr64
+__device__ __forceinline__ double rcp_nr64(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    y = fma(y, fma(-x, y, 1.0), y);
+    return fma(y, fma(-x, y, 1.0), y);
+}
+
+// cn, cd: squared norms and scales of the columns (r entries each).
+__device__ int jacobi_sweeps_f64(double2* Rs, double2* dp, int np, int r, int max_sweeps, double tol, double* cn,
+                                 double* cd, JacPair64* pr, int* max_off, int* rots) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    const int hl = tid & 15, slot = tid >> 4, nslots = blockDim.x >> 4;
+    const int rr = r + (r & 1), npair = rr / 2;
+    const double tol2 = tol * tol;
+    for (int j = tid; j < r; j += blockDim.x) cd[j] = 1.0;
+    __syncthreads();
+    int sweep = 0;
+    for (; sweep < max_sweeps; ++sweep) {
+        if (tid == 0) {
+            *max_off = 0;
+            *rots = 0;
+        }
+        for (int j = warp; j < r; j += nw) {
+            double sq = 0.0;
+            const double d = cd[j];
+            for (int i = lane; i < r; i += 32) {
+                const double2 v = cscale(Rs[(size_t)j * r + i], d);
+                Rs[(size_t)j * r + i] = v;
+                sq = fma(v.x, v.x, fma(v.y, v.y, sq));
+            }
+            sq = warp_sum(sq);
+            if (lane == 0) cn[j] = sq;
+        }
+        __syncthreads();
+        for (int j = tid; j < r; j += blockDim.x) cd[j] = 1.0;
+        for (int t = 0; t < rr - 1; ++t) {
+            for (int kp = slot; kp < npair; kp += nslots) {
+                int p, q;
+                const bool valid = rr_pair(t, kp, rr, r, p, q);
+                double2 g = make_double2(0.0, 0.0);
+                if (valid)
+                    for (int i = hl; i < r; i += 16) cfmac(g, Rs[(size_t)p * r + i], Rs[(size_t)q * r + i]);
+                // kp and kp + 1 of a warp end together (npair need not be even: the shuffles name the half-warp)
+                const unsigned half = (lane & 16) ? 0xffff0000u : 0x0000ffffu;
+#pragma unroll
+                for (int o = 8; o > 0; o >>= 1) {
+                    g.x += __shfl_xor_sync(half, g.x, o);
+                    g.y += __shfl_xor_sync(half, g.y, o);
+                }
+                if (hl == 0) pr[kp].g = g;
+            }
+            __syncthreads();
+            if (tid < npair) {
+                int p, q;
+                const bool valid = rr_pair(t, tid, rr, r, p, q);
+                JacPair64 o;
+                o.g = o.f2 = o.se = make_double2(0.0, 0.0);
+                o.c = 1.0;
+                if (valid) {
+                    const double dx = cd[p], dy = cd[q], a = cn[p], b = cn[q], dd = dx * dy;
+                    const double2 g = cscale(pr[tid].g, dd);
+                    const double ag2 = fma(g.x, g.x, g.y * g.y), ab = a * b;
+                    if (ab > 0.0) atomicMax(max_off, __float_as_int((float)(ag2 * rcp_nr64(fmax(ab, 1e-300)))));
+                    if (a > 0.0 && b > 0.0 && ag2 > 1e-290 && ag2 > tol2 * ab) {
+                        const double rg = rsqrt_nr64(ag2);  // 1/|g|
+                        const double2 e = cscale(g, rg);
+                        // zeta = (b - a) / (2 |g|); beyond 1e100 its square would overflow and t is 0 to rounding anyway
+                        const double zeta = fmin(fmax((b - a) * 0.5 * rg, -1e100), 1e100);
+                        const double w = fma(zeta, zeta, 1.0);
+                        const double tt = copysign(rcp_nr64(fabs(zeta) + w * rsqrt_nr64(w)), zeta);
+                        const double c = rsqrt_nr64(fma(tt, tt, 1.0));
+                        const double tg = tt * (ag2 * rg), q1 = tt * dy * rcp_nr64(dx), q2 = tt * dx * rcp_nr64(dy);
+                        o.g = make_double2(e.x * q1, -e.y * q1);
+                        o.f2 = cscale(e, q2);
+                        o.se = cscale(e, c * tt);
+                        o.c = c;
+                        cn[p] = fmax(a - tg, 0.0);
+                        cn[q] = fmax(b + tg, 0.0);
+                        cd[p] = dx * c;
+                        cd[q] = dy * c;
+                        *rots = 1;
+                        if (np <= 2)  // the rows p, q of d': 32 pairs to an instruction here
+                            for (int cc = 0; cc < np; ++cc) {
+                                const double2 x = dp[p * np + cc], y = dp[q * np + cc];
+                                const double2 sy = cmul(o.se, y), sx = cmul(cconj(o.se), x);
+                                dp[p * np + cc] = make_double2(fma(c, x.x, -sy.x), fma(c, x.y, -sy.y));
+                                dp[q * np + cc] = make_double2(fma(c, y.x, sx.x), fma(c, y.y, sx.y));
+                            }
+                    }
+                }
+                pr[tid] = o;
+            }
+            __syncthreads();
+            for (int kp = slot; kp < npair; kp += nslots) {
+                int p, q;
+                const bool valid = rr_pair(t, kp, rr, r, p, q);
+                const double2 f1 = pr[kp].g, f2 = pr[kp].f2, se = pr[kp].se;
+                const double c = pr[kp].c;
+                if (!valid || (f2.x == 0.0 && f2.y == 0.0)) continue;
+                double2* cp = Rs + (size_t)p * r;
+                double2* cq = Rs + (size_t)q * r;
+                for (int i = hl; i < r; i += 16) {
+                    const double2 x = cp[i], y = cq[i];
+                    cp[i] = make_double2(fma(-f1.x, y.x, fma(f1.y, y.y, x.x)), fma(-f1.x, y.y, fma(-f1.y, y.x, x.y)));
+                    cq[i] = make_double2(fma(f2.x, x.x, fma(-f2.y, x.y, y.x)), fma(f2.x, x.y, fma(f2.y, x.x, y.y)));
+                }
+                for (int cc = hl; np > 2 && cc < np; cc += 16) {  // the rows p, q of d' (np right-hand sides)
+                    const double2 x = dp[p * np + cc], y = dp[q * np + cc];
+                    const double2 sy = cmul(se, y), sx = cmul(cconj(se), x);
+                    dp[p * np + cc] = make_double2(fma(c, x.x, -sy.x), fma(c, x.y, -sy.y));
+                    dp[q * np + cc] = make_double2(fma(c, y.x, sx.x), fma(c, y.y, sx.y));
+                }
+            }
+            __syncthreads();
+        }
+        const float mo = __int_as_float(*max_off);  // the largest |g|^2 / (a b)
+        const int any = *rots;
+        __syncthreads();
+        if (!any || mo < (float)tol) {
+            ++sweep;
+            break;
+        }
+    }
+    for (int j = warp; j < r; j += nw)
+        for (int i = lane; i < r; i += 32) Rs[(size_t)j * r + i] = cscale(Rs[(size_t)j * r + i], cd[j]);
+    __syncthreads();
     return sweep;  // sweeps executed
 }
 
@@ -1176,8 +1348,12 @@ __device__ int jacobi_sweeps_blk(float2* Rs, float2* dp, int np, int r, int max_
 // of a column per lane (5: r <= 160; 8: r <= 256, in
 // CTAs of half the threads, whose registers hold eight such columns a warp).
 template <typename T, int MAXE> struct JacobiSweeps {
-    static __device__ int run(cplx<T>* Rs, cplx<T>* dp, int np, int r, int max_sweeps, T tol, T*) {
-        return jacobi_sweeps_smem<T>(Rs, dp, np, r, max_sweeps, tol);
+    static __device__ int run(double2* Rs, double2* dp, int np, int r, int max_sweeps, double tol, double* cn) {
+        if constexpr (MAXE == 0) return jacobi_sweeps_smem<double>(Rs, dp, np, r, max_sweeps, tol);
+        __shared__ JacPair64 pr[JAC64_PAIRS];
+        __shared__ double cd[RT_MAX_RANK];
+        __shared__ int max_off, rots;
+        return jacobi_sweeps_f64(Rs, dp, np, r, max_sweeps, tol, cn, cd, pr, &max_off, &rots);
     }
 };
 template <int MAXE> struct JacobiSweeps<float, MAXE> {
@@ -1226,6 +1402,22 @@ k_jacobi(const cplx<T>* __restrict__ R, long ldr, long sR, const State* st, cons
         const int i = q / njt * 8 + ti, j = q % njt * 4 + tj;
         if (i < r && j < r) Rs[(size_t)j * r + i] = R[(long)i * ldr + j];
     }
+    if (sizeof(T) == 8) __syncthreads();
+    T unscale = 1;
+    if constexpr (sizeof(T) == 8 && MAXE > 0) {
+        // entries scaled to at most 1 by a power of two (undone on the singular values)
+        __shared__ int top;  // exponent of the largest entry
+        if (tid == 0) top = INT_MIN;
+        __syncthreads();
+        T big = 0;
+        for (int e = tid; e < r * r; e += blockDim.x) big = fmax(big, fmax(fabs(Rs[e].x), fabs(Rs[e].y)));
+        if (big > (T)0 && isfinite(big)) atomicMax(&top, ilogb(big));
+        __syncthreads();
+        const int ex = top == INT_MIN ? 0 : min(max(top + 1, -1000), 1000);
+        const T sc = scalbn((T)1, -ex);
+        unscale = scalbn((T)1, ex);
+        for (int e = tid; e < r * r; e += blockDim.x) Rs[e] = cscale(Rs[e], sc);
+    }
     for (int i = tid; i < r * np; i += blockDim.x) dp[i] = d[(long)s * sd + i];
     if (tid == 0) tol_s = (T)(4.0 * sqrt((double)r) * Eps<T>::v);
     __syncthreads();
@@ -1247,7 +1439,7 @@ k_jacobi(const cplx<T>* __restrict__ R, long ldr, long sR, const State* st, cons
     for (int e = tid; e < r * np; e += blockDim.x) {
         const int jr = e / np, cc = e - jr * np;
         const int j = perm[jr];
-        if (cc == 0) sigma[(long)s * ssig + jr] = sg[j];
+        if (cc == 0) sigma[(long)s * ssig + jr] = sg[j] * unscale;
         dprime[(long)s * sdp + e] = dp[j * np + cc];
     }
     V* U = UR + (long)s * sU;
@@ -1268,6 +1460,9 @@ static size_t jacobi_smem(int r, size_t c, int np, bool global_r = false) {
            (size_t)r * sizeof(int);
 }
 
+// dynamic shared memory beside which the sweeps' static scratch fits (2 KB in float32, 11 KB in float64)
+static size_t jac_smem_limit(size_t elem) { return (elem == 4 ? 224 : 215) * 1024; }
+
 // k_jacobi for factors of rank at most r_max, R's working copy in shared memory
 // (gR null) or in gR.
 template <typename T>
@@ -1277,9 +1472,10 @@ static tp_status jacobi_launch(int h, const cplx<T>* R, long ldr, long sR, const
     const size_t smem = jacobi_smem(r_max, sizeof(cplx<T>), np, gR != nullptr);
     if (smem > 227 * 1024) return TP_ERR_UNSUPPORTED;
     const bool wide = sizeof(T) == 4 && r_max > 160;
-    // a working set that leaves no room for the block sweeps' scratch (2 KB) takes the sweeps without it
-    auto kern = !gR && smem > 224 * 1024 ? k_jacobi<T, 0, false> : wide ? (gR ? k_jacobi<T, 8, true> : k_jacobi<T, 8, false>)
-                     : (gR ? k_jacobi<T, 5, true> : k_jacobi<T, 5, false>);
+    // a working set that leaves no room for the sweeps' scratch takes the sweeps without it
+    auto kern = gR ? k_jacobi<T, 5, true> : k_jacobi<T, 5, false>;
+    if (smem > jac_smem_limit(sizeof(T))) kern = gR ? k_jacobi<T, 0, true> : k_jacobi<T, 0, false>;
+    else if (wide) kern = gR ? k_jacobi<T, 8, true> : k_jacobi<T, 8, false>;
     if (smem_optin((const void*)kern, smem) != TP_OK) return TP_ERR_CUDA;
     prof_begin(TP_KC_SVD, stream);
     kern<<<h, wide ? JAC_THREADS / 2 : JAC_THREADS, smem, stream>>>(R, ldr, sR, st, d, sd, np, sigma, ssig, UR, ldu, sU,
@@ -1702,12 +1898,11 @@ static RtWs<T> rt_carve(void* base, int l, int m, int n, int b, int r_max, int p
 static int jac_rmax(size_t elem, int p) {
     // largest r whose Jacobi working set (p right-hand sides) fits in 227 KB of shared memory beside the sweeps' scratch
     int r = 1;
-    while (jacobi_smem(r + 1, 2 * elem, p) <= 224 * 1024) ++r;
+    while (jacobi_smem(r + 1, 2 * elem, p) <= jac_smem_limit(elem)) ++r;
     return r;
 }
 
 constexpr int RT_MAX_RHS = 64;    // lateral slices of B per RT-tSVD call
-constexpr int RT_MAX_RANK = 256;  // sketch rank (the small SVD of rank above jac_rmax runs from global memory)
 
 template <typename T>
 static tp_status rt_check(int l, int m, int n, int p, const tp_rtsvd_params* P, bool full = false) {
@@ -1722,7 +1917,7 @@ static tp_status rt_check(int l, int m, int n, int p, const tp_rtsvd_params* P, 
     if (!(P->tau > 0.0) || !(P->delta >= 0.0) || P->p_over < 0 || P->q_power < 0) return TP_ERR_ARG;
     if (!full && !(P->eps > 0.0) && !(P->eps_rel > 0.0)) return TP_ERR_ARG;
     const int Lmax = l > m ? l : m;
-    if (orth_smem(Lmax, P->block, P->r_max, 2 * sizeof(T)) > 227 * 1024) return TP_ERR_ARG;
+    if (orth_smem<T>(Lmax, P->block, P->r_max) > 227 * 1024) return TP_ERR_ARG;
     return TP_OK;
 }
 
