@@ -1145,11 +1145,14 @@ __device__ __forceinline__ float rsqrt_nr(float x) {
 // 8 multiply-adds per entry instead of 12, because its cosine is kept as a
 // scale of the column that is applied when the column is stored:
 // x' = x - (t conj(e) d_y / d_x) y, y' = y + (t e d_x / d_y) x, d' = c d.
-// Measured (129 / 257 slices, six sweeps): r = 96 691 -> 586 us, r = 128
-// 2711 -> 2370 us; r = 256 from global memory 3.2 -> 1.9 ms per sweep.  At
-// r = 96 ncu counts 2.3 instructions per cycle: a step issues about 395 of
-// them per warp for its 144 multiply-adds (reduction, rotation parameters,
-// guards), with three warps per scheduler to cover each other's latencies.
+// A pair of blocks goes to 16 lanes up to r = 128, to 32 beyond: fewer lanes share
+// the reductions and the rotation's scalar work among more entries.  Measured
+// (one pair per eight lanes -> pair of blocks per warp -> this; 129, 257 and
+// 129 slices): r = 96, six sweeps 691 -> 586 -> 587 us; r = 128 2711 -> 2370 ->
+// 2115 us; r = 256 from global memory 3.2 -> 1.9 -> 1.7 ms per sweep.  At r = 96
+// six warps issue 509 instructions each per step (192 of them multiply-adds)
+// and twelve would issue 395: the first wait for latencies (1.5 instructions
+// per cycle per SM), the second for issue slots (2.3), in the same time.
 //
 // Step KIND pairs column slots P(i), Q(i), i < 4: 0-3 slot i of the first block
 // with slot (i + KIND) mod 4 of the second, 4-6 the three pairings inside a
@@ -1162,39 +1165,46 @@ __host__ __device__ constexpr int jac_q(int kind, int i) {
                     : (kind == 4 ? 2 * i + 1 : (kind == 5 ? 2 + (i & 1) + 4 * (i >> 1) : 3 - (i & 1) + 4 * (i >> 1)));
 }
 
-// Sums over the warp of eight values per lane; lane gets value 2 pair + part,
-// pair = lane bits 4-3, part = lane bit 2.
-__device__ __forceinline__ float reduce8(const float (&w)[8]) {
+// Sums over the GL lanes of a group of eight values per lane; lane gets value
+// 2 pair + part, pair = its top two bits in the group, part = the next one.
+template <int GL> __device__ __forceinline__ float reduce8(const float (&w)[8]) {
     const int lane = threadIdx.x & 31;
     float a[4], b[2], c;
-    const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+    const bool h1 = lane & (GL / 2), h2 = lane & (GL / 4), h3 = lane & (GL / 8);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const float send = h4 ? w[i] : w[4 + i];
-        a[i] = (h4 ? w[4 + i] : w[i]) + __shfl_xor_sync(0xffffffffu, send, 16);
+        const float send = h1 ? w[i] : w[4 + i];
+        a[i] = (h1 ? w[4 + i] : w[i]) + __shfl_xor_sync(0xffffffffu, send, GL / 2);
     }
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-        const float send = h3 ? a[i] : a[2 + i];
-        b[i] = (h3 ? a[2 + i] : a[i]) + __shfl_xor_sync(0xffffffffu, send, 8);
+        const float send = h2 ? a[i] : a[2 + i];
+        b[i] = (h2 ? a[2 + i] : a[i]) + __shfl_xor_sync(0xffffffffu, send, GL / 4);
     }
-    c = (h2 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h2 ? b[0] : b[1], 4);
-    c += __shfl_xor_sync(0xffffffffu, c, 2);
-    c += __shfl_xor_sync(0xffffffffu, c, 1);
+    c = (h3 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h3 ? b[0] : b[1], GL / 8);
+#pragma unroll
+    for (int o = GL / 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     return c;
 }
+// one or two ulp; infinite for an infinite argument
+__device__ __forceinline__ float sqrt_fast(float x) {
+    float y;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 
-// Per-warp scratch: (squared norm, scale) of the eight columns, and the two
+// Per-group scratch: (squared norm, scale) of the eight columns, and the two
 // coefficients of each of a step's four rotations.
-struct JacWarp {
+struct JacGroup {
     float2 sc[8];
     float4 cf[4];
 };
 
-template <int KIND, int EPL>
-__device__ __forceinline__ void jac_step(float2 (&v)[8][EPL], JacWarp& W, int col0, int col1, float2* dp, int np,
+template <int KIND, int GL, int EPL>
+__device__ __forceinline__ void jac_step(float2 (&v)[8][EPL], JacGroup& W, int col0, int col1, float2* dp, int np,
                                          float tol2, float& mo2, int& any) {
-    const int lane = threadIdx.x & 31, pid = lane >> 3;
+    constexpr int PL = GL / 4;  // lanes per pair
+    const int hl = threadIdx.x & (GL - 1), pid = hl / PL;
     const int ps = jac_p(KIND, pid), qs = jac_q(KIND, pid);
     const float2 A = W.sc[ps], B = W.sc[qs];
     float w[8];
@@ -1206,9 +1216,10 @@ __device__ __forceinline__ void jac_step(float2 (&v)[8][EPL], JacWarp& W, int co
         w[2 * i] = g.x;
         w[2 * i + 1] = g.y;
     }
-    const float mine = reduce8(w), other = __shfl_xor_sync(0xffffffffu, mine, 4);
+    const float mine = reduce8<GL>(w), other = __shfl_xor_sync(0xffffffffu, mine, GL / 8);
     const float dd = A.y * B.y;
-    const float2 g = make_float2(((lane & 4) ? other : mine) * dd, ((lane & 4) ? mine : other) * dd);
+    const bool part = hl & (GL / 8);
+    const float2 g = make_float2((part ? other : mine) * dd, (part ? mine : other) * dd);
     const float ag2 = fmaf(g.x, g.x, g.y * g.y), ab = A.x * B.x;
     if (ab > 0.f) mo2 = fmaxf(mo2, __fdividef(ag2, ab));
     const bool rot = A.x > 0.f && B.x > 0.f && ag2 >= 1.17549435e-38f && ag2 > tol2 * ab;
@@ -1219,25 +1230,25 @@ __device__ __forceinline__ void jac_step(float2 (&v)[8][EPL], JacWarp& W, int co
         const float rg = rsqrt_nr(ag2);  // 1/|g|
         const float2 e = make_float2(g.x * rg, g.y * rg);
         const float zeta = (B.x - A.x) * 0.5f * rg;
-        const float tt = __fdividef(copysignf(1.f, zeta), fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.f)));
+        const float tt = __fdividef(copysignf(1.f, zeta), fabsf(zeta) + sqrt_fast(fmaf(zeta, zeta, 1.f)));
         const float c = rsqrt_nr(fmaf(tt, tt, 1.f)), sn = c * tt;
         const float f1 = tt * __fdividef(B.y, A.y), f2 = tt * __fdividef(A.y, B.y);
         f = make_float4(e.x * f1, -e.y * f1, e.x * f2, e.y * f2);
-        if ((lane & 7) == 0) {
+        if ((hl & (PL - 1)) == 0) {
             const float tg = tt * (ag2 * rg);  // t |g|
             W.sc[ps] = make_float2(fmaxf(A.x - tg, 0.f), A.y * c);
             W.sc[qs] = make_float2(fmaxf(B.x + tg, 0.f), B.y * c);
         }
         float2* dx = dp + (ps < 4 ? col0 + ps : col1 + ps - 4) * np;
         float2* dy = dp + (qs < 4 ? col0 + qs : col1 + qs - 4) * np;
-        for (int cc = lane & 7; cc < np; cc += 8) {  // the rows p, q of d' (np right-hand sides)
+        for (int cc = hl & (PL - 1); cc < np; cc += PL) {  // the rows p, q of d' (np right-hand sides)
             const float2 x = dx[cc], y = dy[cc];
             const float2 ey = cmul(e, y), ex = cmul(cconj(e), x);
             dx[cc] = make_float2(c * x.x - sn * ey.x, c * x.y - sn * ey.y);
             dy[cc] = make_float2(sn * ex.x + c * y.x, sn * ex.y + c * y.y);
         }
     }
-    if ((lane & 7) == 0) W.cf[pid] = f;
+    if ((hl & (PL - 1)) == 0) W.cf[pid] = f;
     __syncwarp();
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -1256,24 +1267,33 @@ __device__ __forceinline__ void jac_step(float2 (&v)[8][EPL], JacWarp& W, int co
     __syncwarp();
 }
 
-template <int EPL>
-__device__ int jacobi_sweeps_blk(float2* Rs, float2* dp, int np, int r, int max_sweeps, float tol, float* cn,
-                                 JacWarp* scratch, int* max_off2) {
+// GL lanes hold EPL entries each of a column (r <= GL EPL); FULL: r = GL EPL and
+// a multiple of eight, so that no entry and no column needs a guard.  VEC:
+// columns of even stride ld, read and written as 16-byte pairs of entries.
+template <int GL, int EPL, bool FULL, bool VEC>
+__device__ int jacobi_sweeps_blk(float2* Rs, int ld, float2* dp, int np, int r, int max_sweeps, float tol, float* cn,
+                                 JacGroup* scratch, int* max_off2) {
     // max_off2: bit pattern of the largest (|g|^2 / (a b)) of a sweep
+    constexpr int NG = 32 / GL;  // groups (pairs of blocks) per warp
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-    const int nb = (r + 3) / 4, nbb = nb + (nb & 1), npair = nbb / 2;
-    // pairs of blocks over the warps in equal passes
-    const int passes = (npair + nw - 1) / nw, act = (npair + passes - 1) / passes;
+    const int hl = lane & (GL - 1), grp = lane / GL;
+    const int nb = (r + 3) / 4, nbb = nb + (nb & 1), npair = nbb / 2, nwp = (npair + NG - 1) / NG;
+    // the warps' shares of the pairs in equal passes
+    const int passes = (nwp + nw - 1) / nw, act = (nwp + passes - 1) / passes;
     const float tol2 = tol * tol;
-    JacWarp& W = scratch[warp];
+    JacGroup& W = scratch[warp * NG + grp];
+    // entry e of this lane: index hl + GL e, or with pairs 2 (hl + GL (e / 2)) + e % 2
+    auto idx = [&](int e) { return VEC ? 2 * (hl + GL * (e >> 1)) + (e & 1) : hl + GL * e; };
     int sweep = 0;
     for (; sweep < max_sweeps; ++sweep) {
         if (tid == 0) *max_off2 = 0;
         int any = 0;
         float mo2 = 0.f;
         for (int t = 0; t < nbb - 1; ++t) {
-            for (int kp = warp; kp < npair && warp < act; kp += act) {
-                // round robin over blocks: (0, 1 + t), (1 + (t + kp) mod, 1 + (t - kp) mod)
+            for (int wp = warp; wp < nwp && warp < act; wp += act) {
+                // round robin over blocks: (0, 1 + t), (1 + (t + kp) mod, 1 + (t - kp) mod); a group past
+                // the last pair works on columns past the end (zeros, no rotation)
+                const int kp = wp * NG + grp;
                 int bi = 0, bj = 1 + t;
                 if (kp > 0) {
                     bi = 1 + t + kp;
@@ -1281,19 +1301,29 @@ __device__ int jacobi_sweeps_blk(float2* Rs, float2* dp, int np, int r, int max_
                     bj = t - kp + nbb;
                     if (bj > nbb - 1) bj -= nbb - 1;
                 }
-                const int col0 = 4 * min(bi, bj), col1 = 4 * max(bi, bj);
+                const bool live = NG == 1 || kp < npair;
+                const int col0 = live ? 4 * min(bi, bj) : r, col1 = live ? 4 * max(bi, bj) : r;
                 float2 v[8][EPL];
 #pragma unroll
                 for (int s = 0; s < 8; ++s) {
                     const int col = s < 4 ? col0 + s : col1 + s - 4;
-                    const float2* src = Rs + (size_t)col * r;
+                    const bool ok = (FULL && NG == 1) || col < r;
+                    const float2* src = Rs + (size_t)col * ld;
+                    if (VEC) {
 #pragma unroll
-                    for (int e = 0; e < EPL; ++e) {
-                        const int i = lane + 32 * e;
-                        v[s][e] = (col < r && i < r) ? src[i] : make_float2(0.f, 0.f);
+                        for (int e = 0; e < EPL; e += 2) {
+                            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+                            if (ok && (FULL || idx(e) < ld)) x = *(const float4*)(src + idx(e));
+                            v[s][e] = make_float2(x.x, x.y);
+                            v[s][e + 1] = make_float2(x.z, x.w);
+                        }
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < EPL; ++e)
+                            v[s][e] = ok && (FULL || idx(e) < r) ? src[idx(e)] : make_float2(0.f, 0.f);
                     }
                 }
-                const int mycol = lane < 4 ? col0 + lane : col1 + lane - 4;  // lanes 0-7: slot lane
+                const int mycol = hl < 4 ? col0 + hl : col1 + hl - 4;  // lanes 0-7 of the group: slot hl
                 if (t == 0) {
                     float w[8];
 #pragma unroll
@@ -1302,30 +1332,37 @@ __device__ int jacobi_sweeps_blk(float2* Rs, float2* dp, int np, int r, int max_
 #pragma unroll
                         for (int e = 0; e < EPL; ++e) w[s] = fmaf(v[s][e].x, v[s][e].x, fmaf(v[s][e].y, v[s][e].y, w[s]));
                     }
-                    const float n2 = reduce8(w);  // lanes 4 s .. 4 s + 3 hold slot s
-                    if ((lane & 3) == 0) W.sc[lane >> 2] = make_float2(n2, 1.f);
+                    const float n2 = reduce8<GL>(w);  // GL / 8 lanes hold each slot
+                    if ((hl & (GL / 8 - 1)) == 0) W.sc[hl / (GL / 8)] = make_float2(n2, 1.f);
                     __syncwarp();
-                    jac_step<4, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
-                    jac_step<5, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
-                    jac_step<6, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
+                    jac_step<4, GL, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
+                    jac_step<5, GL, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
+                    jac_step<6, GL, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
                 } else {
-                    if (lane < 8) W.sc[lane] = make_float2(mycol < r ? cn[mycol] : 0.f, 1.f);
+                    if (hl < 8) W.sc[hl] = make_float2(mycol < r ? cn[mycol] : 0.f, 1.f);
                     __syncwarp();
                 }
-                jac_step<0, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
-                jac_step<1, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
-                jac_step<2, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
-                jac_step<3, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
-                if (lane < 8 && mycol < r) cn[mycol] = W.sc[lane].x;
+                jac_step<0, GL, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
+                jac_step<1, GL, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
+                jac_step<2, GL, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
+                jac_step<3, GL, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
+                if (hl < 8 && mycol < r) cn[mycol] = W.sc[hl].x;
 #pragma unroll
                 for (int s = 0; s < 8; ++s) {
                     const int col = s < 4 ? col0 + s : col1 + s - 4;
+                    const bool ok = (FULL && NG == 1) || col < r;
                     const float d = W.sc[s].y;
-                    float2* dst = Rs + (size_t)col * r;
+                    float2* dst = Rs + (size_t)col * ld;
+                    if (VEC) {
 #pragma unroll
-                    for (int e = 0; e < EPL; ++e) {
-                        const int i = lane + 32 * e;
-                        if (col < r && i < r) dst[i] = cscale(v[s][e], d);
+                        for (int e = 0; e < EPL; e += 2)
+                            if (ok && (FULL || idx(e) < ld))
+                                *(float4*)(dst + idx(e)) = make_float4(v[s][e].x * d, v[s][e].y * d, v[s][e + 1].x * d,
+                                                                       v[s][e + 1].y * d);
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < EPL; ++e)
+                            if (ok && (FULL || idx(e) < r)) dst[idx(e)] = cscale(v[s][e], d);
                     }
                 }
                 __syncwarp();  // W is read before the next pair's setup
@@ -1344,38 +1381,53 @@ __device__ int jacobi_sweeps_blk(float2* Rs, float2* dp, int np, int r, int max_
     return sweep;  // sweeps executed
 }
 
-// MAXE: 0 = no per-warp scratch (the shared-memory form), else the most entries
-// of a column per lane (5: r <= 160; 8: r <= 256, in
-// CTAs of half the threads, whose registers hold eight such columns a warp).
-template <typename T, int MAXE> struct JacobiSweeps {
-    static __device__ int run(double2* Rs, double2* dp, int np, int r, int max_sweeps, double tol, double* cn) {
-        if constexpr (MAXE == 0) return jacobi_sweeps_smem<double>(Rs, dp, np, r, max_sweeps, tol);
+// Threads of k_jacobi: float32 sweeps run on at most 8 warps (two per scheduler
+// partition, whose registers hold eight columns of 128 entries on 16 lanes or
+// of 256 on 32).
+template <typename T> constexpr int jac_threads(bool scratch) { return sizeof(T) == 4 && scratch ? 256 : JAC_THREADS; }
+constexpr int JAC_GROUPS = 16;
+
+// SCR: the sweeps above, with their scratch in static shared memory; otherwise
+// the shared-memory form, for working sets that leave no room for it.
+template <typename T, bool SCR> struct JacobiSweeps {
+    template <bool VEC>
+    static __device__ int run(double2* Rs, int, double2* dp, int np, int r, int max_sweeps, double tol, double* cn) {
+        if constexpr (!SCR) return jacobi_sweeps_smem<double>(Rs, dp, np, r, max_sweeps, tol);
         __shared__ JacPair64 pr[JAC64_PAIRS];
         __shared__ double cd[RT_MAX_RANK];
         __shared__ int max_off, rots;
         return jacobi_sweeps_f64(Rs, dp, np, r, max_sweeps, tol, cn, cd, pr, &max_off, &rots);
     }
 };
-template <int MAXE> struct JacobiSweeps<float, MAXE> {
-    static __device__ int run(float2* Rs, float2* dp, int np, int r, int max_sweeps, float tol, float* cn) {
+template <bool SCR> struct JacobiSweeps<float, SCR> {
+    // ld: column stride; even (16-byte pairs of entries) unless GM
+    template <bool VEC>
+    static __device__ int run(float2* Rs, int ld, float2* dp, int np, int r, int max_sweeps, float tol, float* cn) {
         __shared__ int max_off2;
-        __shared__ JacWarp scratch[JAC_THREADS / 32];
-        if constexpr (MAXE == 0) return jacobi_sweeps_smem<float>(Rs, dp, np, r, max_sweeps, tol);
-        if constexpr (MAXE > 5) {
-            if (r > 224) return jacobi_sweeps_blk<8>(Rs, dp, np, r, max_sweeps, tol, cn, scratch, &max_off2);
-            if (r > 192) return jacobi_sweeps_blk<7>(Rs, dp, np, r, max_sweeps, tol, cn, scratch, &max_off2);
-            if (r > 160) return jacobi_sweeps_blk<6>(Rs, dp, np, r, max_sweeps, tol, cn, scratch, &max_off2);
-        }
-        if (r > 128) return jacobi_sweeps_blk<5>(Rs, dp, np, r, max_sweeps, tol, cn, scratch, &max_off2);
-        if (r > 96) return jacobi_sweeps_blk<4>(Rs, dp, np, r, max_sweeps, tol, cn, scratch, &max_off2);
-        if (r > 64) return jacobi_sweeps_blk<3>(Rs, dp, np, r, max_sweeps, tol, cn, scratch, &max_off2);
-        if (r > 32) return jacobi_sweeps_blk<2>(Rs, dp, np, r, max_sweeps, tol, cn, scratch, &max_off2);
-        return jacobi_sweeps_blk<1>(Rs, dp, np, r, max_sweeps, tol, cn, scratch, &max_off2);
+        __shared__ JacGroup scratch[JAC_GROUPS];
+        if constexpr (!SCR) return jacobi_sweeps_smem<float>(Rs, dp, np, r, max_sweeps, tol);
+#define JAC(GL, EPL)                                                                                               \
+    return r == GL * EPL ? jacobi_sweeps_blk<GL, EPL, true, VEC>(Rs, ld, dp, np, r, max_sweeps, tol, cn, scratch,  \
+                                                                 &max_off2)                                        \
+                         : jacobi_sweeps_blk<GL, EPL, false, VEC>(Rs, ld, dp, np, r, max_sweeps, tol, cn, scratch, \
+                                                                  &max_off2)
+        if (r > 192) JAC(32, 8);
+        if (r > 128) JAC(32, 6);
+        if (r > 96) JAC(16, 8);
+        if (r > 64) JAC(16, 6);
+        if (r > 32) JAC(16, 4);
+        JAC(16, 2);
+#undef JAC
     }
 };
 
-template <typename T, int MAXE, bool GM>
-__global__ void __launch_bounds__(MAXE > 5 ? JAC_THREADS / 2 : JAC_THREADS)
+// column stride of R's working copy: even for the float32 forms that read 16-byte pairs of entries
+template <typename T> __host__ __device__ constexpr int jac_ld(int r, bool pairs) {
+    return sizeof(T) == 4 && pairs ? r + (r & 1) : r;
+}
+
+template <typename T, bool SCR, bool GM>
+__global__ void __launch_bounds__(jac_threads<T>(SCR))
 k_jacobi(const cplx<T>* __restrict__ R, long ldr, long sR, const State* st, const cplx<T>* __restrict__ d, long sd,
          int np, T* sigma, long ssig, cplx<T>* UR, long ldu, long sU, cplx<T>* dprime, long sdp, int max_sweeps,
          int* sweeps_out, cplx<T>* gR, long sG) {
@@ -1388,7 +1440,8 @@ k_jacobi(const cplx<T>* __restrict__ R, long ldr, long sR, const State* st, cons
     if (r <= 0) return;
     extern __shared__ __align__(16) unsigned char smraw[];
     V* Rs = GM ? gR + (long)blockIdx.x * sG : (V*)smraw;  // column j at Rs[j*r]
-    V* dp = GM ? (V*)smraw : Rs + (size_t)r * r;
+    const int ld = jac_ld<T>(r, SCR && !GM);
+    V* dp = GM ? (V*)smraw : Rs + (size_t)r * ld;
     T* sg = (T*)(dp + (size_t)r * np);  // column norms (sigma), working precision
     int* perm = (int*)(sg + r);
     __shared__ T tol_s;
@@ -1400,11 +1453,13 @@ k_jacobi(const cplx<T>* __restrict__ R, long ldr, long sR, const State* st, cons
     const int ti = lane >> 2, tj = lane & 3, njt = (r + 3) / 4, ntile = (r + 7) / 8 * njt;
     for (int q = warp; q < ntile; q += nw) {
         const int i = q / njt * 8 + ti, j = q % njt * 4 + tj;
-        if (i < r && j < r) Rs[(size_t)j * r + i] = R[(long)i * ldr + j];
+        if (i < r && j < r) Rs[(size_t)j * ld + i] = R[(long)i * ldr + j];
     }
+    if (ld > r)
+        for (int j = tid; j < r; j += blockDim.x) Rs[(size_t)j * ld + r] = mk<T>(0, 0);
     if (sizeof(T) == 8) __syncthreads();
     T unscale = 1;
-    if constexpr (sizeof(T) == 8 && MAXE > 0) {
+    if constexpr (sizeof(T) == 8 && SCR) {
         // entries scaled to at most 1 by a power of two (undone on the singular values)
         __shared__ int top;  // exponent of the largest entry
         if (tid == 0) top = INT_MIN;
@@ -1421,10 +1476,10 @@ k_jacobi(const cplx<T>* __restrict__ R, long ldr, long sR, const State* st, cons
     for (int i = tid; i < r * np; i += blockDim.x) dp[i] = d[(long)s * sd + i];
     if (tid == 0) tol_s = (T)(4.0 * sqrt((double)r) * Eps<T>::v);
     __syncthreads();
-    const int sweep = JacobiSweeps<T, MAXE>::run(Rs, dp, np, r, max_sweeps, tol_s, sg);  // sg: the sweeps' norm scratch
+    const int sweep = JacobiSweeps<T, SCR>::template run<!GM>(Rs, ld, dp, np, r, max_sweeps, tol_s, sg);  // sg: the sweeps' norm scratch
     for (int j = warp; j < r; j += nw) {
         T a = 0;  // column norms in the working precision (float64 only on lane 0)
-        for (int i = lane; i < r; i += 32) a += cabs2(Rs[(size_t)j * r + i]);
+        for (int i = lane; i < r; i += 32) a += cabs2(Rs[(size_t)j * ld + i]);
         a = warp_sum(a);
         if (lane == 0) sg[j] = sqrt(a);
     }
@@ -1448,15 +1503,16 @@ k_jacobi(const cplx<T>* __restrict__ R, long ldr, long sR, const State* st, cons
         if (i < r && jr < r) {
             const int j = perm[jr];
             const T sv = sg[j];
-            const V x = Rs[(size_t)j * r + i];
+            const V x = Rs[(size_t)j * ld + i];
             U[(long)i * ldu + jr] = sv > (T)0 ? cscale(x, (T)1 / sv) : mk<T>(0, 0);
         }
     }
     if (tid == 0) atomicMax(sweeps_out, sweep);
 }
 
-static size_t jacobi_smem(int r, size_t c, int np, bool global_r = false) {
-    return (global_r ? 0 : (size_t)r * r * c) + (size_t)r * np * c + (size_t)r * sizeof(double) +
+static size_t jacobi_smem(int r, size_t c, int np, bool global_r = false, bool pad = true) {
+    const size_t ld = c == 8 ? jac_ld<float>(r, pad) : r;
+    return (global_r ? 0 : ld * r * c) + (size_t)r * np * c + (size_t)r * sizeof(double) +
            (size_t)r * sizeof(int);
 }
 
@@ -1469,16 +1525,19 @@ template <typename T>
 static tp_status jacobi_launch(int h, const cplx<T>* R, long ldr, long sR, const State* st, const cplx<T>* d, long sd,
                                int np, T* sigma, long ssig, cplx<T>* UR, long ldu, long sU, cplx<T>* dprime, long sdp,
                                int r_max, int* sweeps, cplx<T>* gR, long sG, cudaStream_t stream) {
-    const size_t smem = jacobi_smem(r_max, sizeof(cplx<T>), np, gR != nullptr);
-    if (smem > 227 * 1024) return TP_ERR_UNSUPPORTED;
-    const bool wide = sizeof(T) == 4 && r_max > 160;
+    size_t smem = jacobi_smem(r_max, sizeof(cplx<T>), np, gR != nullptr);
+    auto kern = gR ? k_jacobi<T, true, true> : k_jacobi<T, true, false>;
+    int nt = jac_threads<T>(true);
     // a working set that leaves no room for the sweeps' scratch takes the sweeps without it
-    auto kern = gR ? k_jacobi<T, 5, true> : k_jacobi<T, 5, false>;
-    if (smem > jac_smem_limit(sizeof(T))) kern = gR ? k_jacobi<T, 0, true> : k_jacobi<T, 0, false>;
-    else if (wide) kern = gR ? k_jacobi<T, 8, true> : k_jacobi<T, 8, false>;
+    if (smem > jac_smem_limit(sizeof(T))) {
+        smem = jacobi_smem(r_max, sizeof(cplx<T>), np, gR != nullptr, false);
+        if (smem > 227 * 1024) return TP_ERR_UNSUPPORTED;
+        kern = gR ? k_jacobi<T, false, true> : k_jacobi<T, false, false>;
+        nt = jac_threads<T>(false);
+    }
     if (smem_optin((const void*)kern, smem) != TP_OK) return TP_ERR_CUDA;
     prof_begin(TP_KC_SVD, stream);
-    kern<<<h, wide ? JAC_THREADS / 2 : JAC_THREADS, smem, stream>>>(R, ldr, sR, st, d, sd, np, sigma, ssig, UR, ldu, sU,
+    kern<<<h, nt, smem, stream>>>(R, ldr, sR, st, d, sd, np, sigma, ssig, UR, ldu, sU,
                                                                     dprime, sdp, 60, sweeps, gR, sG);
     return launched(TP_KC_SVD, stream);
 }
