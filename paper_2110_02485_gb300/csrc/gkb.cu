@@ -146,7 +146,7 @@ __device__ T normalize_vec(cplx<T>* u, int L, double* red, NormBc<T>* nb) {
 // 16-byte vector loads straight from global memory (the slice is contiguous),
 // eight rows in flight per thread, one CTA barrier per product.
 
-// u = A^H q - z * w.  Requires m / VW <= blockDim (one vector column per
+// u = A^H q - z * w (w null: u = A^H q).  Requires m / VW <= blockDim (one vector column per
 // thread); rg = blockDim / (m / VW) row groups; part holds blockDim * VW entries.
 template <typename T>
 __device__ void mv_h_vec(const cplx<T>* __restrict__ A, int l, int m, const cplx<T>* q, const cplx<T>* w, T z,
@@ -190,20 +190,24 @@ __device__ void mv_h_vec(const cplx<T>* __restrict__ A, int l, int m, const cplx
     for (int j = tid; j < m; j += NT) {
         V t = mk<T>(0, 0);
         for (int p = 0; p < rg; ++p) t = cadd(t, part[p * m + j]);
-        u[j] = csub(t, cscale(w[j], z));
+        u[j] = w ? csub(t, cscale(w[j], z)) : t;
     }
     __syncthreads();
 }
 
-// u = A w - c * q.  A warp takes RB = 4 consecutive rows, each lane a set of
+// u = A w - c * q (q null: u = A w).  A warp takes RB = 4 consecutive rows, each lane a set of
 // vector columns; the lanes accumulate partial sums of the four rows and one
-// reduce-scatter at the end gives lane j*8 the sum of row j.
+// reduce-scatter at the end gives lane j*8 the sum of row j.  The loads of two
+// vector columns (eight of 16 bytes) are issued before any is used: what the
+// product runs at is the bytes in flight.  (With the bounds of each load tested
+// inside the column loop the compiler kept four in flight: 15.4k cycles for
+// 256 x 256 against 11.8k now; A^H q takes 7.5k.)
 template <typename T>
 __device__ void mv_n_vec(const cplx<T>* __restrict__ A, int l, int m, const cplx<T>* w, const cplx<T>* q, T cq,
                          cplx<T>* u) {
     typedef cplx<T> V;
     typedef typename Vec16<T>::type LV;
-    constexpr int VW = Vec16<T>::VW, RB = 4;
+    constexpr int VW = Vec16<T>::VW, RB = 4, CB = 2;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int mv = m / VW;
     const LV* Av = (const LV*)A;
@@ -211,20 +215,52 @@ __device__ void mv_n_vec(const cplx<T>* __restrict__ A, int l, int m, const cplx
         V acc[RB];
 #pragma unroll
         for (int r = 0; r < RB; ++r) acc[r] = mk<T>(0, 0);
-#pragma unroll 2
-        for (int cv = lane; cv < mv; cv += 32) {  // two iterations' loads in flight
+        const LV* row = Av + (long)i0 * mv + lane;
+        const long rs = i0 + RB <= l ? mv : 0;  // rows past the end read row i0 again (not stored)
+        int cv = lane;
+        for (; cv + 32 < mv; cv += 64, row += 64) {
+            LV a[CB][RB];
+#pragma unroll
+            for (int c = 0; c < CB; ++c)
+#pragma unroll
+                for (int r = 0; r < RB; ++r) a[c][r] = __ldcg(row + r * rs + 32 * c);
+#pragma unroll
+            for (int c = 0; c < CB; ++c) {
+                V wv[VW];
+#pragma unroll
+                for (int v = 0; v < VW; ++v) wv[v] = w[(cv + 32 * c) * VW + v];
+#pragma unroll
+                for (int r = 0; r < RB; ++r) {
+                    V e[VW];
+                    unpack<T>(a[c][r], e);
+#pragma unroll
+                    for (int v = 0; v < VW; ++v) cfma(acc[r], e[v], wv[v]);
+                }
+            }
+        }
+        if (cv < mv) {
             V wv[VW];
 #pragma unroll
             for (int v = 0; v < VW; ++v) wv[v] = w[cv * VW + v];
             LV a[RB];
 #pragma unroll
-            for (int r = 0; r < RB; ++r)
-                if (i0 + r < l) a[r] = __ldcg(Av + (long)(i0 + r) * mv + cv);
+            for (int r = 0; r < RB; ++r) a[r] = __ldcg(row + r * rs);
 #pragma unroll
             for (int r = 0; r < RB; ++r) {
-                if (i0 + r < l) {
-                    V e[VW];
-                    unpack<T>(a[r], e);
+                V e[VW];
+                unpack<T>(a[r], e);
+#pragma unroll
+                for (int v = 0; v < VW; ++v) cfma(acc[r], e[v], wv[v]);
+            }
+        }
+        if (rs == 0) {  // the last rows of an l that is no multiple of four, one by one
+            for (int r = 1; i0 + r < l; ++r) {
+                acc[r] = mk<T>(0, 0);
+                for (int c2 = lane; c2 < mv; c2 += 32) {
+                    V wv[VW], e[VW];
+#pragma unroll
+                    for (int v = 0; v < VW; ++v) wv[v] = w[c2 * VW + v];
+                    unpack<T>(__ldcg(Av + (long)(i0 + r) * mv + c2), e);
 #pragma unroll
                     for (int v = 0; v < VW; ++v) cfma(acc[r], e[v], wv[v]);
                 }
@@ -232,76 +268,75 @@ __device__ void mv_n_vec(const cplx<T>* __restrict__ A, int l, int m, const cplx
         }
         const V sum = warp_reduce_scatter<V, RB>(acc);
         const int i = i0 + (lane >> 3);
-        if ((lane & 7) == 0 && i < l) u[i] = csub(sum, cscale(q[i], cq));
+        if ((lane & 7) == 0 && i < l) u[i] = q ? csub(sum, cscale(q[i], cq)) : sum;
     }
     __syncthreads();
 }
 
 // Two classical Gram-Schmidt passes of u (length L, shared) against cnt basis
-// vectors of stride L: the first kc live in shared memory (sb), the rest in
-// global memory (gb).  Loads of each phase are unrolled so that many are in
-// flight.  part: 4*L scratch.
+// vectors of stride L at gb (global).  A warp per basis vector forms the
+// coefficients; for the update a warp takes eight entries of u, its four lane
+// groups every fourth basis vector, four loads in flight each, and two
+// shuffles join them: two barriers per pass, no division and no scratch (the
+// form before split the basis over groups of threads that met in shared
+// memory; with up to 16 vectors both are bound by issued instructions and
+// barriers, not by the basis reads: a copy of the basis in shared memory
+// changed nothing).  With the two-barrier Normalize below, a step of 256 x 256
+// slices went from 20.7 to 17.6 us (16 steps: 331 -> 282 us).
+// Returns this thread's partial sum of |u_e|^2 over the entries it holds (for
+// normalize_into); the last update is not followed by a barrier.
 template <typename T>
-__device__ __forceinline__ const cplx<T>* bvec(const cplx<T>* sb, const cplx<T>* gb, int kc, int i, int L) {
-    return (i < kc ? sb : gb) + (long)i * L;
-}
-
-template <typename T>
-__device__ decltype(cplx<T>().x) reorth2(cplx<T>* u, const cplx<T>* sb, const cplx<T>* __restrict__ gb, int kc,
-                                         int cnt, int L, cplx<T>* cf, cplx<T>* part) {
-    // Returns this thread's partial sum of |u_e|^2 over its entries
-    // e = threadIdx.x + j blockDim.x of the result (for normalize_into); the
-    // last update is not followed by a barrier.
+__device__ decltype(cplx<T>().x) reorth2(cplx<T>* u, const cplx<T>* __restrict__ gb, int cnt, int L, cplx<T>* cf) {
     typedef cplx<T> V;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, NT = blockDim.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    T p = 0;
     if (cnt <= 0) {
-        T p = 0;
-        for (int e = threadIdx.x; e < L; e += NT) p += cabs2(u[e]);
+        for (int e = threadIdx.x; e < L; e += blockDim.x) p += cabs2(u[e]);
         return p;
     }
-    T p = 0;
+    const int g = lane >> 3, e8 = lane & 7;
     for (int pass = 0; pass < 2; ++pass) {
         for (int i = warp; i < cnt; i += nw) {
-            const V* bv = bvec<T>(sb, gb, kc, i, L);
+            const V* bv = gb + (long)i * L + lane;
+            const V* uv = u + lane;
             V acc = mk<T>(0, 0);
             int e = lane;
-            for (; e + 96 < L; e += 128) {
-                const V b0 = bv[e], b1 = bv[e + 32], b2 = bv[e + 64], b3 = bv[e + 96];
-                cfmac(acc, b0, u[e]);
-                cfmac(acc, b1, u[e + 32]);
-                cfmac(acc, b2, u[e + 64]);
-                cfmac(acc, b3, u[e + 96]);
+            for (; e + 96 < L; e += 128, bv += 128, uv += 128) {
+                const V b0 = bv[0], b1 = bv[32], b2 = bv[64], b3 = bv[96];
+                cfmac(acc, b0, uv[0]);
+                cfmac(acc, b1, uv[32]);
+                cfmac(acc, b2, uv[64]);
+                cfmac(acc, b3, uv[96]);
             }
-            for (; e < L; e += 32) cfmac(acc, bv[e], u[e]);
+            for (; e < L; e += 32, bv += 32, uv += 32) cfmac(acc, bv[0], uv[0]);
             acc.x = warp_sum(acc.x);
             acc.y = warp_sum(acc.y);
             if (lane == 0) cf[i] = acc;
         }
         __syncthreads();
-        // u -= sum_i basis_i cf_i, the basis split over G groups of threads
-        const int G = (NT / L) >= 4 ? 4 : ((NT / L) >= 2 ? 2 : 1);
-        for (int idx = threadIdx.x; idx < L * G; idx += NT) {
-            const int g = idx / L, e = idx - g * L;
-            V acc = mk<T>(0, 0);
-            int i = g;
-            for (; i + 3 * G < cnt; i += 4 * G) {
-                const V b0 = bvec<T>(sb, gb, kc, i, L)[e], b1 = bvec<T>(sb, gb, kc, i + G, L)[e];
-                const V b2 = bvec<T>(sb, gb, kc, i + 2 * G, L)[e], b3 = bvec<T>(sb, gb, kc, i + 3 * G, L)[e];
-                cfma(acc, b0, cf[i]);
-                cfma(acc, b1, cf[i + G]);
-                cfma(acc, b2, cf[i + 2 * G]);
-                cfma(acc, b3, cf[i + 3 * G]);
-            }
-            for (; i < cnt; i += G) cfma(acc, bvec<T>(sb, gb, kc, i, L)[e], cf[i]);
-            part[g * L + e] = acc;
-        }
-        __syncthreads();
         p = 0;
-        for (int e = threadIdx.x; e < L; e += NT) {
-            V t = u[e];
-            for (int g = 0; g < G; ++g) t = csub(t, part[g * L + e]);
-            u[e] = t;
-            p += cabs2(t);
+        for (int e0 = warp * 8; e0 < L; e0 += nw * 8) {
+            const int e = e0 + e8;
+            const bool ok = e < L;
+            const V* b = gb + (long)g * L + (ok ? e : 0);
+            V acc = mk<T>(0, 0);
+            for (int i = g; i < cnt; i += 16, b += 16 * (long)L) {
+                V x[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) x[k] = i + 4 * k < cnt ? b[4 * k * (long)L] : mk<T>(0, 0);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) cfma(acc, x[k], cf[min(i + 4 * k, cnt - 1)]);
+            }
+#pragma unroll
+            for (int o = 8; o <= 16; o <<= 1) {
+                acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+                acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+            }
+            if (g == 0 && ok) {
+                const V t = csub(u[e], acc);
+                u[e] = t;
+                p += cabs2(t);
+            }
         }
         if (pass == 0) __syncthreads();
     }
@@ -309,47 +344,59 @@ __device__ decltype(cplx<T>().x) reorth2(cplx<T>* u, const cplx<T>* sb, const cp
 }
 
 // Normalize u (length L, shared) given each thread's partial sum of squares
-// over its entries e = threadIdx.x + j blockDim.x (as reorth2 returns it):
-// writes u / ||u|| to dst (shared) and, if given, dstg (global), and returns
-// ||u|| in the working precision; a zero vector gives zeros and norm 0.  One
-// thread forms the norm and its reciprocal (float64 only when the
-// working-precision reciprocal of a positive sum is not finite).
+// (reorth2): writes u / ||u|| to dst (shared) and dstg (global), and returns
+// ||u|| in the working precision; a zero vector gives zeros and norm 0.  In
+// float32 every warp adds the warps' partial sums for itself (the same sum in
+// the same order), which saves the barrier of handing the result round; in
+// float64 one thread forms the norm and its reciprocal (64 times the issue
+// cost).  Where the working-precision reciprocal of a positive sum is not
+// finite the scaling goes through float64.
 template <typename T>
 __device__ T normalize_into(const cplx<T>* u, int L, T p, double* red, NormBc<T>* nb, cplx<T>* dst,
                             cplx<T>* dstg) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     p = warp_sum(p);
     T* redt = (T*)red;
-    __syncthreads();  // u complete; redt free
-    if (lane == 0) redt[warp] = p;
-    __syncthreads();
-    if (warp == 0) {
-        T t = lane < nw ? redt[lane] : (T)0;
-        t = warp_sum(t);
-        if (lane == 0) {
-            const T inv = t > (T)0 ? (T)1 / sqrt(t) : (T)0;
-            nb->nrm = sqrt(t);
-            nb->inv = inv;
-            nb->mode = (t > (T)0 && !isfinite(inv)) ? 1 : 0;
-            if (nb->mode) nb->invd = 1.0 / sqrt((double)t);
+    if (lane == 0) redt[warp] = p;  // red is free: its last readers are a barrier behind
+    __syncthreads();                // and u is complete
+    T nrm, inv;
+    int mode;
+    double invd = 0.0;
+    if constexpr (sizeof(T) == 4) {
+        const T t = warp_sum(lane < nw ? redt[lane] : (T)0);
+        nrm = sqrt(t);
+        inv = t > (T)0 ? (T)1 / nrm : (T)0;
+        mode = (t > (T)0 && !isfinite(inv)) ? 1 : 0;
+        if (mode) invd = 1.0 / sqrt((double)t);
+    } else {
+        if (warp == 0) {
+            T t = lane < nw ? redt[lane] : (T)0;
+            t = warp_sum(t);
+            if (lane == 0) {
+                nb->nrm = sqrt(t);
+                nb->inv = t > (T)0 ? (T)1 / sqrt(t) : (T)0;
+                nb->mode = (t > (T)0 && !isfinite(nb->inv)) ? 1 : 0;
+                if (nb->mode) nb->invd = 1.0 / sqrt((double)t);
+            }
         }
+        __syncthreads();
+        nrm = nb->nrm;
+        inv = nb->inv;
+        mode = nb->mode;
+        invd = nb->invd;
     }
-    __syncthreads();
-    const T nrm = nb->nrm;
-    if (nb->mode == 0) {
-        const T inv = nb->inv;
+    if (mode == 0) {
         for (int e = threadIdx.x; e < L; e += blockDim.x) {
             const cplx<T> v = cscale(u[e], inv);
             dst[e] = v;
-            if (dstg) dstg[e] = v;
+            dstg[e] = v;
         }
     } else {
-        const double inv = nb->invd;
         for (int e = threadIdx.x; e < L; e += blockDim.x) {
             const cplx<T> x = u[e];
-            const cplx<T> v = mk<T>((T)((double)x.x * inv), (T)((double)x.y * inv));
+            const cplx<T> v = mk<T>((T)((double)x.x * invd), (T)((double)x.y * invd));
             dst[e] = v;
-            if (dstg) dstg[e] = v;
+            dstg[e] = v;
         }
     }
     __syncthreads();
@@ -362,7 +409,7 @@ template <typename T, bool VEC, int NT>
 __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : (NT >= 512 ? 2 : 4))
 k_gkb(const cplx<T>* __restrict__ Ahat, const cplx<T>* __restrict__ Bhat, int l, int m, int n, int h, int k_max,
       double tau_delta, cplx<T>* Wb, cplx<T>* Qb, T* cc, T* zz, double* res2, unsigned* counters,
-      cplx<T>* Xhat, State* st, tp_info* info, double* res_hist, long long spin_cycles, int write_info, int kc,
+      cplx<T>* Xhat, State* st, tp_info* info, double* res_hist, long long spin_cycles, int write_info,
       int bs, int extra) {
     // bs: column stride of Bhat and Xhat (the lateral slice count of B; the
     // pointers already point at this slice's column)
@@ -373,10 +420,7 @@ k_gkb(const cplx<T>* __restrict__ Ahat, const cplx<T>* __restrict__ Bhat, int l,
     V* w = q + l;               // m
     V* u = w + m;               // L
     V* cf = u + L;              // k_max + 1
-    V* part = cf + k_max + 1;   // max(4 L, NT * VW)
-    const int part_n = (4 * L > NT * (16 / (int)sizeof(V))) ? 4 * L : NT * (16 / (int)sizeof(V));
-    V* Wc = part + part_n;      // kc cached vectors of W (m each)
-    V* Qc = Wc + (long)kc * m;  // kc cached vectors of Q (l each)
+    V* part = cf + k_max + 1;   // NT * VW (row groups' partial sums of A^H q)
     __shared__ GkbShared S;
     __shared__ double red[33];
     __shared__ NormBc<T> nb;
@@ -397,7 +441,6 @@ k_gkb(const cplx<T>* __restrict__ Ahat, const cplx<T>* __restrict__ Bhat, int l,
     for (int e = tid; e < l; e += blockDim.x) {
         q[e] = u[e];
         Qv[e] = u[e];
-        if (kc > 0) Qc[e] = u[e];
     }
     if (tid == 0) {
         zs_[0] = z1;
@@ -461,10 +504,8 @@ k_gkb(const cplx<T>* __restrict__ Ahat, const cplx<T>* __restrict__ Bhat, int l,
         }
         if (!step) break;
         // reorthogonalise ; Normalize -> c_i, w = W_i
-        const T pw = reorth2<T>(u, Wc, W, kc, i - 1, m, cf, part);
+        const T pw = reorth2<T>(u, W, i - 1, m, cf);
         const T ci = normalize_into<T>(u, m, pw, red, &nb, w, W + (long)(i - 1) * m);
-        if (i - 1 < kc)
-            for (int e = tid; e < m; e += blockDim.x) Wc[(long)(i - 1) * m + e] = w[e];
         // Q_{i+1} = A * W_i - Q_i * c_i ; reorthogonalise ; Normalize -> z_{i+1}
         if (VEC) {
             mv_n_vec<T>(A, l, m, w, q, ci, u);
@@ -474,10 +515,8 @@ k_gkb(const cplx<T>* __restrict__ Ahat, const cplx<T>* __restrict__ Bhat, int l,
             for (int e = tid; e < l; e += blockDim.x) u[e] = csub(u[e], cscale(q[e], ci));
             __syncthreads();
         }
-        const T pq = reorth2<T>(u, Qc, Qv, kc, i, l, cf, part);
+        const T pq = reorth2<T>(u, Qv, i, l, cf);
         const T zi = normalize_into<T>(u, l, pq, red, &nb, q, Qv + (long)i * l);
-        if (i < kc)
-            for (int e = tid; e < l; e += blockDim.x) Qc[(long)i * l + e] = q[e];
         if (tid == 0) {
             cs_[i - 1] = ci;
             zs_[i] = zi;
@@ -629,7 +668,7 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : (NT >= 512 ? 2 : 4)) k_gk
     V* u = w + m;               // L
     V* bj = u + L;              // l: the current lateral slice
     V* cf = bj + l;             // k_max + 1
-    V* part = cf + k_max + 1;   // max(4 L, NT * VW)
+    V* part = cf + k_max + 1;   // NT * VW (row groups' partial sums of A^H q)
     __shared__ GknShared S;
     __shared__ double red[64];
     __shared__ NormBc<T> nb;
@@ -685,7 +724,7 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : (NT >= 512 ? 2 : 4)) k_gk
                 for (int e = tid; e < m; e += NT) u[e] = csub(u[e], cscale(w[e], zprev));
                 __syncthreads();
             }
-            const T pw = reorth2<T>(u, nullptr, W, 0, i - 1, m, cf, part);
+            const T pw = reorth2<T>(u, W, i - 1, m, cf);
             const T ci = normalize_into<T>(u, m, pw, red, &nb, w, W + (long)(i - 1) * m);
             if (VEC) {
                 mv_n_vec<T>(A, l, m, w, q, ci, u);
@@ -695,7 +734,7 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : (NT >= 512 ? 2 : 4)) k_gk
                 for (int e = tid; e < l; e += NT) u[e] = csub(u[e], cscale(q[e], ci));
                 __syncthreads();
             }
-            const T pq = reorth2<T>(u, nullptr, Qv, 0, i, l, cf, part);
+            const T pq = reorth2<T>(u, Qv, i, l, cf);
             const T zi = normalize_into<T>(u, l, pq, red, &nb, q, Qv + (long)i * l);
             const double2 cn = block_dot<T>(q, bj, l, red);  // q_{i+1}^H b_j
             if (tid == 0) {
@@ -959,10 +998,10 @@ __device__ void fill_lam(const TikState* ts, R* lam) {
 // precision; "above" means sum/n > (tau delta)^2, i.e. residual > tau*delta.
 template <typename R>
 __device__ void tik_select(const R* out, int h, R thr, double log_tol, TikState* ts, R* lamv) {
-    __shared__ unsigned char above[TIK_P];
+    __shared__ unsigned above[TIK_P / 32];  // a bit per point
     const int p = threadIdx.x;
     R a = 0, comp = 0;
-    constexpr int SB = 16;  // slice values loaded ahead of the (ordered) Kahan additions
+    constexpr int SB = 32;  // slice values loaded ahead of the (ordered) Kahan additions
     for (int s0 = 0; s0 < h; s0 += SB) {
         R v[SB];
 #pragma unroll
@@ -976,28 +1015,31 @@ __device__ void tik_select(const R* out, int h, R thr, double log_tol, TikState*
             a = t;
         }
     }
-    above[p] = a > thr ? 1 : 0;
+    const unsigned bits = __ballot_sync(0xffffffffu, a > thr);
+    if ((p & 31) == 0) above[p >> 5] = bits;
     __syncthreads();
     if (p == 0) {
         const double lo = ts->lo, hi = ts->hi;
         bool fin = false;
         if (ts->round == 0) {
-            if (above[TIK_P - 1]) {  // even mu_hi leaves the residual above tau*delta
+            if (above[TIK_P / 32 - 1] >> 31) {  // even mu_hi leaves the residual above tau*delta
                 ts->t = hi;
                 ts->status = TP_ERR_NOT_CONVERGED;
                 fin = true;
-            } else if (!above[0]) {
+            } else if (!(above[0] & 1u)) {
                 ts->t = lo;
                 fin = true;
             }
         }
         if (!fin) {
-            int ps = TIK_P - 1;
-            for (int i = 1; i < TIK_P; ++i)
-                if (!above[i]) {
-                    ps = i;
+            int ps = TIK_P - 1;  // the first point from 1 on that is not above
+            for (int i = 0; i < TIK_P / 32; ++i) {
+                const unsigned m = ~above[i] & (i == 0 ? ~1u : ~0u);
+                if (m) {
+                    ps = 32 * i + __ffs(m) - 1;
                     break;
                 }
+            }
             auto pt = [&](int i) {
                 return i == 0 ? lo : (i == TIK_P - 1 ? hi : lo + (hi - lo) * (double)i / (double)(TIK_P - 1));
             };
@@ -1256,20 +1298,13 @@ static tp_status gk_single(const GkWs<T>& w, const cplx<T>* Bhat_j, cplx<T>* Xha
     // One CTA per Fourier slice, all resident (cooperative launch): 1024
     // threads when one CTA per SM suffices, else 512 (two per SM) or 256
     // (four per SM, up to n = 1214 on 152 SMs).  Vector loads need
-    // 16-byte aligned rows.  Spare shared memory caches the first kc vectors
-    // of both Krylov bases.
+    // 16-byte aligned rows.
     const size_t vb = sizeof(cplx<T>);
     const int nt = (h <= nsm) ? 1024 : (h <= 2 * nsm ? 512 : 256);  // 1, 2 or 4 CTAs per SM
     const bool vec = ((size_t)m * vb) % 16 == 0 && (size_t)m * vb / 16 <= (size_t)nt;
-    const size_t part_n = std::max<size_t>(4 * (size_t)L, 16 / vb * (size_t)nt);
+    const size_t part_n = 16 / vb * (size_t)nt;
     const size_t base_bytes = ((size_t)l + m + L + k_max + 1 + part_n) * vb;
-    const size_t static_bytes = 24 * 1024;  // GkbShared and small arrays
-    const size_t per_cta = (size_t)(228 * 1024) / (size_t)((h + nsm - 1) / nsm) - 2048;
-    const size_t avail = per_cta > base_bytes + static_bytes ? per_cta - base_bytes - static_bytes : 0;
-    // A shared-memory cache of the bases measured slower: it takes the L1
-    // capacity that the streaming loads of A-hat need in flight.
-    const int kc = 0 * (int)std::min<size_t>((size_t)k_max + 1, avail / (((size_t)l + m) * vb));
-    const size_t smem = base_bytes + (size_t)kc * ((size_t)l + m) * vb;
+    const size_t smem = base_bytes;
     const void* kern;
     if (nt == 1024) kern = vec ? (const void*)k_gkb<T, true, 1024> : (const void*)k_gkb<T, false, 1024>;
     else if (nt == 512) kern = vec ? (const void*)k_gkb<T, true, 512> : (const void*)k_gkb<T, false, 512>;
@@ -1281,10 +1316,10 @@ static tp_status gk_single(const GkWs<T>& w, const cplx<T>* Bhat_j, cplx<T>* Xha
     const cplx<T>* Ahat = w.Ahat;
     int l_ = l, m_ = m, n_ = n, h_ = h, k_ = k_max, wi = write_info, bs_ = bs;
     long long spin = wait_budget(4000000000LL);  // ~2 s at the GB300 SM clock
-    int kc_ = kc, extra_ = wait_stall();
+    int extra_ = wait_stall();
     void* args[] = {(void*)&Ahat, (void*)&Bhat_j, &l_, &m_, &n_, &h_, &k_, &td, (void*)&w.W, (void*)&w.Q,
                     (void*)&w.cc, (void*)&w.zz, (void*)&w.res2, (void*)&w.counters, (void*)&Xhat_j,
-                    (void*)&w.st, (void*)&info, (void*)&res_hist, &spin, &wi, &kc_, &bs_, &extra_};
+                    (void*)&w.st, (void*)&info, (void*)&res_hist, &spin, &wi, &bs_, &extra_};
     prof_begin(TP_KC_GKB, st);
     if (cudaLaunchCooperativeKernel(kern, dim3(h), dim3(nt), args, smem, st) != cudaSuccess)
         return TP_ERR_CUDA;
@@ -1431,7 +1466,7 @@ tp_status gkn_solve(const T* A, const T* B, int l, int m, int n, int p, const tp
     const size_t vb = sizeof(cplx<T>);
     const int nt = (h <= nsm) ? 1024 : (h <= 2 * nsm ? 512 : 256);  // 1, 2 or 4 CTAs per SM
     const bool vec = ((size_t)m * vb) % 16 == 0 && (size_t)m * vb / 16 <= (size_t)nt;
-    const size_t part_n = std::max<size_t>(4 * (size_t)L, 16 / vb * (size_t)nt);
+    const size_t part_n = 16 / vb * (size_t)nt;
     const size_t smem = ((size_t)l + m + L + l + k_max + 1 + part_n) * vb;
     const void* kern;
     if (nt == 1024) kern = vec ? (const void*)k_gkb_nested<T, true, 1024> : (const void*)k_gkb_nested<T, false, 1024>;
@@ -1826,7 +1861,11 @@ __device__ void tadj_unproj(const cplx<T>* Q, cplx<T>* Qbar, long ld, int cnt, i
 // y[i] = sum_e a[i][e] v[e] - alpha u[i] (rows i < l of the l x m slice; a warp per row).
 template <typename T>
 __device__ void tadj_mv_n(const cplx<T>* a, int l, int m, const cplx<T>* v, double alpha, const cplx<T>* u,
-                          cplx<T>* y) {
+                          cplx<T>* y, bool vec) {
+    if (vec) {
+        mv_n_vec<T>(a, l, m, v, u, (T)alpha, y);
+        return;
+    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int i = warp; i < l; i += nw) {
         cplx<T> acc = mk<T>(0, 0);
@@ -1844,7 +1883,11 @@ __device__ void tadj_mv_n(const cplx<T>* a, int l, int m, const cplx<T>* v, doub
 // y[e] = sum_i conj(a[i][e]) t[i] - beta v[e] (columns e < m; a thread per column).
 template <typename T>
 __device__ void tadj_mv_c(const cplx<T>* a, int l, int m, const cplx<T>* t, double beta, const cplx<T>* v,
-                          cplx<T>* y) {
+                          cplx<T>* y, bool vec, cplx<T>* vpart) {
+    if (vec) {
+        mv_h_vec<T>(a, l, m, t, v, (T)beta, y, vpart);
+        return;
+    }
     // columns e < m, the rows split into blockDim / m (at most 4) interleaved shares whose partial sums meet in
     // the shared array (fixed order); two accumulators per thread
     __shared__ cplx<T> part[3 * (TIKADJ_THREADS / 4)];  // (shares - 1) x span <= 3 x blockDim / 4
@@ -1909,6 +1952,10 @@ struct TadjArgs {
 template <typename T>
 __global__ void __launch_bounds__(TIKADJ_THREADS) k_tikadj_rev(const TadjArgs<T> g) {
     typedef cplx<T> V;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    V* vpart = (V*)smraw;  // row groups' partial sums of A^H t: threads x entries per 16 bytes
+    // 16-byte loads of A-hat, as in the forward
+    const bool vec = (g.m * (int)sizeof(V)) % 16 == 0 && g.m * (int)sizeof(V) / 16 <= TIKADJ_THREADS;
     // first-pass coefficients (U^H t0, V^H w0), second-pass ones (U^H t1, V^H w1), and Q^H fbar
     __shared__ double2 cdot[GKB_KMAX + 1], c2[GKB_KMAX + 1], qf[GKB_KMAX + 1];
     __shared__ double red[33];
@@ -1985,7 +2032,7 @@ __global__ void __launch_bounds__(TIKADJ_THREADS) k_tikadj_rev(const TadjArgs<T>
         const V* vj = Vv + (long)j * m;
         const double aj = (double)c[j], bj1 = (double)z[j + 1];
         // forward of the step, recomputed: t0 = a v_j - c_j u_j, t1 = t0 - U (U^H t0) over u_0 .. u_j
-        tadj_mv_n<T>(a, l, m, vj, aj, uj, t0);
+        tadj_mv_n<T>(a, l, m, vj, aj, uj, t0, vec);
         tadj_dots<T>(U, l, j + 1, t0, l, cdot);
         for (int e = tid; e < l; e += blockDim.x) {
             T sr = 0, si = 0;
@@ -2004,14 +2051,14 @@ __global__ void __launch_bounds__(TIKADJ_THREADS) k_tikadj_rev(const TadjArgs<T>
         tadj_unproj<T>(U, Ub, l, j + 1, l, c2, qf, tb, t1, tb);
         tadj_unproj<T>(U, Ub, l, j + 1, l, cdot, qf, tb, t0, tb);
         // t0 = a v_j - c_j u_j
-        tadj_mv_c<T>(a, l, m, tb, 0.0, nullptr, w0);  // a^H t0bar into w0 (scratch)
+        tadj_mv_c<T>(a, l, m, tb, 0.0, nullptr, w0, vec, vpart);  // a^H t0bar into w0 (scratch)
         const double ru = tadj_redot<T>(uj, tb, l, red);
         for (int e = tid; e < m; e += blockDim.x) Vb[(long)j * m + e] = cadd(Vb[(long)j * m + e], w0[e]);
         for (int e = tid; e < l; e += blockDim.x) Ub[(long)j * l + e] = csub(Ub[(long)j * l + e], cscale(tb[e], (T)aj));
         if (tid == 0) albar[j] -= ru;
         __syncthreads();
         // forward, recomputed: w0 = a^H u_j - z_j v_{j-1}, w1 = w0 - V (V^H w0) over v_0 .. v_{j-1}
-        tadj_mv_c<T>(a, l, m, uj, j > 0 ? (double)z[j] : 0.0, j > 0 ? Vv + (long)(j - 1) * m : nullptr, w0);
+        tadj_mv_c<T>(a, l, m, uj, j > 0 ? (double)z[j] : 0.0, j > 0 ? Vv + (long)(j - 1) * m : nullptr, w0, vec, vpart);
         tadj_dots<T>(Vv, m, j, w0, m, cdot);
         for (int e = tid; e < m; e += blockDim.x) {
             T sr = 0, si = 0;
@@ -2030,7 +2077,7 @@ __global__ void __launch_bounds__(TIKADJ_THREADS) k_tikadj_rev(const TadjArgs<T>
         tadj_unproj<T>(Vv, Vb, m, j, m, c2, qf, wb, w1, wb);
         tadj_unproj<T>(Vv, Vb, m, j, m, cdot, qf, wb, w0, wb);
         // w0 = a^H u_j - z_j v_{j-1}
-        tadj_mv_n<T>(a, l, m, wb, 0.0, nullptr, t1);  // a w0bar into t1 (scratch)
+        tadj_mv_n<T>(a, l, m, wb, 0.0, nullptr, t1, vec);  // a w0bar into t1 (scratch)
         double rv = 0.0;
         if (j > 0) rv = tadj_redot<T>(Vv + (long)(j - 1) * m, wb, m, red);
         for (int e = tid; e < l; e += blockDim.x) Ub[(long)j * l + e] = cadd(Ub[(long)j * l + e], t1[e]);
@@ -2090,7 +2137,7 @@ static tp_status tadj_run(const T* G, int l, int m, int n, const tp_tgkb_params*
     a.tik = tik;
     TRY(rdft<T>(G, (void*)a.Gh, n, m, 1, 1, m, nullptr, nullptr, st));
     prof_begin(TP_KC_MISC, st);
-    k_tikadj_rev<T><<<h, TIKADJ_THREADS, 0, st>>>(a);
+    k_tikadj_rev<T><<<h, TIKADJ_THREADS, (size_t)TIKADJ_THREADS * 16, st>>>(a);
     TRY(launched(TP_KC_MISC, st));
     return irdft<T>(a.Yh, dB, n, l, 1, 1, l, nullptr, st);
 }

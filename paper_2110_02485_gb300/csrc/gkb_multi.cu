@@ -160,10 +160,18 @@ __device__ void mvn_multi(const cplx<T>* __restrict__ A, int l, int m, const cpl
 
 // Two classical Gram-Schmidt passes of u_j (length len) against the cnt
 // basis vectors of lateral slice j (global, vector t at gb + j bsj + t len),
-// for every active j.  cf: PB x cfs coefficient scratch.
+// for every active j.  cf: PB x cfs coefficient scratch.  The basis is read four
+// times (coefficients and update of both passes) with ordinary loads: the group's
+// bases (PB cnt vectors, 123 KB at 256 entries and the mean cnt of 7.5) stay in
+// the L1 beside this kernel's 52 KB of shared memory, and A, whose loads bypass
+// it, does not evict them.  (Bypassing L1 here too: 18.1k + 22.5k cycles per
+// step on the two sides, now 16.2k + 19.9k.  Measured and not kept, both on 512
+// threads of 128 registers: four columns or rows of A per lane in the products,
+// 49k + 43k against 38k + 44k cycles, and 16 basis loads in flight here, 24k +
+// 25k.)
 template <typename T, int PB>
-__device__ void reorth_multi(cplx<T>* u, int lu, int len, const cplx<T>* __restrict__ gb, long bsj, int cnt,
-                             const int* act, cplx<T>* cf, int cfs) {
+__device__ void reorth_multi(cplx<T>* u, int lu, int len, const cplx<T>* gb, long bsj, int cnt, const int* act,
+                             cplx<T>* cf, int cfs) {
     typedef cplx<T> V;
     if (cnt <= 0) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, NT = blockDim.x;
@@ -171,11 +179,18 @@ __device__ void reorth_multi(cplx<T>* u, int lu, int len, const cplx<T>* __restr
         for (int it = warp; it < PB * cnt; it += nw) {
             const int j = it / cnt, t = it - j * cnt;
             if (!act[j]) continue;
-            const V* bv = gb + j * bsj + (long)t * len;
-            const V* uj = u + j * lu;
+            const V* bv = gb + j * bsj + (long)t * len + lane;
+            const V* uj = u + j * lu + lane;
             V acc = mk<T>(0, 0);
-#pragma unroll 4
-            for (int e = lane; e < len; e += 32) cfmac(acc, __ldcg(bv + e), uj[e]);
+            int e = lane;
+            for (; e + 224 < len; e += 256, bv += 256, uj += 256) {
+                V x[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) x[k] = bv[32 * k];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) cfmac(acc, x[k], uj[32 * k]);
+            }
+            for (; e < len; e += 32, bv += 32, uj += 32) cfmac(acc, bv[0], uj[0]);
             acc.x = warp_sum(acc.x);
             acc.y = warp_sum(acc.y);
             if (lane == 0) cf[j * cfs + t] = acc;
@@ -187,8 +202,16 @@ __device__ void reorth_multi(cplx<T>* u, int lu, int len, const cplx<T>* __restr
             const V* bj = gb + j * bsj + e;
             const V* cfj = cf + j * cfs;
             V acc = mk<T>(0, 0);
+            int t = 0;
+            for (; t + 7 < cnt; t += 8, bj += 8 * (long)len) {
+                V x[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) x[k] = bj[k * (long)len];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) cfma(acc, x[k], cfj[t + k]);
+            }
 #pragma unroll 4
-            for (int t = 0; t < cnt; ++t) cfma(acc, __ldcg(bj + (long)t * len), cfj[t]);
+            for (; t < cnt; ++t, bj += len) cfma(acc, bj[0], cfj[t]);
             u[j * lu + e] = csub(u[j * lu + e], acc);
         }
         __syncthreads();

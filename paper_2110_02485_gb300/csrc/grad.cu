@@ -39,50 +39,52 @@ __global__ void __launch_bounds__(256) k_sep_gamma(const cplx<T>* Xh, const cplx
     if (threadIdx.x == 0) gamma[s] = make_double2(re, im);
 }
 
-// One CTA: the twiddles w^j (j < n), c-hat_s for the h half-spectrum slices,
-// a_s = -(w_s / n) (gamma_s + add_s) / c-hat_s, then dc_k = sum_s Re(a_s w^{sk}).
-// A slice with c-hat_s = 0 contributes nothing (its forward solve divides by
-// zero).  Shared memory: (n + h) double2.
-__global__ void __launch_bounds__(256) k_grad_c(const double* c, int n, const double2* gamma, const double* add,
-                                                double* dc) {
-    extern __shared__ double2 gsm[];
-    double2* tw = gsm;
-    double2* a = gsm + n;
-    const int h = n / 2 + 1;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        double sn, cs;
-        sincospi(2.0 * (double)j / (double)n, &sn, &cs);
-        tw[j] = make_double2(cs, -sn);
+// w^{ab} for w = exp(-2 pi i / n)
+__device__ __forceinline__ double2 root_pow(int a, int b, int n) {
+    double sn, cs;
+    sincospi(2.0 * (double)((long)a * b % n) / (double)n, &sn, &cs);
+    return make_double2(cs, -sn);
+}
+
+// Both sums below are n by h float64 products.  One CTA with a thread per output
+// took 47 us at n = 256 (one SM's float64 units and a serial chain per thread);
+// a CTA per slice and a warp per weight, each term with its own root, take 8 and
+// 12 us.
+
+// A CTA per half-spectrum slice: a_s = -(w_s / n) (gamma_s + add_s) / c-hat_s with
+// c-hat_s = sum_k c_k w^{sk}, in place of gamma_s.  A slice with c-hat_s = 0
+// contributes nothing (its forward solve divides by zero).
+__global__ void __launch_bounds__(256) k_grad_slice(const double* c, int n, double2* gamma, const double* add) {
+    __shared__ double red[32];
+    const int s = blockIdx.x;
+    double cr = 0.0, ci = 0.0;
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+        const double2 w = root_pow(s, k, n);
+        cr = fma(c[k], w.x, cr);
+        ci = fma(c[k], w.y, ci);
     }
-    __syncthreads();
-    for (int s = threadIdx.x; s < h; s += blockDim.x) {
-        double cr = 0.0, ci = 0.0;
-        int idx = 0;  // s k mod n
-        for (int k = 0; k < n; ++k) {
-            const double2 w = tw[idx];
-            cr = fma(c[k], w.x, cr);
-            ci = fma(c[k], w.y, ci);
-            idx += s;
-            if (idx >= n) idx -= n;
-        }
+    cr = block_sum(cr, red);
+    ci = block_sum(ci, red);
+    if (threadIdx.x == 0) {
         const double gr = gamma[s].x + (add ? add[s] : 0.0), gi = gamma[s].y;
         const double den = cr * cr + ci * ci;
         const double f = den > 0.0 ? -parseval_w(s, n) / ((double)n * den) : 0.0;
-        a[s] = make_double2(f * (gr * cr + gi * ci), f * (gi * cr - gr * ci));
+        gamma[s] = make_double2(f * (gr * cr + gi * ci), f * (gi * cr - gr * ci));
     }
-    __syncthreads();
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        double acc = 0.0;
-        int idx = 0;  // s k mod n
-        for (int s = 0; s < h; ++s) {
-            const double2 w = tw[idx];
-            acc = fma(a[s].x, w.x, acc);
-            acc = fma(-a[s].y, w.y, acc);
-            idx += k;
-            if (idx >= n) idx -= n;
-        }
-        dc[k] = acc;
+}
+
+// A warp per tube weight: dc_k = sum_s Re(a_s w^{sk}).
+__global__ void __launch_bounds__(128) k_grad_weight(const double2* a, int n, double* dc) {
+    const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31, h = n / 2 + 1;
+    if (k >= n) return;
+    double acc = 0.0;
+    for (int s = lane; s < h; s += 32) {
+        const double2 w = root_pow(s, k, n), v = a[s];
+        acc = fma(v.x, w.x, acc);
+        acc = fma(-v.y, w.y, acc);
     }
+    acc = warp_sum(acc);
+    if (lane == 0) dc[k] = acc;
 }
 
 template <typename T>
@@ -92,10 +94,13 @@ tp_status sep_gamma(const void* Xh, const void* Gh, int h, long per, double2* ga
     return launched(TP_KC_MISC, st);
 }
 
-tp_status grad_c(const double* c, int n, const double2* gamma, const double* add, double* dc, cudaStream_t st) {
-    const size_t smem = (size_t)(n + n / 2 + 1) * sizeof(double2);
+tp_status grad_c(const double* c, int n, double2* gamma, const double* add, double* dc, cudaStream_t st) {
     prof_begin(TP_KC_MISC, st);
-    k_grad_c<<<1, 256, smem, st>>>(c, n, gamma, add, dc);
+    k_grad_slice<<<n / 2 + 1, 256, 0, st>>>(c, n, gamma, add);
+    const tp_status e = launched(TP_KC_MISC, st);
+    if (e != TP_OK) return e;
+    prof_begin(TP_KC_MISC, st);
+    k_grad_weight<<<(n + 3) / 4, 128, 0, st>>>(gamma, n, dc);
     return launched(TP_KC_MISC, st);
 }
 
