@@ -162,6 +162,8 @@ static size_t gemm_ws(int l, int kk, int m, int n, size_t c) {
 template <typename T>
 static tp_status gemm_t(const void* A, const void* B, void* C, int l, int kk, int m, int n, int trans, void* ws,
                         cudaStream_t st, int tc_passes = 3) {
+    if (sizeof(T) == 4 && tc_passes == 3 && tprod_direct_fits(l, kk, m, n))
+        return tprod_direct((const float*)A, (const float*)B, (float*)C, l, kk, m, n, trans, st);
     const int h = n / 2 + 1;
     const size_t c = 2 * sizeof(T);
     char* p = (char*)ws;

@@ -40,6 +40,8 @@
 // The forward kernel can also emit one float64 partial sum of squares per CTA
 // (used for ||A||_F^2); squares are summed per thread in the working precision
 // and combined in float64 across the CTA.
+#include <limits.h>
+
 #include <algorithm>
 
 #include "common.cuh"
@@ -223,6 +225,9 @@ struct DftPlan {
     int lns;                  // log2 of the sequences per sub-tile
     int nt;                   // threads per CTA
     int kb;                   // direct part: pairs (k, D - k) per thread
+    int cls;                  // dft_class
+    bool split;               // one CTA per sub-tile
+    size_t smem;
 };
 
 // Fewest passes, then the smallest sum of radices, largest radix first.
@@ -250,9 +255,26 @@ static size_t dft_smem(const DftPlan& P, size_t elem, bool fwd) {
     return (P.D > 1 && fwd ? 2 : 1) * buf + (size_t)P.n * c + (((size_t)P.n * 2 + 15) & ~(size_t)15);
 }
 
-static DftPlan make_plan(int n, size_t elem, bool fwd) {
+// Class of a plan: 0 = powers of two, 1 = radices up to 10, 2 = the other
+// products of small primes, 3 = plans with a direct part or whose tiles are
+// split (the others have the sequence count as a compile-time constant).
+static int dft_class(const DftPlan& P) {
+    if (P.lns != 4 || P.D > 1) return 3;
+    int cls = 0;
+    for (int i = 0; i < P.np; ++i) {
+        const int r = P.r[i];
+        if (r > 10 && r != 16) return 2;
+        if (r & (r - 1)) cls = 1;
+    }
+    for (int i = 0; i < P.np; ++i)
+        if (cls == 1 && P.r[i] > 10) return 2;
+    return cls;
+}
+// split: a CTA per sub-tile of four sequences instead of per tile
+static DftPlan make_plan(int n, size_t elem, bool fwd, bool split) {
     DftPlan P;
     P.n = n;
+    P.split = split;
     int m = n;
     P.D = 1;
     for (int q = 17; q <= m; ++q)
@@ -276,29 +298,45 @@ static DftPlan make_plan(int n, size_t elem, bool fwd) {
         L /= P.r[i];
         P.rm[i] = ((1u << 20) + L - 1) / L;
     }
-    P.lns = 4;
+    P.lns = split ? 2 : 4;
     while (P.lns > 2 && dft_smem(P, elem, fwd) > 112 * 1024) --P.lns;
     // a thread per item of the pass with the fewest items
     const int items = (n / (P.np ? P.r[0] : 1)) << P.lns;
     P.nt = std::min(DFT_MAX_THREADS, std::max(64, (items + 31) & ~31));
-    if (P.D > 1) P.nt = DFT_MAX_THREADS;
-    // the direct part's groups of kb pairs run in rounds of nt / (sequences / 2): about kb + 1/2 units of time each
-    P.kb = 4;
-    long best = 1L << 60;
-    for (int kb : {3, 4, 6}) {
-        const int slots = P.nt >> (P.lns - 1), groups = n / P.D * ((P.D / 2 + kb) / kb);
-        const long cost = (long)((groups + slots - 1) / slots) * (2 * kb + 1);
-        if (cost < best) {
-            best = cost;
-            P.kb = kb;
-        }
+    // The direct part: groups of kb pairs on sequences / 2 lanes each, about 12 kb + 4 instructions per entry.
+    // Up to about 370 points one round of some width does (17 .. 61 points on 64 or 128 threads, 331 on 256):
+    // the cheapest of those, counting no fewer than three warps (fewer leave the SM waiting).  Beyond, 256 threads
+    // and the fewest rounds, about kb + 1/2 units of time each.
+    if (P.D > 1) {
+        int cost1 = INT_MAX, cost2 = INT_MAX, nt1 = 0, kb1 = 0, kb2 = 4;
+        for (int nt = DFT_MAX_THREADS; nt >= 64; nt /= 2)
+            for (int kb : {2, 3, 4, 6}) {
+                const int slots = nt >> (P.lns - 1), groups = n / P.D * ((P.D / 2 + kb) / kb);
+                const int rounds = (groups + slots - 1) / slots;
+                const int c1 = std::max(nt, 96) * (12 * kb + 4), c2 = rounds * (2 * kb + 1);
+                if (rounds == 1 && c1 < cost1) {
+                    cost1 = c1;
+                    nt1 = nt;
+                    kb1 = kb;
+                }
+                if (nt == DFT_MAX_THREADS && c2 < cost2) {
+                    cost2 = c2;
+                    kb2 = kb;
+                }
+            }
+        P.nt = nt1 ? nt1 : DFT_MAX_THREADS;
+        P.kb = nt1 ? kb1 : kb2;
+    } else {
+        P.kb = 0;
     }
+    P.smem = dft_smem(P, elem, fwd);
+    P.cls = dft_class(P);
     return P;
 }
 
 // The plans of the last lengths that a thread used (the search takes about a
 // microsecond, which a small transform would notice).
-static const DftPlan& dft_plan(int n, size_t elem, bool fwd) {
+static const DftPlan& dft_plan(int n, size_t elem, bool fwd, bool split) {
     struct Slot {
         DftPlan P;
         size_t elem = 0;
@@ -306,29 +344,14 @@ static const DftPlan& dft_plan(int n, size_t elem, bool fwd) {
     };
     thread_local Slot slots[16];
     Slot& s = slots[((n * 4) ^ (elem == 4 ? 2 : 0) ^ (fwd ? 1 : 0)) & 15];
-    if (s.elem != elem || s.fwd != fwd || s.P.n != n) {
-        s.P = make_plan(n, elem, fwd);
+    if (s.elem != elem || s.fwd != fwd || s.P.n != n || s.P.split != split) {
+        s.P = make_plan(n, elem, fwd, split);
         s.elem = elem;
         s.fwd = fwd;
     }
     return s.P;
 }
 
-// Class of a plan: 0 = powers of two, 1 = radices up to 10, 2 = the other
-// products of small primes, 3 = plans with a direct part or whose tiles are
-// split (the others have the sequence count as a compile-time constant).
-static int dft_class(const DftPlan& P) {
-    if (P.lns != 4 || P.D > 1) return 3;
-    int cls = 0;
-    for (int i = 0; i < P.np; ++i) {
-        const int r = P.r[i];
-        if (r > 10 && r != 16) return 2;
-        if (r & (r - 1)) cls = 1;
-    }
-    for (int i = 0; i < P.np; ++i)
-        if (cls == 1 && P.r[i] > 10) return 2;
-    return cls;
-}
 constexpr int DFT_CTAS[4] = {4, 4, 3, 2};  // CTAs per SM that the registers of each class allow (float32)
 
 // ---- kernels ----------------------------------------------------------------------
@@ -416,6 +439,7 @@ __device__ __forceinline__ void pass_smem(cplx<T>* z, const cplx<T>* tw, int n, 
         }                                                    \
     } else {                                                 \
         switch (r) {                                         \
+            case 1: GO(1); break;                            \
             case 2: GO(2); break;                            \
             case 3: GO(3); break;                            \
             case 4: GO(4); break;                            \
@@ -598,8 +622,13 @@ k_rdft(const __grid_constant__ DftPlan P, const T* __restrict__ X, cplx<T>* __re
     fill_tables<T>(P, tw, pos, false);
     __syncthreads();
     T total = 0;
-    for (int sub = 0; sub < DFT_SEQ; sub += ns) {
-        const long t0 = (long)blockIdx.x * DFT_TILE + 2 * (sub + (threadIdx.x & (ns - 1)));
+    // all sub-tiles of tile blockIdx.x, or (split) one
+    const int nsub = DFT_SEQ >> lns;
+    const long tile = CLS == 3 && P.split ? blockIdx.x / nsub : blockIdx.x;
+    const int sub0 = CLS == 3 && P.split ? (blockIdx.x % nsub) << lns : 0;
+    const int sub1 = CLS == 3 && P.split ? sub0 + ns : DFT_SEQ;
+    for (int sub = sub0; sub < sub1; sub += ns) {
+        const long t0 = tile * DFT_TILE + 2 * (sub + (threadIdx.x & (ns - 1)));
         const bool la = t0 < tubes, lb = t0 + 1 < tubes;
         const T* xa = X + (la ? tube_off(t0, cols, ld) : 0);
         const T* xb = X + (lb ? tube_off(t0 + 1, cols, ld) : 0);
@@ -622,7 +651,7 @@ k_rdft(const __grid_constant__ DftPlan P, const T* __restrict__ X, cplx<T>* __re
         total += acc;
         if (!finite) {
             // the defining sum, tube by tube
-            const long f0 = (long)blockIdx.x * DFT_TILE + 2 * sub;
+            const long f0 = tile * DFT_TILE + 2 * sub;
             for (int e = threadIdx.x; e < h * 2 * ns; e += blockDim.x) {
                 const int s = e / (2 * ns), tt = e - s * 2 * ns;
                 const long t = f0 + tt;
@@ -659,7 +688,8 @@ k_rdft(const __grid_constant__ DftPlan P, const T* __restrict__ X, cplx<T>* __re
         if (CLS == 3 && P.D > 1) {
             direct_fold<T>(z, n, P.D, lns);
             auto put = [&](int b, int k, int q, V v) { z2[((size_t)(b * P.D + k) << lns) + q] = v; };
-            if (P.kb == 3) direct_part<T, 3>(z, tw, n, P.D, lns, put);
+            if (P.kb == 2) direct_part<T, 2>(z, tw, n, P.D, lns, put);
+            else if (P.kb == 3) direct_part<T, 3>(z, tw, n, P.D, lns, put);
             else if (P.kb == 4) direct_part<T, 4>(z, tw, n, P.D, lns, put);
             else direct_part<T, 6>(z, tw, n, P.D, lns, put);
             __syncthreads();
@@ -696,9 +726,13 @@ k_irdft(const __grid_constant__ DftPlan P, const cplx<T>* __restrict__ Xh, T* __
     V* tw = z + ((size_t)n << lns);
     unsigned short* freq = (unsigned short*)(tw + n);
     fill_tables<T>(P, tw, freq, true);
-    for (int sub = 0; sub < DFT_SEQ; sub += ns) {
+    const int nsub = DFT_SEQ >> lns;
+    const long tile = CLS == 3 && P.split ? blockIdx.x / nsub : blockIdx.x;
+    const int sub0 = CLS == 3 && P.split ? (blockIdx.x % nsub) << lns : 0;
+    const int sub1 = CLS == 3 && P.split ? sub0 + ns : DFT_SEQ;
+    for (int sub = sub0; sub < sub1; sub += ns) {
         const int p = threadIdx.x & (ns - 1), sst = blockDim.x >> lns;
-        const long t0 = (long)blockIdx.x * DFT_TILE + 2 * (sub + p);
+        const long t0 = tile * DFT_TILE + 2 * (sub + p);
         const bool la = t0 < tubes, lb = t0 + 1 < tubes;
         T* xa = X + (la ? tube_off(t0, cols, ld) : 0);
         T* xb = X + (lb ? tube_off(t0 + 1, cols, ld) : 0);
@@ -732,7 +766,7 @@ k_irdft(const __grid_constant__ DftPlan P, const cplx<T>* __restrict__ Xh, T* __
         const bool finite = !__syncthreads_or(bad != (T)0 || isnan(bad));
         if (!finite) {
             // the defining sum, tube by tube
-            const long f0 = (long)blockIdx.x * DFT_TILE + 2 * sub;
+            const long f0 = tile * DFT_TILE + 2 * sub;
             const T inv = (T)1 / (T)n;
             for (int e = threadIdx.x; e < n * 2 * ns; e += blockDim.x) {
                 const int k = e / (2 * ns), tt = e - k * 2 * ns;
@@ -772,14 +806,15 @@ k_irdft(const __grid_constant__ DftPlan P, const cplx<T>* __restrict__ Xh, T* __
         if (CLS == 3 && P.D > 1) {
             const T inv = (T)1 / (T)n;
             const int nb = n / P.D;
-            const long f0 = (long)blockIdx.x * DFT_TILE + 2 * sub;
+            const long f0 = tile * DFT_TILE + 2 * sub;
             direct_fold<T>(z, n, P.D, lns);
             auto put = [&](int b, int k, int q, V v) {
                 const long t = f0 + 2 * q, off = (long)(freq[b * P.D] + nb * k) * ss;
                 if (t < tubes) X[tube_off(t, cols, ld) + off] = v.y * inv;
                 if (t + 1 < tubes) X[tube_off(t + 1, cols, ld) + off] = v.x * inv;
             };
-            if (P.kb == 3) direct_part<T, 3>(z, tw, n, P.D, lns, put);
+            if (P.kb == 2) direct_part<T, 2>(z, tw, n, P.D, lns, put);
+            else if (P.kb == 3) direct_part<T, 3>(z, tw, n, P.D, lns, put);
             else if (P.kb == 4) direct_part<T, 4>(z, tw, n, P.D, lns, put);
             else direct_part<T, 6>(z, tw, n, P.D, lns, put);
         } else {
@@ -803,20 +838,27 @@ template <typename T> static int hat_pair_ok(const void* Xh, long tubes) {
     return (tubes & 1) == 0 && ((size_t)Xh & 15) == 0;
 }
 
+// Float64 transforms of few tubes take a CTA per sub-tile: the time is that of
+// one SM's float64 units on its 16 sequences (n = 73, 1600 tubes in 50 tiles:
+// 41 -> 31 us), and most SMs would be idle.  Not where the norm
+// partials are wanted, which are one per tile.
+template <typename T> static bool dft_split(unsigned tiles, const double* sumsq) {
+    return sizeof(T) == 8 && !sumsq && tiles <= 76;
+}
+
 template <typename T>
 tp_status rdft(const T* X, void* Xh, int n, int rows, int cols, long ld, long ss, double* sumsq,
                const int* skip, cudaStream_t st) {
     const long tubes = (long)rows * cols;
     if (tubes == 0) return TP_OK;
-    const unsigned grid = (unsigned)((tubes + DFT_TILE - 1) / DFT_TILE);
-    const DftPlan& P = dft_plan(n, sizeof(T), true);
-    const size_t smem = dft_smem(P, sizeof(T), true);
-    const int cls = dft_class(P);
-    auto kern = cls == 0 ? k_rdft<T, 0> : (cls == 1 ? k_rdft<T, 1> : (cls == 2 ? k_rdft<T, 2> : k_rdft<T, 3>));
-    if (smem_optin((const void*)kern, smem) != TP_OK) return TP_ERR_CUDA;
+    const unsigned tiles = (unsigned)((tubes + DFT_TILE - 1) / DFT_TILE);
+    const DftPlan& P = dft_plan(n, sizeof(T), true, dft_split<T>(tiles, sumsq));
+    auto kern = P.cls == 0 ? k_rdft<T, 0> : (P.cls == 1 ? k_rdft<T, 1> : (P.cls == 2 ? k_rdft<T, 2> : k_rdft<T, 3>));
+    if (smem_optin((const void*)kern, P.smem) != TP_OK) return TP_ERR_CUDA;
     prof_begin(TP_KC_DFT, st);
-    kern<<<grid, P.nt, smem, st>>>(P, X, (cplx<T>*)Xh, tubes, cols, ld, ss, pair_ok<T>(X, tubes, cols, ld, ss),
-                                        hat_pair_ok<T>(Xh, tubes), sumsq, skip);
+    kern<<<tiles * (P.split ? DFT_SEQ >> P.lns : 1), P.nt, P.smem, st>>>(
+        P, X, (cplx<T>*)Xh, tubes, cols, ld, ss, pair_ok<T>(X, tubes, cols, ld, ss), hat_pair_ok<T>(Xh, tubes), sumsq,
+        skip);
     return launched(TP_KC_DFT, st);
 }
 
@@ -825,15 +867,15 @@ tp_status irdft(const void* Xh, T* X, int n, int rows, int cols, long ld, long s
                 cudaStream_t st) {
     const long tubes = (long)rows * cols;
     if (tubes == 0) return TP_OK;
-    const unsigned grid = (unsigned)((tubes + DFT_TILE - 1) / DFT_TILE);
-    const DftPlan& P = dft_plan(n, sizeof(T), false);
-    const size_t smem = dft_smem(P, sizeof(T), false);
-    const int cls = dft_class(P);
-    auto kern = cls == 0 ? k_irdft<T, 0> : (cls == 1 ? k_irdft<T, 1> : (cls == 2 ? k_irdft<T, 2> : k_irdft<T, 3>));
-    if (smem_optin((const void*)kern, smem) != TP_OK) return TP_ERR_CUDA;
+    const unsigned tiles = (unsigned)((tubes + DFT_TILE - 1) / DFT_TILE);
+    const DftPlan& P = dft_plan(n, sizeof(T), false, dft_split<T>(tiles, nullptr));
+    auto kern =
+        P.cls == 0 ? k_irdft<T, 0> : (P.cls == 1 ? k_irdft<T, 1> : (P.cls == 2 ? k_irdft<T, 2> : k_irdft<T, 3>));
+    if (smem_optin((const void*)kern, P.smem) != TP_OK) return TP_ERR_CUDA;
     prof_begin(TP_KC_DFT, st);
-    kern<<<grid, P.nt, smem, st>>>(P, (const cplx<T>*)Xh, X, tubes, cols, ld, ss, hat_pair_ok<T>(Xh, tubes),
-                                         pair_ok<T>(X, tubes, cols, ld, ss), skip);
+    kern<<<tiles * (P.split ? DFT_SEQ >> P.lns : 1), P.nt, P.smem, st>>>(
+        P, (const cplx<T>*)Xh, X, tubes, cols, ld, ss, hat_pair_ok<T>(Xh, tubes), pair_ok<T>(X, tubes, cols, ld, ss),
+        skip);
     return launched(TP_KC_DFT, st);
 }
 

@@ -122,6 +122,12 @@ struct GkmArgs {
 template <typename T> tp_status gkm_config(int l, int m, int n, int k_max, int* nt, size_t* smem);
 template <typename T> tp_status gkm_launch(const GkmArgs& a, int nt, size_t smem, cudaStream_t st);
 
+// C = op(A) * op(B) (trans as tprod_gemm) by the circular convolution itself, one
+// launch, for the small float32 sizes that _fits accepts (tdirect.cu).
+bool tprod_direct_fits(int l, int kk, int m, int n);
+tp_status tprod_direct(const float* A, const float* B, float* C, int l, int kk, int m, int n, int trans,
+                       cudaStream_t st);
+
 // Device-side bookkeeping shared by a solve.
 struct State {
     double norm_a2;   // ||A||_F^2

@@ -1695,33 +1695,73 @@ k_dp_scan(const cplx<T>* __restrict__ KhT, long sK, const cplx<T>* __restrict__ 
         for (int c0 = q_lo; c0 < q_hi; c0 += DP_CC) {
             const int nc = min(DP_CC, q_hi - c0), kb = k_init + c0;  // candidates kb .. kb + nc - 1
             if (CORR) {
-                // T[i][q] = sum_{j < kb+q} U[i][j] a_j: the first column in full, the others by one more
-                // term each (a thread per row i)
-                for (int i = tid; i < r; i += blockDim.x) {
-                    V acc = mk<T>(0, 0);
-                    const V* Ui = U + (long)i * ldu;
-#pragma unroll 4
-                    for (int j = 0; j < kb; ++j) cfma(acc, Ui[j], al[(long)j * np + c]);
-                    Tm[i * DP_CC] = acc;
-                    for (int q = 1; q < nc; ++q) {
-                        const int j = kb + q - 1;
-                        cfma(acc, Ui[j], al[(long)j * np + c]);
-                        Tm[i * DP_CC + q] = acc;
+                // T[i][q] = sum_{j < kb+q} U[i][j] a_j.  First candidate: a warp takes four rows i, its lanes along
+                // them; the others: a thread per row adds one more term for each
+                for (int i0 = 4 * warp; i0 < r; i0 += 4 * nw) {
+                    V acc[4];
+#pragma unroll
+                    for (int d = 0; d < 4; ++d) acc[d] = mk<T>(0, 0);
+                    const V* Ui = U + (long)i0 * ldu;
+                    const long rs = i0 + 4 <= r ? ldu : 0;  // the last rows of an r that is no multiple of four
+#pragma unroll 2
+                    for (int j = lane; j < kb; j += 32) {
+                        const V a = al[(long)j * np + c];
+#pragma unroll
+                        for (int d = 0; d < 4; ++d) cfma(acc[d], Ui[d * rs + j], a);
                     }
+                    if (rs == 0)
+                        for (int d = 1; i0 + d < r; ++d) {
+                            acc[d] = mk<T>(0, 0);
+                            for (int j = lane; j < kb; j += 32) cfma(acc[d], Ui[(long)d * ldu + j], al[(long)j * np + c]);
+                        }
+                    const V t = warp_reduce_scatter<V, 4>(acc);  // lanes 8 d ..: row i0 + d
+                    if ((lane & 7) == 0 && i0 + (lane >> 3) < r) Tm[(i0 + (lane >> 3)) * DP_CC] = t;
                 }
                 __syncthreads();
-                // alpha^(k)_j = 2 a_j - sum_i conj(U[i][j]) T[i][q]
-                for (int e = tid; e < r * nc; e += blockDim.x) {
-                    const int q = e / r, j = e - q * r;
-                    V v = mk<T>(0, 0);
-                    if (j < kb + q) {
-                        V acc = mk<T>(0, 0);
-#pragma unroll 4
-                        for (int i = 0; i < r; ++i) cfmac(acc, U[(long)i * ldu + j], Tm[i * DP_CC + q]);
-                        const V a = al[(long)j * np + c];
-                        v = mk<T>((T)2 * a.x - acc.x, (T)2 * a.y - acc.y);
+                for (int i = tid; i < r; i += blockDim.x) {
+                    V x[DP_CC - 1], t = Tm[i * DP_CC];
+#pragma unroll
+                    for (int q = 1; q < DP_CC; ++q)
+                        x[q - 1] = q < nc ? U[(long)i * ldu + kb + q - 1] : mk<T>(0, 0);
+#pragma unroll
+                    for (int q = 1; q < DP_CC; ++q)
+                        if (q < nc) {
+                            cfma(t, x[q - 1], al[(long)(kb + q - 1) * np + c]);
+                            Tm[i * DP_CC + q] = t;
+                        }
+                }
+                __syncthreads();
+                // alpha^(k)_j = 2 a_j - sum_i conj(U[i][j]) T[i][q]: a thread per column j holds every candidate's
+                // sum (each entry of U read once for all of them), the rows i shared by as many thread groups as fit
+                const int rw = (r + 31) & ~31, G = max(1, (int)blockDim.x / rw);
+                const int g = tid / rw, j = tid - g * rw, rows = (r + G - 1) / G;
+                V sum[DP_CC];
+#pragma unroll
+                for (int q = 0; q < DP_CC; ++q) sum[q] = mk<T>(0, 0);
+                if (g < G && j < r) {
+                    const int i1 = min(r, (g + 1) * rows);
+#pragma unroll 8
+                    for (int i = g * rows; i < i1; ++i) {
+                        const V x = U[(long)i * ldu + j];
+#pragma unroll
+                        for (int q = 0; q < DP_CC; ++q)
+                            if (q < nc) cfmac(sum[q], x, Tm[i * DP_CC + q]);
                     }
-                    ak[q * r + j] = v;
+                }
+                for (int gg = 0; gg < G; ++gg) {
+                    if (g == gg && j < r) {
+#pragma unroll
+                        for (int q = 0; q < DP_CC; ++q)
+                            if (q < nc) {
+                                V v = gg ? cadd(ak[q * r + j], sum[q]) : sum[q];
+                                if (gg == G - 1) {
+                                    const V a = al[(long)j * np + c];
+                                    v = j < kb + q ? mk<T>((T)2 * a.x - v.x, (T)2 * a.y - v.y) : mk<T>(0, 0);
+                                }
+                                ak[q * r + j] = v;
+                            }
+                    }
+                    if (gg + 1 < G) __syncthreads();
                 }
             } else {
                 for (int e = tid; e < r * nc; e += blockDim.x) {
