@@ -143,10 +143,50 @@ __device__ void chol16_par(const cplx<T>* G, cplx<T>* Rk, T* invd, int b, T shif
 }
 
 
-// Row stride (floats) of the partial coefficient tiles of the tensor-core
-// products: 32 re/im entries padded to 40, so that the (row g, columns 2t, 2t+1)
-// pairs of a half-warp's float2 stores fall on 32 distinct banks.
-constexpr int PART_LD = 40;
+// ---- partial coefficient tiles of the tensor-core products -----------------
+// A 16 x 32 (re | im) tile of C is split over KC shares of the reduction, one
+// warp each.  Shares 1 .. KC - 1 leave their accumulators in `part` as they lie
+// in the lanes' registers (2 KB a tile, 16-byte stores of consecutive lanes);
+// share 0 keeps its own, adds the others in order after one barrier, and writes
+// the finished tile.  At most PART_TILES tiles meet there (mt row tiles).
+constexpr int PART_TILES = 15;
+__device__ __forceinline__ int part_shares(int mt, int nw, int nks) {
+    const int kc = min(nw / mt, PART_TILES / mt + 1);
+    return max(1, min(kc, nks));
+}
+__device__ __forceinline__ void part_put(float* part, int tile, const float (&acc)[4][4]) {
+    float4* p = (float4*)part + tile * 128 + (threadIdx.x & 31);
+#pragma unroll
+    for (int a = 0; a < 4; ++a) p[32 * a] = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
+}
+__device__ __forceinline__ void part_add(const float* part, int tile, float (&acc)[4][4]) {
+    const float4* p = (const float4*)part + tile * 128 + (threadIdx.x & 31);
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        const float4 v = p[32 * a];
+        acc[a][0] += v.x;
+        acc[a][1] += v.y;
+        acc[a][2] += v.z;
+        acc[a][3] += v.w;
+    }
+}
+// the finished tile to C (rows row0 .. row0 + 15 below nrow, 16 complex columns); returns its largest component
+__device__ __forceinline__ float part_out(const float (&acc)[4][4], float2* C, int row0, int nrow) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    float m = 0.f;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int row = row0 + g + 8 * h;
+        if (row >= nrow) continue;
+#pragma unroll
+        for (int jh = 0; jh < 2; ++jh) {
+            const float4 v = make_float4(acc[jh][2 * h], acc[2 + jh][2 * h], acc[jh][2 * h + 1], acc[2 + jh][2 * h + 1]);
+            *(float4*)(C + row * 16 + jh * 8 + 2 * t) = v;
+            m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+        }
+    }
+    return m;
+}
 
 // ---- float32 Gram matrix on the tensor cores (mma.sync m16n8k8, tf32) -------
 // The Gram matrix of a block, C = Y^H Y (a coefficient product with the
@@ -181,27 +221,23 @@ __device__ __forceinline__ void mma3(float (&d)[4], const uint32_t (&ah)[4], con
 // Cp (r_prev x 16) = conj(Q) Y for 16 columns of Y (Ys column-major with
 // column stride LP, L a multiple of 16); row i of Q starts at Q + i QS, in
 // global memory (GQ, read with cache-global loads) or in shared memory.
-// Warps take (16-row tile, k range) items; the partial tiles meet in `part`
-// (at most 16 x 16 x PART_LD floats) and are summed over the k ranges in a fixed
-// order.  Ends with a barrier.
+// Warps take (16-row tile, k range) items (part_shares).  Ends with a barrier.
 template <bool GQ>
 __device__ void orth_coef_mma(const float2* __restrict__ Q, int QS, const float2* Ys, int L, int LP, int r_prev,
                               float2* Cp, float* part) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int g = lane >> 2, t = lane & 3;
-    const int mt = (r_prev + 15) / 16, nks = L / 4;
-    int KC = nw / mt;
-    KC = KC < 1 ? 1 : (KC > nks ? nks : KC);
+    const int mt = (r_prev + 15) / 16, nks = L / 4, KC = part_shares(mt, nw, nks);
     constexpr uint32_t SGN = 0x80000000u;
-    for (int it = warp; it < mt * KC; it += nw) {
-        const int mtile = it / KC, kc = it - mtile * KC;
+    const int mtile = warp % mt, kc = warp / mt;  // mt KC <= nw: at most one item per warp
+    float acc[4][4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
+    if (kc < KC) {
         const int ks0 = kc * nks / KC, ks1 = (kc + 1) * nks / KC;
         const int i0 = mtile * 16 + g, i1 = i0 + 8;
-        float acc[4][4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
         for (int ks = ks0; ks < ks1; ++ks) {
             const int e = ks * 4 + t;
             const float2 z = make_float2(0.f, 0.f);
@@ -222,25 +258,12 @@ __device__ void orth_coef_mma(const float2* __restrict__ Q, int QS, const float2
                 mma3(acc[2 + jh], ah, al, yh, yl, xh ^ SGN, xl ^ SGN);    // Im: sum Qr Yi - Qi Yr
             }
         }
-        float* P = part + (size_t)kc * mt * 16 * PART_LD;
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int row = mtile * 16 + g + h * 8, col = nt * 8 + 2 * t;
-                *(float2*)(P + row * PART_LD + col) = make_float2(acc[nt][2 * h], acc[nt][2 * h + 1]);
-            }
+        if (kc > 0) part_put(part, (kc - 1) * mt + mtile, acc);
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < r_prev * 16; idx += blockDim.x) {
-        const int i = idx >> 4, j = idx & 15;
-        float sr = 0.f, si = 0.f;
-        for (int kc = 0; kc < KC; ++kc) {
-            const float* P = part + (size_t)kc * mt * 16 * PART_LD + i * PART_LD;
-            sr += P[j];
-            si += P[16 + j];
-        }
-        Cp[i * 16 + j] = make_float2(sr, si);
+    if (kc == 0) {
+        for (int k = 1; k < KC; ++k) part_add(part, (k - 1) * mt + mtile, acc);
+        part_out(acc, Cp, mtile * 16, r_prev);
     }
     __syncthreads();
 }
@@ -307,31 +330,28 @@ __device__ __forceinline__ float max_of(const float* wmax, int n) {
 // Cp (r_prev x 16) = conj(Q) Y for the 16 columns of Y (Ys column-major with
 // column stride LP, L a multiple of 16); row i of Q (a unit vector) starts at
 // Q + i L in global memory (cache-global loads).  ymax: the largest component
-// of Y.  Warps take (16-row tile, k range) items; the partial tiles, scaled
-// back, meet in `part` and are summed over the k ranges in a fixed order.
+// of Y.  Warps take (16-row tile, k range) items (part_shares).
 // The largest component of Cp goes to cmax_w (one entry per warp).  Ends with
 // a barrier.
 __device__ void orth_coef_h16(const float2* __restrict__ Q, const float2* Ys, int L, int LP, int r_prev, float ymax,
                               float2* Cp, float* part, float* cmax_w) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int g = lane >> 2, t = lane & 3;
-    const int mt = (r_prev + 15) / 16, nks = L / 8;
-    int KC = nw / mt;
-    KC = KC < 1 ? 1 : (KC > nks ? nks : KC);
+    const int mt = (r_prev + 15) / 16, nks = L / 8, KC = part_shares(mt, nw, nks);
     const float sy = h16_scale(ymax), back = 1.f / (H16_QSCALE * sy);
     constexpr uint32_t HI = 0x80000000u;
-    for (int it = warp; it < mt * KC; it += nw) {
-        const int mtile = it / KC, kc = it - mtile * KC;
+    const int mtile = warp % mt, kc = warp / mt;  // mt KC <= nw: at most one item per warp
+    float acc[4][4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[a][c] = 0.f;
+    if (kc < KC) {
         const int ks0 = kc * nks / KC, ks1 = (kc + 1) * nks / KC;
         const int i0 = mtile * 16 + g, i1 = i0 + 8;
         const bool ok0 = i0 < r_prev, ok1 = i1 < r_prev;
         const float2* q0 = Q + (long)i0 * L;
         const float2* q1 = Q + (long)i1 * L;
-        float acc[4][4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) acc[a][c] = 0.f;
         for (int ks = ks0; ks < ks1; ++ks) {
             const int e0 = ks * 8 + t, e1 = e0 + 4;
             const float2 z = make_float2(0.f, 0.f);
@@ -354,27 +374,17 @@ __device__ void orth_coef_h16(const float2* __restrict__ Q, const float2* Ys, in
                       swap_neg(r1l, HI));
             }
         }
-        float* P = part + (size_t)kc * mt * 16 * PART_LD;
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
+        for (int a = 0; a < 4; ++a)
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int row = mtile * 16 + g + h * 8, col = nt * 8 + 2 * t;
-                *(float2*)(P + row * PART_LD + col) = make_float2(acc[nt][2 * h] * back, acc[nt][2 * h + 1] * back);
-            }
+            for (int c = 0; c < 4; ++c) acc[a][c] *= back;
+        if (kc > 0) part_put(part, (kc - 1) * mt + mtile, acc);
     }
     __syncthreads();
     float cm = 0.f;
-    for (int idx = threadIdx.x; idx < r_prev * 16; idx += blockDim.x) {
-        const int i = idx >> 4, j = idx & 15;
-        float sr = 0.f, si = 0.f;
-        for (int kc = 0; kc < KC; ++kc) {
-            const float* P = part + (size_t)kc * mt * 16 * PART_LD + i * PART_LD;
-            sr += P[j];
-            si += P[16 + j];
-        }
-        Cp[i * 16 + j] = make_float2(sr, si);
-        cm = fmaxf(cm, fmaxf(fabsf(sr), fabsf(si)));
+    if (kc == 0) {
+        for (int k = 1; k < KC; ++k) part_add(part, (k - 1) * mt + mtile, acc);
+        cm = part_out(acc, Cp, mtile * 16, r_prev);
     }
     warp_max_to(cm, cmax_w);
     __syncthreads();
@@ -437,17 +447,26 @@ __device__ void orth_update_h16(const float2* __restrict__ Q, float2* Ys, int L,
 }
 
 // Shared-memory extents of k_orth beyond its matrices: the partial tiles of
-// the tensor-core deflation (float32, 16 columns) and the Gram partials (one
-// per thread, at least one per upper-triangle entry).
+// the tensor-core products (float32, 16 columns), and the Gram partials (one
+// per thread, at least one per upper-triangle entry; none in the TC kernel).
 template <typename T, int BB> constexpr size_t orth_part_bytes() {
-    return (sizeof(T) == 4 && BB == 16) ? (size_t)16 * 16 * PART_LD * sizeof(float) : 0;
+    return (sizeof(T) == 4 && BB == 16) ? (size_t)PART_TILES * 2048 : 0;
 }
 template <typename T, int BB> constexpr size_t orth_gram_elems() {
     return (size_t)(BB * (BB + 1) / 2 > OrthThreads<T, BB>::v ? BB * (BB + 1) / 2 : OrthThreads<T, BB>::v);
 }
 
-template <typename T, int BB>
-__global__ void __launch_bounds__(OrthThreads<T, BB>::v)
+// TC: float32 blocks of 16 columns whose products run on the tensor cores (L a
+// multiple of 16, r_prev <= 256); a kernel of its own, without the SIMT forms'
+// code and registers (64 a thread instead of 122), and with shared memory for
+// what the launch needs only (no accumulated R unless R is an output, whose rows
+// above the block are summed in place), so that two CTAs share an SM: with more slices than SMs (n =
+// 512: 257) the launch is one wave instead of two.  512^3 solve (tf32 sketch)
+// 11.00 -> 10.65 ms; seven solves of sizes 64 .. 384 on four streams 8.15 ->
+// 7.40 ms, their CTAs sharing SMs; with at most one slice per SM (256^3) the
+// narrower register file costs nothing (2.57 -> 2.56 ms).
+template <typename T, int BB, bool TC>
+__global__ void __launch_bounds__(OrthThreads<T, BB>::v, TC ? 2 : 1)
 k_orth(cplx<T>* Y, long sY, int L, int b, const cplx<T>* Qb, long sQ, int r_prev, cplx<T>* Qout,
        cplx<T>* R, long ldr, long sR, int r_rows, double* normsq, const int* skip, int final_pass, State* eta,
        int n_dft, int r_new) {
@@ -459,14 +478,15 @@ k_orth(cplx<T>* Y, long sY, int L, int b, const cplx<T>* Qb, long sQ, int r_prev
     // reads) free of shared-memory bank conflicts
     const int LP = L + 1;
     V* Ys = (V*)smraw;
-    V* Cs = Ys + (size_t)BB * LP;           // r_prev x BB, summed over both passes
-    V* Cp = Cs + (size_t)r_prev * BB;       // r_prev x BB, this pass
+    // 16-byte multiples up to here and between (BB (L + 1) is even for BB > 1; BB = 1 is float64)
+    V* Cp = Ys + (size_t)BB * LP;           // r_prev x BB, this pass
     V* G = Cp + (size_t)r_prev * BB;        // BB x BB Gram / Cholesky work
     V* Rk = G + BB * BB;                    // this pass's R
-    V* Ra = Rk + BB * BB;                   // accumulated in-block R
-    V* Rt = Ra + BB * BB;                   // scratch for the product
-    float* part = (float*)(Rt + BB * BB);   // tensor-core deflation: partial coefficient tiles
-    V* gpart = (V*)((unsigned char*)part + orth_part_bytes<T, BB>());  // Gram partials
+    float* part = (float*)(Rk + BB * BB);   // partial coefficient tiles
+    constexpr size_t GRAM = TC ? 0 : orth_gram_elems<T, BB>(), PART = orth_part_bytes<T, BB>();
+    V* gpart = (V*)((unsigned char*)part + PART);  // Gram partials
+    V* Rt = gpart + GRAM;                   // copy of G (SIMT Cholesky), scratch for the product Rk Ra
+    V* Ra = Rt + BB * BB;                   // accumulated in-block R (R an output)
     __shared__ double red[33];
     const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int NW = OrthThreads<T, BB>::v / 32;
@@ -506,7 +526,8 @@ k_orth(cplx<T>* Y, long sY, int L, int b, const cplx<T>* Qb, long sQ, int r_prev
         const int j = b + e / L, row = e - (j - b) * L;
         Ys[j * LP + row] = mk<T>(0, 0);
     }
-    for (int e = tid; e < BB * BB; e += blockDim.x) Ra[e] = mk<T>((e / BB) == (e % BB) ? (T)1 : (T)0, 0);
+    if (R)
+        for (int e = tid; e < BB * BB; e += blockDim.x) Ra[e] = mk<T>((e / BB) == (e % BB) ? (T)1 : (T)0, 0);
     __shared__ float wmax_y[32], wmax_c[32];  // per-warp maxima of |Y| and |Cp| components
     warp_max_to(ymax, wmax_y);                 // published by the barriers of the norm
     const double nnd = block_sum_t(nn, red);
@@ -517,9 +538,8 @@ k_orth(cplx<T>* Y, long sY, int L, int b, const cplx<T>* Qb, long sQ, int r_prev
     if (r_prev > 0) {
         const V* Q = Qb + (long)s * sQ;
         const int dpasses = final_pass ? 2 : 1;
-        const bool tc = sizeof(T) == 4 && BB == 16 && (L & 15) == 0 && r_prev <= 256;  // part: 16 row tiles
         for (int pass = 0; pass < dpasses; ++pass) {
-          if (tc) {
+          if constexpr (TC) {
             orth_coef_h16((const float2*)Q, (const float2*)Ys, L, LP, r_prev, max_of(wmax_y, NW), (float2*)Cp,
                           part, wmax_c);
             orth_update_h16((const float2*)Q, (float2*)Ys, L, LP, r_prev, (const float2*)Cp, max_of(wmax_c, NW),
@@ -596,7 +616,12 @@ k_orth(cplx<T>* Y, long sY, int L, int b, const cplx<T>* Qb, long sQ, int r_prev
                 }
             }
           }
-            for (int e = tid; e < r_prev * BB; e += blockDim.x) Cs[e] = pass ? cadd(Cs[e], Cp[e]) : Cp[e];
+            if (R)  // both passes' coefficients are summed in place (an entry stays with its thread)
+                for (int e = tid; e < r_prev * BB; e += blockDim.x) {
+                    const int i = e / BB, j = e - i * BB;
+                    V* r = R + (long)s * sR + (long)i * ldr + r_prev + j;
+                    if (j < b) *r = pass ? cadd(*r, Cp[e]) : Cp[e];
+                }
             __syncthreads();
         }
     }
@@ -615,9 +640,9 @@ k_orth(cplx<T>* Y, long sY, int L, int b, const cplx<T>* Qb, long sQ, int r_prev
         // coefficient product with the block's own columns as the basis, the
         // full 16 x 16, 3xTF32); otherwise the upper triangle incl. diagonal by
         // a thread per (entry, chunk of rows), the chunk sums meeting in gpart
-        if (sizeof(T) == 4 && BB == 16 && (L & 15) == 0) {
+        if (TC || (sizeof(T) == 4 && BB == 16 && (L & 15) == 0)) {
             orth_coef_mma<false>((const float2*)Ys, LP, (const float2*)Ys, L, LP, 16, (float2*)G, part);
-        } else {
+        } else if constexpr (!TC) {
             constexpr int NE = BB * (BB + 1) / 2;
             // chunks of at least four rows, at most 32 (their sums are added one after another)
             const int nch = max(1, min((int)blockDim.x / NE, min(32, L / 4)));
@@ -761,11 +786,10 @@ k_orth(cplx<T>* Y, long sY, int L, int b, const cplx<T>* Qb, long sQ, int r_prev
     }
     if (R) {
         V* Rs = R + (long)s * sR;
-        for (int e = tid; e < r_rows * b; e += blockDim.x) {
+        for (int e = r_prev * b + tid; e < r_rows * b; e += blockDim.x) {
             const int i = e / b, j = e - i * b;
             V v = mk<T>(0, 0);  // rows below this block stay zero: R is block upper triangular
-            if (i < r_prev) v = Cs[(size_t)i * BB + j];
-            else if (i < r_prev + b) v = Ra[(i - r_prev) * BB + j];
+            if (i < r_prev + b) v = Ra[(i - r_prev) * BB + j];
             Rs[(long)i * ldr + r_prev + j] = v;
         }
     }
@@ -805,12 +829,32 @@ template <typename T> static int orth_cols(int b) {
     return b <= 16 ? 16 : 32;
 }
 
-template <typename T> static size_t orth_smem(int L, int b, int r_prev) {
+template <typename T> static bool orth_tc(int L, int b, int r_prev) {
+    return sizeof(T) == 4 && b <= 16 && (L & 15) == 0 && r_prev <= 256;
+}
+
+template <typename T> static void orth_extents(int BB, size_t& part, size_t& gram) {
+    part = BB == 16 ? orth_part_bytes<T, 16>() : 0;
+    gram = BB == 1 ? orth_gram_elems<T, 1>() : (BB == 4 ? orth_gram_elems<T, 4>() :
+           (BB == 16 ? orth_gram_elems<T, 16>() : orth_gram_elems<T, 32>()));
+}
+template <typename T> static size_t orth_smem(int L, int b, int r_prev, bool has_r) {
     const int BB = orth_cols<T>(b);
-    const size_t part = BB == 16 ? orth_part_bytes<T, 16>() : 0;
-    const size_t gram = BB == 1 ? orth_gram_elems<T, 1>() : (BB == 4 ? orth_gram_elems<T, 4>() :
-                        (BB == 16 ? orth_gram_elems<T, 16>() : orth_gram_elems<T, 32>()));
-    return ((size_t)BB * (L + 1) + 2 * (size_t)r_prev * BB + 4 * BB * BB + gram) * sizeof(cplx<T>) + part;
+    const bool tc = orth_tc<T>(L, b, r_prev);
+    size_t part, gram;
+    orth_extents<T>(BB, part, gram);
+    size_t e = (size_t)BB * (L + 1) + (size_t)r_prev * BB + 2 * BB * BB + (tc ? 0 : gram + BB * BB);
+    if (has_r) e += (tc ? 2 : 1) * BB * BB;
+    return e * sizeof(cplx<T>) + part;
+}
+// The sizes a solve takes: with 40 KB for the tensor-core partials and both
+// coefficient blocks the largest launch stays within 227 KB (orth_smem is less).
+template <typename T> static bool orth_fits(int L, int b, int r) {
+    const int BB = orth_cols<T>(b);
+    size_t part, gram;
+    orth_extents<T>(BB, part, gram);
+    const size_t e = (size_t)BB * (L + 1) + 2 * (size_t)r * BB + 4 * BB * BB + gram;
+    return e * sizeof(cplx<T>) + (part ? 40960 : 0) <= 227 * 1024;
 }
 
 template <typename T>
@@ -818,10 +862,12 @@ static tp_status orth(int h, cplx<T>* Y, long sY, int L, int b, const cplx<T>* Q
                       cplx<T>* Qout, cplx<T>* R, long ldr, long sR, int r_rows, double* normsq, const int* skip,
                       cudaStream_t st, State* eta = nullptr, int n_dft = 0, int r_new = 0) {
     const int final_pass = (Qout != nullptr || R != nullptr) ? 1 : 0;
-    const size_t smem = orth_smem<T>(L, b, r_prev);
-    auto kern = b <= 16 ? k_orth<T, 16> : k_orth<T, 32>;
+    const size_t smem = orth_smem<T>(L, b, r_prev, R != nullptr);
+    auto kern = b <= 16 ? k_orth<T, 16, false> : k_orth<T, 32, false>;
     if constexpr (sizeof(T) == 8)
-        if (b <= 4) kern = b == 1 ? k_orth<T, 1> : k_orth<T, 4>;
+        if (b <= 4) kern = b == 1 ? k_orth<T, 1, false> : k_orth<T, 4, false>;
+    if constexpr (sizeof(T) == 4)
+        if (orth_tc<T>(L, b, r_prev)) kern = k_orth<T, 16, true>;
     const int nt = b <= 16 ? OrthThreads<T, 16>::v : OrthThreads<T, 32>::v;
     if (smem_optin((const void*)kern, smem) != TP_OK) return TP_ERR_CUDA;
     prof_begin(TP_KC_ORTH, st);
@@ -2016,7 +2062,7 @@ static tp_status rt_check(int l, int m, int n, int p, const tp_rtsvd_params* P, 
     if (!(P->tau > 0.0) || !(P->delta >= 0.0) || P->p_over < 0 || P->q_power < 0) return TP_ERR_ARG;
     if (!full && !(P->eps > 0.0) && !(P->eps_rel > 0.0)) return TP_ERR_ARG;
     const int Lmax = l > m ? l : m;
-    if (orth_smem<T>(Lmax, P->block, P->r_max) > 227 * 1024) return TP_ERR_ARG;
+    if (!orth_fits<T>(Lmax, P->block, P->r_max)) return TP_ERR_ARG;
     return TP_OK;
 }
 

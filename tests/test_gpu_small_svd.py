@@ -82,6 +82,17 @@ def test_tall_and_wide(tp, l, m):
     assert float((X.double() - ref).norm() / ref.norm()) < 40 * 1.2e-7 * 10 * math.sqrt(24)
 
 
+@pytest.mark.parametrize("l,m,n", [(64, 64, 331), (48, 40, 320), (16, 16, 609)])
+def test_more_slices_than_multiprocessors(tp, l, m, n):
+    """Two orthonormalisation blocks share a multiprocessor (row counts that are multiples of 16; 40 is not one)."""
+    A, B, _ = problem(l, m, n, 1, 7)
+    Ad, Bd = (torch.from_numpy(v).to("cuda", torch.float32) for v in (A, B))
+    X, info = tp.ttsvd_solve(Ad, Bd, 0.0, 1.1)
+    Ah, Bh = (torch.fft.rfft(v.double(), dim=0) for v in (Ad, Bd))
+    ref = torch.fft.irfft(torch.linalg.pinv(Ah) @ Bh, n=n, dim=0)
+    assert float((X.double() - ref).norm() / ref.norm()) < 40 * 1.2e-7 * 10 * math.sqrt(min(l, m))
+
+
 def test_triplets_at_the_largest_working_set(tp):
     """tgkb_triplets with k = 119 fills the shared memory of the small SVD."""
     n, N, k = 2, 130, 119
