@@ -58,7 +58,7 @@ NCU_TRAFFIC = {
     "gkb": {"bytes": 68.89e6, "sources": ["gkb.cu"], "profile": "profiles/k_gkb_n256.md"},
     "orth": {"bytes": 7.38e6, "sources": ["rtsvd.cu"], "profile": "profiles/k_orth_n256.md"},
     "svd": {"bytes": 9.71e6, "sources": ["rtsvd.cu"], "profile": "profiles/k_jacobi_n256.md"},
-    "dft": {"bytes": 26.68e6, "sources": ["dft.cu"], "profile": "profiles/k_rdft_16q_n256_n512.md"},
+    "dft": {"bytes": 26.68e6, "sources": ["dft.cu"], "profile": "profiles/k_rdft_n256_n384.md"},
     "dp": {"bytes": 17.66e6, "sources": ["rtsvd.cu"], "profile": "profiles/launches_n256_bench_step.md"},
 }
 
