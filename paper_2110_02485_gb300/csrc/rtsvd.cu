@@ -1187,18 +1187,19 @@ __device__ __forceinline__ float rsqrt_nr(float x) {
 // lanes and round moved every column to and from shared memory once per
 // rotation (half of its time at r = 96, and four times that through L2 when R
 // is in global memory); here a column moves once per four rotations, a
-// barrier comes once per 16 pairs instead of once per 4, and a rotation takes
-// 8 multiply-adds per entry instead of 12, because its cosine is kept as a
-// scale of the column that is applied when the column is stored:
-// x' = x - (t conj(e) d_y / d_x) y, y' = y + (t e d_x / d_y) x, d' = c d.
+// barrier comes once per 16 pairs instead of once per 4.  Columns and right-hand
+// sides take the same rounded pair (c, s e), 12 multiply-adds per entry:
+// x' = c x - conj(s e) y, y' = c y + s e x, whose columns are orthogonal and
+// equally long whatever the rounding.  (Keeping the cosines as scales of the
+// columns takes 8, but its two coefficients t d_y / d_x and t d_x / d_y round apart
+// from each other and from the right-hand sides' pair: the error of a solution
+// grew by a fifth, r = 128, condition 3: 27 u against 22.)
 // A pair of blocks goes to 16 lanes up to r = 128, to 32 beyond: fewer lanes share
 // the reductions and the rotation's scalar work among more entries.  Measured
-// (one pair per eight lanes -> pair of blocks per warp -> this; 129, 257 and
-// 129 slices): r = 96, six sweeps 691 -> 586 -> 587 us; r = 128 2711 -> 2370 ->
-// 2115 us; r = 256 from global memory 3.2 -> 1.9 -> 1.7 ms per sweep.  At r = 96
-// six warps issue 509 instructions each per step (192 of them multiply-adds)
-// and twelve would issue 395: the first wait for latencies (1.5 instructions
-// per cycle per SM), the second for issue slots (2.3), in the same time.
+// (one pair per eight lanes -> this; 129, 257 and 129 slices): r = 96, six sweeps
+// 691 -> 559 us; r = 128, seven sweeps 2711 -> 2271 us; r = 256 from global memory 3.2
+// -> 1.46 ms per sweep.  At r = 96 twelve warps of 32 lanes per pair of blocks take
+// the same time as six of 16: fewer instructions a warp, but twice the warps.
 //
 // Step KIND pairs column slots P(i), Q(i), i < 4: 0-3 slot i of the first block
 // with slot (i + KIND) mod 4 of the second, 4-6 the three pairings inside a
@@ -1232,18 +1233,12 @@ template <int GL> __device__ __forceinline__ float reduce8(const float (&w)[8]) 
     for (int o = GL / 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     return c;
 }
-// one or two ulp; infinite for an infinite argument
-__device__ __forceinline__ float sqrt_fast(float x) {
-    float y;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 
-// Per-group scratch: (squared norm, scale) of the eight columns, and the two
-// coefficients of each of a step's four rotations.
+// Per-group scratch: the squared norms of the eight columns, and (c, s e) of each
+// of a step's four rotations.
 struct JacGroup {
-    float2 sc[8];
     float4 cf[4];
+    float sq[8];
 };
 
 template <int KIND, int GL, int EPL>
@@ -1252,7 +1247,7 @@ __device__ __forceinline__ void jac_step(float2 (&v)[8][EPL], JacGroup& W, int c
     constexpr int PL = GL / 4;  // lanes per pair
     const int hl = threadIdx.x & (GL - 1), pid = hl / PL;
     const int ps = jac_p(KIND, pid), qs = jac_q(KIND, pid);
-    const float2 A = W.sc[ps], B = W.sc[qs];
+    const float A = W.sq[ps], B = W.sq[qs];
     float w[8];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -1263,35 +1258,33 @@ __device__ __forceinline__ void jac_step(float2 (&v)[8][EPL], JacGroup& W, int c
         w[2 * i + 1] = g.y;
     }
     const float mine = reduce8<GL>(w), other = __shfl_xor_sync(0xffffffffu, mine, GL / 8);
-    const float dd = A.y * B.y;
     const bool part = hl & (GL / 8);
-    const float2 g = make_float2((part ? other : mine) * dd, (part ? mine : other) * dd);
-    const float ag2 = fmaf(g.x, g.x, g.y * g.y), ab = A.x * B.x;
+    const float2 g = make_float2(part ? other : mine, part ? mine : other);
+    const float ag2 = fmaf(g.x, g.x, g.y * g.y), ab = A * B;
     if (ab > 0.f) mo2 = fmaxf(mo2, __fdividef(ag2, ab));
-    const bool rot = A.x > 0.f && B.x > 0.f && ag2 >= 1.17549435e-38f && ag2 > tol2 * ab;
+    const bool rot = A > 0.f && B > 0.f && ag2 >= 1.17549435e-38f && ag2 > tol2 * ab;
     if (!__any_sync(0xffffffffu, rot)) return;
     any = 1;
-    float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 f = make_float4(1.f, 0.f, 0.f, 0.f);
     if (rot) {
         const float rg = rsqrt_nr(ag2);  // 1/|g|
-        const float2 e = make_float2(g.x * rg, g.y * rg);
-        const float zeta = (B.x - A.x) * 0.5f * rg;
-        const float tt = __fdividef(copysignf(1.f, zeta), fabsf(zeta) + sqrt_fast(fmaf(zeta, zeta, 1.f)));
+        const float zeta = (B - A) * 0.5f * rg;
+        const float tt = __fdividef(copysignf(1.f, zeta), fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.f)));
         const float c = rsqrt_nr(fmaf(tt, tt, 1.f)), sn = c * tt;
-        const float f1 = tt * __fdividef(B.y, A.y), f2 = tt * __fdividef(A.y, B.y);
-        f = make_float4(e.x * f1, -e.y * f1, e.x * f2, e.y * f2);
+        const float2 se = make_float2(g.x * rg * sn, g.y * rg * sn);
+        f = make_float4(c, se.x, se.y, 0.f);
         if ((hl & (PL - 1)) == 0) {
             const float tg = tt * (ag2 * rg);  // t |g|
-            W.sc[ps] = make_float2(fmaxf(A.x - tg, 0.f), A.y * c);
-            W.sc[qs] = make_float2(fmaxf(B.x + tg, 0.f), B.y * c);
+            W.sq[ps] = fmaxf(A - tg, 0.f);
+            W.sq[qs] = fmaxf(B + tg, 0.f);
         }
         float2* dx = dp + (ps < 4 ? col0 + ps : col1 + ps - 4) * np;
         float2* dy = dp + (qs < 4 ? col0 + qs : col1 + qs - 4) * np;
         for (int cc = hl & (PL - 1); cc < np; cc += PL) {  // the rows p, q of d' (np right-hand sides)
             const float2 x = dx[cc], y = dy[cc];
-            const float2 ey = cmul(e, y), ex = cmul(cconj(e), x);
-            dx[cc] = make_float2(c * x.x - sn * ey.x, c * x.y - sn * ey.y);
-            dy[cc] = make_float2(sn * ex.x + c * y.x, sn * ex.y + c * y.y);
+            const float2 sy = cmul(se, y), sx = cmul(cconj(se), x);
+            dx[cc] = make_float2(fmaf(c, x.x, -sy.x), fmaf(c, x.y, -sy.y));
+            dy[cc] = make_float2(fmaf(c, y.x, sx.x), fmaf(c, y.y, sx.y));
         }
     }
     if ((hl & (PL - 1)) == 0) W.cf[pid] = f;
@@ -1304,10 +1297,10 @@ __device__ __forceinline__ void jac_step(float2 (&v)[8][EPL], JacGroup& W, int c
             float2& x = v[jac_p(KIND, i)][k];
             float2& y = v[jac_q(KIND, i)][k];
             const float2 x0 = x, y0 = y;
-            x.x = fmaf(-r.x, y0.x, fmaf(r.y, y0.y, x0.x));
-            x.y = fmaf(-r.x, y0.y, fmaf(-r.y, y0.x, x0.y));
-            y.x = fmaf(r.z, x0.x, fmaf(-r.w, x0.y, y0.x));
-            y.y = fmaf(r.z, x0.y, fmaf(r.w, x0.x, y0.y));
+            x.x = fmaf(r.x, x0.x, -fmaf(r.y, y0.x, r.z * y0.y));
+            x.y = fmaf(r.x, x0.y, -fmaf(r.y, y0.y, -r.z * y0.x));
+            y.x = fmaf(r.x, y0.x, fmaf(r.y, x0.x, -r.z * x0.y));
+            y.y = fmaf(r.x, y0.y, fmaf(r.y, x0.y, r.z * x0.x));
         }
     }
     __syncwarp();
@@ -1379,36 +1372,34 @@ __device__ int jacobi_sweeps_blk(float2* Rs, int ld, float2* dp, int np, int r, 
                         for (int e = 0; e < EPL; ++e) w[s] = fmaf(v[s][e].x, v[s][e].x, fmaf(v[s][e].y, v[s][e].y, w[s]));
                     }
                     const float n2 = reduce8<GL>(w);  // GL / 8 lanes hold each slot
-                    if ((hl & (GL / 8 - 1)) == 0) W.sc[hl / (GL / 8)] = make_float2(n2, 1.f);
+                    if ((hl & (GL / 8 - 1)) == 0) W.sq[hl / (GL / 8)] = n2;
                     __syncwarp();
                     jac_step<4, GL, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
                     jac_step<5, GL, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
                     jac_step<6, GL, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
                 } else {
-                    if (hl < 8) W.sc[hl] = make_float2(mycol < r ? cn[mycol] : 0.f, 1.f);
+                    if (hl < 8) W.sq[hl] = mycol < r ? cn[mycol] : 0.f;
                     __syncwarp();
                 }
                 jac_step<0, GL, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
                 jac_step<1, GL, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
                 jac_step<2, GL, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
                 jac_step<3, GL, EPL>(v, W, col0, col1, dp, np, tol2, mo2, any);
-                if (hl < 8 && mycol < r) cn[mycol] = W.sc[hl].x;
+                if (hl < 8 && mycol < r) cn[mycol] = W.sq[hl];
 #pragma unroll
                 for (int s = 0; s < 8; ++s) {
                     const int col = s < 4 ? col0 + s : col1 + s - 4;
                     const bool ok = (FULL && NG == 1) || col < r;
-                    const float d = W.sc[s].y;
                     float2* dst = Rs + (size_t)col * ld;
                     if (VEC) {
 #pragma unroll
                         for (int e = 0; e < EPL; e += 2)
                             if (ok && (FULL || idx(e) < ld))
-                                *(float4*)(dst + idx(e)) = make_float4(v[s][e].x * d, v[s][e].y * d, v[s][e + 1].x * d,
-                                                                       v[s][e + 1].y * d);
+                                *(float4*)(dst + idx(e)) = make_float4(v[s][e].x, v[s][e].y, v[s][e + 1].x, v[s][e + 1].y);
                     } else {
 #pragma unroll
                         for (int e = 0; e < EPL; ++e)
-                            if (ok && (FULL || idx(e) < r)) dst[idx(e)] = cscale(v[s][e], d);
+                            if (ok && (FULL || idx(e) < r)) dst[idx(e)] = v[s][e];
                     }
                 }
                 __syncwarp();  // W is read before the next pair's setup
