@@ -1,41 +1,49 @@
 // Mode-3 DFT along the tubes of a frontal-slice-major tensor (Section 2:
 // fft(A,[],3) and its inverse), real data <-> half spectrum, any n.
 //
-// One CTA owns 32 neighbouring tubes as 16 packed complex sequences (tube 2p
-// the real, tube 2p + 1 the imaginary part of sequence p), so that a row of a
-// slice is one 8-byte load per lane and a row of the spectrum one 16-byte
-// store.  n = r_1 r_2 .. r_np D: the transform is an in-place
-// decimation-in-frequency FFT in shared memory, one pass per radix r_i <= 16
-// (the register DFTs below), followed by direct DFTs of length D, the part of
-// n made of primes above 13 (D = 1 for most n).  The passes leave the
-// spectrum in digit-reversed order.
-//   forward: the first pass reads its r_1 rows straight from global memory
-//     (r_1 loads in flight per thread); the last pass writes shared memory, from
-//     which the two tubes of a sequence are separated by conjugate symmetry;
-//   inverse: the half spectrum becomes the packed full spectrum in shared
-//     memory (re and im swapped: the inverse DFT is the swapped DFT of the
-//     swapped data); the last pass writes its rows straight to global memory.
-// So n = r_1 r_2 moves every element through shared memory two (inverse) or
-// three (forward) times.
+// Every tube is transformed by itself: no sum or product takes entries of two
+// tubes, so a tube's error is relative to its own norm whatever lies beside it
+// (lateral slices of very different scale, zeros, a NaN).  Two tubes as the real
+// and imaginary part of one complex sequence halve the work too, but carry the
+// larger one's rounding into the smaller: a slice 1e-6 of its neighbour came out
+// with a relative error of 6e-2.
 //
-// What bounds it: HBM (12 bytes per element and direction), short of it the
-// issue rate (62 % of the issue slots at 256 x 256 x 256, register DFTs,
-// twiddles and shared-memory addresses) with 50 % occupancy.  Measured from a
-// flushed L2 (CUDA events, forward / inverse), before: the direct sums over n
-// that every n but the powers of two took, a radix-2 kernel for those, and
-// kernels written for n = 256 and 512:
-//   n    tubes      now                     before
-//   96   256 x 256   21 / 23 us              116 / 140 us   (direct)
-//   128  256 x 256   21 / 23 us              54 / 38 us     (radix 2)
-//   256  256 x 256   36 / 40 us (3.8 TB/s)   38 / 43 us     (16 x 16)
-//   331  256 x 256   322 / 289 us            1169 / 1484 us (direct; 331 is prime)
-//   384  384 x 384   118 / 118 us (3.9 TB/s) 3392 / 4326 us (direct)
-//   512  512 x 512   275 / 283 us (3.9 TB/s) 274 / 436 us   (16 x 32; radix 2)
-//   1000 256 x 256   219 / 184 us            18654 / 19093 us (direct)
+// One CTA owns 32 neighbouring tubes, a lane each: a row of a slice is 128 bytes a
+// warp, a row of the spectrum 256.  n = first M, M = r_0 r_1 ..: decimation in
+// frequency, whose first step is a real DFT of `first` points over the rows j, j + M,
+// .., j < M; only its outputs k <= first / 2 are kept (the others are conjugates),
+// times exp(-2 pi i j k / n): blocks of M complex words, whose DFTs are the frequencies
+// k + first k2, one pass per radix r_i <= 16 (the register DFTs below).
+//   forward: the first pass reads its rows straight from global memory, the last
+//     one writes its frequencies straight to the spectrum (the conjugate where
+//     one is above n / 2);
+//   inverse: the transpose: the first pass reads the blocks from the half spectrum
+//     (re and im swapped: the inverse DFT is the swapped DFT of the swapped data),
+//     the last one is the real inverse of `first` points, whose rows go to global
+//     memory.
+// So n = first r_0 moves every element through shared memory once.  Where n has
+// primes above 13, their product is `first` and its real DFTs are direct sums
+// (e_q, o_q below), formed on pairs of tubes part by part.
 //
-// Two tubes share a sequence, so a NaN or infinity in one would reach the
-// other.  A CTA that meets one (or squares that overflow) evaluates the
-// defining sums tube by tube instead (rare, slow, correct).
+// What bounds it: HBM (about 4 bytes per element to read and 4 to write, in
+// either direction), short of it the issue rate and, at n near 256, the loads in
+// flight.  Measured on 256 x 256 tubes with buffers that exceed the L2 (CUDA events
+// over a graph of launches, forward / inverse), and before: the direct sums over n
+// that every n but the powers of two took (1), a radix-2 kernel for those and
+// 16 x 16 and 16 x 32 forms for n = 256 and 512, and two tubes as one complex sequence (2):
+//   n     now                      (1)              (2)
+//   96    16.0 / 14.8 us           111 / 135        14.6 / 15.0
+//   128   14.7 / 16.6 us           49 / 32          14.2 / 16.6
+//   256   30.7 / 32.8 us (4.4 TB/s) 31 / 37         29.9 / 34.1
+//   331   280 / 268 us             1166 / 1480      324 / 283   (prime)
+//   384   48.9 / 50.0 us (4.1 TB/s) 1571 / 1980     53.5 / 55.2
+//   512   62.7 / 67.1 us (4.3 TB/s) 73 / 123        73.0 / 77.8
+//   1000  210 / 182 us             18651 / 19087    215 / 178
+// The forward's root mean square error at 256 and 384 is 0.90e-7 and 0.95e-7 (0.99e-7 and
+// 1.19e-7 in the form (2)): the first sums and differences are taken on exact data.
+//
+// A tile with a NaN, an infinity or squares that overflow evaluates the defining
+// sums instead (rare, slow): an infinity stays in the entries it reaches.
 //
 // The forward kernel can also emit one float64 partial sum of squares per CTA
 // (used for ||A||_F^2); squares are summed per thread in the working precision
@@ -50,9 +58,9 @@
 namespace tp {
 
 constexpr int DFT_TILE = 32;   // tubes per CTA
-constexpr int DFT_SEQ = 16;    // packed sequences per CTA
 constexpr int DFT_MAX_THREADS = 256;
 constexpr int DFT_MAX_PASS = 10;
+constexpr unsigned DFT_FULL = 4 * 152;  // tiles from which on every SM holds several CTAs
 
 template <typename T> __device__ __forceinline__ void sincospi_t(T x, T* s, T* c);
 template <> __device__ __forceinline__ void sincospi_t<float>(float x, float* s, float* c) { sincospif(x, s, c); }
@@ -215,20 +223,167 @@ template <typename T> struct RDft<T, 12> : RDftComp<T, 4, 3> {};
 template <typename T> struct RDft<T, 15> : RDftComp<T, 3, 5> {};
 template <typename T> struct RDft<T, 16> : RDftComp<T, 4, 4> {};
 
+// R reals: X_k, k <= R / 2, and back, from e_q = x_q + x_{R-q} and o_q = x_q - x_{R-q}
+// (formed first: exact, or nearly, on the symmetric tubes that blurs have).
+//   R odd: X_k = (x_0 + sum e_q cos(2 pi q k / R), -sum o_q sin(2 pi q k / R)); the same sums,
+//     with (Re X_k, Im X_k) for (e, o), give the outputs q and R - q as their sum and difference.
+//   R even, H = R / 2: the even X_k are the DFT of length H of x_t + x_{t+H}, whose pairs are
+//     e_q + e_{H-q} and o_q - o_{H-q}; the odd ones are the sums over e_q - e_{H-q} and o_q + o_{H-q}
+//     (cos changes its sign from q to H - q, sin does not).  The inverse is the transpose.
+template <typename T, int R> struct RealDft {
+    static constexpr int H = R / 2;                            // the last k
+    static constexpr int E = R % 2 ? R / 2 : (R / 2 - 1) / 2;  // pairs (q, R - q), or (t, R / 2 - t)
+    // v += (sum e_q cos(2 pi q k / R), -sum o_q sin(2 pi q k / R)), q = 1 .. E
+    template <int K, int Q> static __device__ __forceinline__ void terms(const T (&e)[E + 1], const T (&o)[E + 1], cplx<T>& v) {
+        if constexpr (Q <= E) {
+            constexpr double cd = root_cos(K * Q, R), sd = root_sin(K * Q, R);
+            const T c = (T)cd, s = (T)sd;
+            v.x = fma(e[Q], c, v.x);
+            v.y = fma(-o[Q], s, v.y);
+            terms<K, Q + 1>(e, o, v);
+        }
+    }
+    template <int K, int STEP> static __device__ __forceinline__ void outputs(const T (&e)[E + 1], const T (&o)[E + 1],
+                                                                              T mid, cplx<T> (&v)[H + 1]) {
+        if constexpr (K <= H) {
+            v[K] = mk<T>(e[0], K % 4 == 3 ? mid : -mid);
+            terms<K, 1>(e, o, v[K]);
+            if constexpr (2 * K == R) v[K].y = 0;
+            outputs<K + STEP, STEP>(e, o, mid, v);
+        }
+    }
+    // P = (R - 1) / 2 pairs e, o (entries 1 .. P), x_0 and, R even, x_{R/2}
+    static constexpr int P = (R - 1) / 2;
+    static __device__ __forceinline__ void from_pairs(T x0, T xh, const T (&e)[P + 1], const T (&o)[P + 1],
+                                                      cplx<T> (&v)[H + 1]) {
+        if constexpr (R % 2) {
+            T a[P + 1], s = x0;
+            a[0] = x0;
+#pragma unroll
+            for (int q = 1; q <= P; ++q) {
+                a[q] = e[q];
+                s += e[q];
+            }
+            outputs<1, 1>(a, o, (T)0, v);
+            v[0] = mk<T>(s, 0);
+        } else {
+            typedef RealDft<T, H> Half;
+            T e2[Half::P + 1], o2[Half::P + 1], a[E + 1], b[E + 1];
+            cplx<T> u[H / 2 + 1];
+            e2[0] = o2[0] = b[0] = 0;
+#pragma unroll
+            for (int q = 1; q <= Half::P; ++q) {
+                e2[q] = e[q] + e[H - q];
+                o2[q] = o[q] - o[H - q];
+            }
+            Half::from_pairs(x0 + xh, H % 2 ? (T)0 : e[H / 2], e2, o2, u);
+#pragma unroll
+            for (int k = 0; k <= H / 2; ++k) v[2 * k] = u[k];
+            a[0] = x0 - xh;
+#pragma unroll
+            for (int q = 1; q <= E; ++q) {
+                a[q] = e[q] - e[H - q];
+                b[q] = o[q] + o[H - q];
+            }
+            outputs<1, 2>(a, b, H % 2 ? (T)0 : o[H / 2], v);
+        }
+    }
+    static __device__ __forceinline__ void forward(const T (&x)[R], cplx<T> (&v)[H + 1]) {
+        T e[P + 1], o[P + 1];
+        e[0] = o[0] = 0;
+#pragma unroll
+        for (int q = 1; q <= P; ++q) {
+            e[q] = x[q] + x[R - q];
+            o[q] = x[q] - x[R - q];
+        }
+        from_pairs(x[0], R % 2 ? (T)0 : x[H], e, o, v);
+    }
+    // odd k of the inverse, the transposed sums: z += (sum a_k cos(2 pi t k / R), -sum b_k sin(2 pi t k / R))
+    template <int TT, int K> static __device__ __forceinline__ void odd_terms(const cplx<T> (&v)[H + 1], cplx<T>& z) {
+        if constexpr (K <= H) {
+            constexpr double cd = root_cos(K * TT, R), sd = root_sin(K * TT, R);
+            const T c = (T)cd, s = (T)sd;
+            z.x = fma(v[K].x, c, z.x);
+            z.y = fma(-v[K].y, s, z.y);
+            odd_terms<TT, K + 2>(v, z);
+        }
+    }
+    template <int TT> static __device__ __forceinline__ void odd_outputs(const cplx<T> (&v)[H + 1], T (&z)[H > 0 ? H : 1]) {
+        if constexpr (TT <= E) {
+            cplx<T> c = mk<T>(0, 0);
+            odd_terms<TT, 1>(v, c);
+            z[TT] = c.x + c.y;
+            z[H - TT] = c.y - c.x;
+            odd_outputs<TT + 1>(v, z);
+        }
+    }
+    // x_q = sum_k v_k.x cos(2 pi q k / R) - v_k.y sin(2 pi q k / R): the caller has doubled the k that stand for two
+    static __device__ __forceinline__ void inverse(const cplx<T> (&v)[H + 1], T (&x)[R]) {
+        if constexpr (R % 2) {
+            T e[E + 1], o[E + 1], s = v[0].x;
+            cplx<T> w[H + 1];
+#pragma unroll
+            for (int k = 0; k <= E; ++k) {
+                e[k] = v[k].x;
+                o[k] = v[k].y;
+                if (k > 0) s += e[k];
+            }
+            outputs<1, 1>(e, o, (T)0, w);
+            x[0] = s;
+#pragma unroll
+            for (int q = 1; q <= E; ++q) {
+                x[q] = w[q].x + w[q].y;
+                x[R - q] = w[q].x - w[q].y;
+            }
+        } else {
+            cplx<T> u[H / 2 + 1];
+            T y[H], z[H];
+#pragma unroll
+            for (int k = 0; k <= H / 2; ++k) u[k] = v[2 * k];
+            RealDft<T, H>::inverse(u, y);
+            z[0] = 0;
+            if constexpr (H % 2 == 0) z[H / 2] = 0;
+#pragma unroll
+            for (int k = 1; k <= H; k += 2) {
+                z[0] += v[k].x;
+                if constexpr (H % 2 == 0) z[H / 2] += k % 4 == 3 ? v[k].y : -v[k].y;
+            }
+            odd_outputs<1>(v, z);
+#pragma unroll
+            for (int t = 0; t < H; ++t) {
+                x[t] = y[t] + z[t];
+                x[t + H] = y[t] - z[t];
+            }
+        }
+    }
+};
+template <typename T> struct RealDft<T, 1> {
+    static constexpr int P = 0;
+    static __device__ __forceinline__ void from_pairs(T x0, T, const T (&)[1], const T (&)[1], cplx<T> (&v)[1]) {
+        v[0] = mk<T>(x0, 0);
+    }
+    static __device__ __forceinline__ void forward(const T (&x)[1], cplx<T> (&v)[1]) { v[0] = mk<T>(x[0], 0); }
+    static __device__ __forceinline__ void inverse(const cplx<T> (&v)[1], T (&x)[1]) { x[0] = v[0].x; }
+};
+
+constexpr int DFT_FIRST[] = {32, 24, 20, 18, 16, 15, 14, 13, 12, 11, 10, 9, 8, 7, 6, 5, 4, 3, 2, 1};  // real
 constexpr int DFT_RADICES[] = {16, 15, 13, 12, 11, 10, 9, 8, 7, 6, 5, 4, 3, 2, 1};
 
 // ---- the plan -------------------------------------------------------------------
 struct DftPlan {
-    int n = 0, np, D;         // n = r[0] .. r[np-1] D
+    int n = 0, first, M;      // n = first M: the real radix (or direct part), and the length of its blocks
+    int D, np;                // direct part (the primes above 13); M = r[0] .. r[np-1]
     int r[DFT_MAX_PASS];
-    unsigned rr[DFT_MAX_PASS], rm[DFT_MAX_PASS];  // ceil(2^20 / r) and ceil(2^20 / M) of each pass (M: see pass_smem)
-    int lns;                  // log2 of the sequences per sub-tile
+    unsigned ff, fm, rr[DFT_MAX_PASS], rm[DFT_MAX_PASS];  // ceil(2^20 / first), / M, / r and / (r's M, see pass_smem)
+    int len;                  // complex words per tube: blocks 0 .. first / 2
+    int lns;                  // log2 of the tubes per sub-tile
     int nt;                   // threads per CTA
     int kb;                   // direct part: pairs (k, D - k) per thread
     int cls;                  // dft_class
-    bool split;               // one CTA per sub-tile
+    bool split, full;         // one CTA per sub-tile; tiles for several CTAs on every SM
     size_t smem;
 };
+enum { DFT_GENERAL = 3, DFT_DIRECT = 4, DFT_CLASSES = 5 };
 
 // Fewest passes, then the smallest sum of radices, largest radix first.
 static void best_radices(int m, int max_idx, int depth, int sum, int* cur, int* best, int* best_np, int* best_sum) {
@@ -248,33 +403,39 @@ static void best_radices(int m, int max_idx, int depth, int sum, int* cur, int* 
         }
 }
 
-// sequences per sub-tile: all 16 while two CTAs fit on an SM (the direct part
-// needs a second buffer in the forward kernel), else 8 or 4, one after another
-static size_t dft_smem(const DftPlan& P, size_t elem, bool fwd) {
-    const size_t c = 2 * elem, buf = ((size_t)P.n << P.lns) * c;
-    return (P.D > 1 && fwd ? 2 : 1) * buf + (size_t)P.n * c + (((size_t)P.n * 2 + 15) & ~(size_t)15);
+// Tubes per sub-tile: a whole tile while two CTAs fit on an SM, else a half or
+// a quarter, one after another.  A direct part works on pairs of tubes (n words
+// of two reals each) beside the blocks, where there are any.
+static size_t dft_smem(const DftPlan& P, size_t elem) {
+    const size_t c = 2 * elem;
+    size_t words = (size_t)P.len << P.lns;
+    if (P.cls == DFT_DIRECT) words = ((size_t)P.n << (P.lns - 1)) + (P.M > 1 ? words : 0);
+    return (words + P.n) * c + (((size_t)P.n * 2 + 15) & ~(size_t)15);
 }
 
 // Class of a plan: 0 = powers of two, 1 = radices up to 10, 2 = the other
-// products of small primes, 3 = plans with a direct part or whose tiles are
-// split (the others have the sequence count as a compile-time constant).
+// products of small primes, 3 = those whose tiles are split (the others have
+// the tube count as a compile-time constant), 4 = lengths with a direct part (and 1).
 static int dft_class(const DftPlan& P) {
-    if (P.lns != 4 || P.D > 1) return 3;
+    if (P.D > 1 || P.n == 1) return DFT_DIRECT;
+    if (P.lns != 5) return DFT_GENERAL;
     int cls = 0;
-    for (int i = 0; i < P.np; ++i) {
-        const int r = P.r[i];
+    for (int i = -1; i < P.np; ++i) {
+        const int r = i < 0 ? P.first : P.r[i];
         if (r > 10 && r != 16) return 2;
         if (r & (r - 1)) cls = 1;
     }
-    for (int i = 0; i < P.np; ++i)
-        if (cls == 1 && P.r[i] > 10) return 2;
+    for (int i = -1; i < P.np; ++i)
+        if (cls == 1 && (i < 0 ? P.first : P.r[i]) > 10) return 2;
     return cls;
 }
-// split: a CTA per sub-tile of four sequences instead of per tile
-static DftPlan make_plan(int n, size_t elem, bool fwd, bool split) {
+// split: a CTA per sub-tile of eight tubes instead of per tile; full: tiles for
+// several CTAs on every SM
+static DftPlan make_plan(int n, size_t elem, bool split, bool full) {
     DftPlan P;
     P.n = n;
     P.split = split;
+    P.full = full;
     int m = n;
     P.D = 1;
     for (int q = 17; q <= m; ++q)
@@ -285,33 +446,69 @@ static DftPlan make_plan(int n, size_t elem, bool fwd, bool split) {
             m /= q;
             P.D *= q;
         }
-    int cur[DFT_MAX_PASS], sum = 1 << 30;
-    P.np = DFT_MAX_PASS + 1;
-    best_radices(m, 0, 0, 0, cur, P.r, &P.np, &sum);
-    if (P.np == 0 && P.D == 1) {  // n = 1
-        P.np = 1;
-        P.r[0] = 1;
+    int cur[DFT_MAX_PASS];
+    if (P.D > 1 || n == 1) {
+        int sum = INT_MAX;
+        P.first = P.D;
+        P.np = DFT_MAX_PASS;
+        best_radices(m, 0, 0, 0, cur, P.r, &P.np, &sum);
+    } else {
+        // Fewest passes, then the least arithmetic, about W words times the radix of a complex pass and n / 3 times the
+        // real one (float32 radices above 10 take more registers: a tenth more).  A single pass of a wide radix counts as
+        // two: most lanes of a small tile would idle (n = 32 in float64, one pass of 32 and 8 x 4: 15.8 and 6.7 us for
+        // 32 x 32 tubes; n = 24 in float32, 256 x 256 tubes: 8.2 and 5.3 us).
+        int passes = INT_MAX;
+        double cost = 0.0;
+        for (int i = 0; DFT_FIRST[i] > 1; ++i) {
+            const int f = DFT_FIRST[i], rest = m / f;
+            if (m % f) continue;
+            int r[DFT_MAX_PASS], np = DFT_MAX_PASS, sum = INT_MAX;
+            best_radices(rest, 0, 0, 0, cur, r, &np, &sum);
+            const int total = np + 1 + (np == 0 && f >= 8 ? 1 : 0);
+            double c = (double)(f / 2 + 1) * rest * (np ? sum : 0) + n * f / 3.0;
+            if (elem == 4 && (f > 10 || (np && r[0] > 10)) && (n & (n - 1))) c *= 1.1;
+            if (total < passes || (total == passes && c < cost)) {
+                passes = total;
+                cost = c;
+                P.first = f;
+                P.np = np;
+                std::copy(r, r + np, P.r);
+            }
+        }
     }
+    P.M = n / P.first;
+    P.len = (P.first / 2 + 1) * P.M;
     // x / d = x ceil(2^20 / d) >> 20 for x <= 1024, d <= 1024
-    for (int i = 0, L = n; i < P.np; ++i) {
-        P.rr[i] = ((1u << 20) + P.r[i] - 1) / P.r[i];
+    auto inverse = [](int d) { return ((1u << 20) + d - 1) / d; };
+    P.ff = inverse(P.first);
+    P.fm = inverse(P.M);
+    for (int i = 0, L = P.M; i < P.np; ++i) {
+        P.rr[i] = inverse(P.r[i]);
         L /= P.r[i];
-        P.rm[i] = ((1u << 20) + L - 1) / L;
+        P.rm[i] = inverse(L);
     }
-    P.lns = split ? 2 : 4;
-    while (P.lns > 2 && dft_smem(P, elem, fwd) > 112 * 1024) --P.lns;
-    // a thread per item of the pass with the fewest items
-    const int items = (n / (P.np ? P.r[0] : 1)) << P.lns;
+    P.lns = split ? 3 : 5;
+    P.cls = dft_class(P);
+    while (P.lns > 3 && dft_smem(P, elem) > 112 * 1024) --P.lns;
+    P.cls = dft_class(P);
+    P.smem = dft_smem(P, elem);
+    // a thread per item of the first pass
+    const int items = P.M << P.lns;
     P.nt = std::min(DFT_MAX_THREADS, std::max(64, (items + 31) & ~31));
-    // The direct part: groups of kb pairs on sequences / 2 lanes each, about 12 kb + 4 instructions per entry.
-    // Up to about 370 points one round of some width does (17 .. 61 points on 64 or 128 threads, 331 on 256):
-    // the cheapest of those, counting no fewer than three warps (fewer leave the SM waiting).  Beyond, 256 threads
+    // where tiles fill the SMs, about 24 words a thread: fewer threads keep more tiles (and loads) in flight (n = 128,
+    // 256 x 256 tubes, 256 and 128 threads: 18.0 and 14.4 us; with 200 tiles in all 4.1 and 4.3 us)
+    const int want = (P.len << P.lns) / 24;
+    if (full) P.nt = std::min(P.nt, want <= 64 ? 64 : (want <= 144 ? 128 : DFT_MAX_THREADS));
+    // The direct part: M columns of groups of kb pairs on a quarter as many lanes as tubes, about 12 kb + 4 instructions
+    // per entry.  Up to about 370 points one round of some width does (17 .. 61 points on 64 or 128 threads, 331 on
+    // 256): the cheapest of those, counting no fewer than three warps (fewer leave the SM waiting).  Beyond, 256 threads
     // and the fewest rounds, about kb + 1/2 units of time each.
+    P.kb = 2;
     if (P.D > 1) {
         int cost1 = INT_MAX, cost2 = INT_MAX, nt1 = 0, kb1 = 0, kb2 = 4;
         for (int nt = DFT_MAX_THREADS; nt >= 64; nt /= 2)
             for (int kb : {2, 3, 4, 6}) {
-                const int slots = nt >> (P.lns - 1), groups = n / P.D * ((P.D / 2 + kb) / kb);
+                const int slots = nt >> (P.lns - 2), groups = P.M * ((P.D / 2 + kb) / kb);
                 const int rounds = (groups + slots - 1) / slots;
                 const int c1 = std::max(nt, 96) * (12 * kb + 4), c2 = rounds * (2 * kb + 1);
                 if (rounds == 1 && c1 < cost1) {
@@ -326,33 +523,28 @@ static DftPlan make_plan(int n, size_t elem, bool fwd, bool split) {
             }
         P.nt = nt1 ? nt1 : DFT_MAX_THREADS;
         P.kb = nt1 ? kb1 : kb2;
-    } else {
-        P.kb = 0;
     }
-    P.smem = dft_smem(P, elem, fwd);
-    P.cls = dft_class(P);
     return P;
 }
 
 // The plans of the last lengths that a thread used (the search takes about a
 // microsecond, which a small transform would notice).
-static const DftPlan& dft_plan(int n, size_t elem, bool fwd, bool split) {
+static const DftPlan& dft_plan(int n, size_t elem, bool split, bool full) {
     struct Slot {
         DftPlan P;
         size_t elem = 0;
-        bool fwd = false;
     };
     thread_local Slot slots[16];
-    Slot& s = slots[((n * 4) ^ (elem == 4 ? 2 : 0) ^ (fwd ? 1 : 0)) & 15];
-    if (s.elem != elem || s.fwd != fwd || s.P.n != n || s.P.split != split) {
-        s.P = make_plan(n, elem, fwd, split);
+    Slot& s = slots[((n * 2) ^ (elem == 4 ? 1 : 0)) & 15];
+    if (s.elem != elem || s.P.n != n || s.P.split != split || s.P.full != full) {
+        s.P = make_plan(n, elem, split, full);
         s.elem = elem;
-        s.fwd = fwd;
     }
     return s.P;
 }
 
-constexpr int DFT_CTAS[4] = {4, 4, 3, 2};  // CTAs per SM that the registers of each class allow (float32)
+// CTAs per SM that the registers of each class allow (float32)
+constexpr int DFT_CTAS[DFT_CLASSES] = {4, 4, 3, 2, 2};
 
 // ---- kernels ----------------------------------------------------------------------
 template <typename T>
@@ -368,41 +560,45 @@ __device__ __forceinline__ long tube_off(long t, int cols, long ld) {
     return r * ld + (t - r * cols);
 }
 
-// n roots exp(-2 pi i m / n), and the digit reversal of the passes: table[pos]
-// = frequency index of shared position pos (inverse) or table[s] = position
-// of frequency s (forward).  Position digits (most significant first) are k_1
-// (weight n / r_1), k_2 (n / (r_1 r_2)), ..., the last one, of the direct part,
-// of weight 1; the frequency is k_1 + r_1 (k_2 + r_2 (k_3 + ...)).
-template <typename T>
-__device__ __forceinline__ void fill_tables(const DftPlan& P, cplx<T>* tw, unsigned short* table, bool by_pos) {
-    const int n = P.n;
+// Digits of x < M in the mixed radix r_0, r_1, .., lowest first, read in the other
+// direction (weights M / r_0, M / (r_0 r_1), ..): the position in a block of its
+// frequency x after the passes.
+__device__ __forceinline__ int dft_reverse(const DftPlan& P, int x) {
+    int pos = 0, w = P.M;
+    for (int i = 0; i < P.np; ++i) {
+        const int q = (int)((x * P.rr[i]) >> 20);
+        w = (int)((w * P.rr[i]) >> 20);
+        pos += (x - q * P.r[i]) * w;
+        x = q;
+    }
+    return pos;
+}
+
+// n roots exp(-2 pi i m / n), and what the passes do to the order:
+//   forward: table[position] = its frequency,
+//   inverse: table[position in a block] = time index in the block.
+template <typename T, bool FWD>
+__device__ __forceinline__ void fill_tables(const DftPlan& P, cplx<T>* tw, unsigned short* table) {
+    const int n = P.n, M = P.M;
     const T step = (T)2 / (T)n;
     const bool pow2 = (n & (n - 1)) == 0;  // 2 m / n without a division then
     for (int m = threadIdx.x; m < n; m += blockDim.x) {
         T s, c;
         sincospi_t<T>(pow2 ? (T)m * step : (T)(2 * m) / (T)n, &s, &c);
         tw[m] = mk<T>(c, -s);
-        int rest = m, pos = 0, w = n;
-        for (int i = 0; i < P.np; ++i) {  // m as a frequency: its digits, lowest first
-            const int r = P.r[i], q = (int)((rest * P.rr[i]) >> 20);
-            w = (int)((w * P.rr[i]) >> 20);
-            pos += (rest - q * r) * w;
-            rest = q;
-        }
-        pos += rest;
-        if (by_pos) table[pos] = (unsigned short)m;
-        else table[m] = (unsigned short)pos;
+        const int k2 = (int)((m * P.ff) >> 20), k1 = m - k2 * P.first;
+        if (FWD && 2 * k1 <= P.first) table[k1 * M + dft_reverse(P, k2)] = (unsigned short)m;
+        if (!FWD && m < M) table[dft_reverse(P, m)] = (unsigned short)m;
     }
 }
 
-// One pass over shared memory: blocks of length L, radix R, M = L / R.
-// LAST: M = 1, no twiddles.  MR = ceil(2^20 / M) divides item numbers by M.
-template <typename T, int R, bool LAST>
-__device__ __forceinline__ void pass_smem(cplx<T>* z, const cplx<T>* tw, int n, int L, int tstep, unsigned MR, int lns) {
-    const int p = threadIdx.x & ((1 << lns) - 1), ust = blockDim.x >> lns, items = n / R;
-    const int M = LAST ? 1 : L / R;
+// One pass over shared memory (len words per tube): blocks of length L, radix R,
+// M = L / R.  MR = ceil(2^20 / M) divides item numbers by M.
+template <typename T, int R>
+__device__ __forceinline__ void pass_smem(cplx<T>* z, const cplx<T>* tw, int len, int L, int tstep, unsigned MR, int lns) {
+    const int p = threadIdx.x & ((1 << lns) - 1), ust = blockDim.x >> lns, items = len / R, M = L / R;
     for (int u = threadIdx.x >> lns; u < items; u += ust) {
-        const int b = LAST ? u : (int)((u * MR) >> 20), j = LAST ? 0 : u - b * M;
+        const int b = (int)((u * MR) >> 20), j = u - b * M;
         cplx<T>* zp = z + ((size_t)(b * L + j) << lns) + p;
         cplx<T> v[R];
 #pragma unroll
@@ -410,7 +606,7 @@ __device__ __forceinline__ void pass_smem(cplx<T>* z, const cplx<T>* tw, int n, 
         RDft<T, R>::run(v);
         zp[0] = v[0];
 #pragma unroll
-        for (int k = 1; k < R; ++k) zp[(k * M) << lns] = LAST ? v[k] : cmul(v[k], tw[j * k * tstep]);
+        for (int k = 1; k < R; ++k) zp[(k * M) << lns] = M == 1 ? v[k] : cmul(v[k], tw[j * k * tstep]);
     }
 }
 
@@ -457,109 +653,185 @@ __device__ __forceinline__ void pass_smem(cplx<T>* z, const cplx<T>* tw, int n, 
         }                                                    \
     }
 
-// First forward pass: rows j, j + M, ... of the real tubes, packed.
+// the first radix
+#define DFT_SWITCH_FIRST(r, GO)                              \
+    if constexpr (CLS >= 2) {                                \
+        switch (r) {                                         \
+            case 14: GO(14); break;                          \
+            case 18: GO(18); break;                          \
+            case 20: GO(20); break;                          \
+            case 24: GO(24); break;                          \
+            case 32: GO(32); break;                          \
+            default: DFT_SWITCH(r, GO)                       \
+        }                                                    \
+    } else {                                                 \
+        DFT_SWITCH(r, GO)                                    \
+    }
+
+// Items of a first pass whose R entries a thread loads before it uses any.
+constexpr int dft_batch(int R) { return R >= 12 ? 1 : (R >= 6 ? 2 : (R > 1 ? 4 : 8)); }
+
+// First forward pass: rows j, j + M, .. of a tube (M = n / R); blocks k <= R / 2 of
+// length M.
 template <typename T, int R>
-__device__ __forceinline__ void pass_load(cplx<T>* z, const cplx<T>* tw, int n, int lns, const T* xa, const T* xb,
-                                          bool la, bool lb, bool vec, long ss, T& acc) {
+__device__ __forceinline__ void pass_load(cplx<T>* z, const cplx<T>* tw, int n, int lns, const T* x, bool live, long ss,
+                                          T& acc) {
+    constexpr int U = dft_batch(R);
     const int p = threadIdx.x & ((1 << lns) - 1), M = n / R, ust = blockDim.x >> lns;
-    for (int j = threadIdx.x >> lns; j < M; j += ust) {
-        cplx<T> v[R];
-        if (vec) {
+    for (int j0 = threadIdx.x >> lns; j0 < M; j0 += U * ust) {
+        T a[U][R];
 #pragma unroll
-            for (int q = 0; q < R; ++q)
-                v[q] = la ? __ldcs((const cplx<T>*)(xa + (long)(j + q * M) * ss)) : mk<T>(0, 0);
-        } else {
+        for (int u = 0; u < U; ++u)
 #pragma unroll
             for (int q = 0; q < R; ++q) {
-                const long off = (long)(j + q * M) * ss;
-                v[q] = mk<T>(la ? __ldcs(xa + off) : (T)0, lb ? __ldcs(xb + off) : (T)0);
+                const int j = j0 + u * ust;
+                a[u][q] = live && j < M ? __ldcs(x + (long)(j + q * M) * ss) : (T)0;
             }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int j = j0 + u * ust;
+            if (j >= M) break;
+            cplx<T> v[R / 2 + 1];
+#pragma unroll
+            for (int q = 0; q < R; ++q) acc = fma(a[u][q], a[u][q], acc);
+            RealDft<T, R>::forward(a[u], v);
+            cplx<T>* zp = z + ((size_t)j << lns) + p;
+            zp[0] = v[0];
+#pragma unroll
+            for (int k = 1; k <= R / 2; ++k) zp[(k * M) << lns] = cmul(v[k], tw[j * k]);
         }
-#pragma unroll
-        for (int q = 0; q < R; ++q) acc = fma(v[q].x, v[q].x, fma(v[q].y, v[q].y, acc));
-        RDft<T, R>::run(v);
-        cplx<T>* zp = z + ((size_t)j << lns) + p;
-        zp[0] = v[0];
-#pragma unroll
-        for (int k = 1; k < R; ++k) zp[(k * M) << lns] = cmul(v[k], tw[j * k]);
     }
 }
 
-// Last inverse pass: block u's outputs are the rows low + (n / R) k of the
-// tubes (low = the frequency of the block's first position), swapped back and
-// scaled.
+// Frequency f of a tube (dst: its column of the spectrum), or, above n / 2, its
+// conjugate to n - f; blocks 0 and first / 2 hold n - f themselves (twice: not one of
+// those).
+template <typename T>
+__device__ __forceinline__ void put_hat(cplx<T>* dst, long tubes, int n, int f, bool twice, cplx<T> v) {
+    if (f == 0 || 2 * f == n) v.y = 0;
+    if (2 * f <= n) dst[(long)f * tubes] = v;
+    else if (twice) dst[(long)(n - f) * tubes] = cconj(v);
+}
+
+// Last forward pass: block u's frequencies low + (n / R) k to the spectrum.
 template <typename T, int R>
-__device__ __forceinline__ void pass_store(const cplx<T>* z, const unsigned short* freq, int n, int lns, T* xa, T* xb,
-                                           bool la, bool lb, bool vec, long ss) {
-    const int p = threadIdx.x & ((1 << lns) - 1), M = n / R, ust = blockDim.x >> lns;
-    const T inv = (T)1 / (T)n;
-    for (int u = threadIdx.x >> lns; u < M; u += ust) {
+__device__ __forceinline__ void pass_out(const cplx<T>* z, const unsigned short* freq, int n, int len, int lns, int lo,
+                                         int hi, cplx<T>* dst, bool live, long tubes) {
+    const int p = threadIdx.x & ((1 << lns) - 1), ust = blockDim.x >> lns, items = len / R, M = n / R;
+    for (int u = threadIdx.x >> lns; u < items; u += ust) {
         const cplx<T>* zp = z + ((size_t)(u * R) << lns) + p;
         cplx<T> v[R];
 #pragma unroll
         for (int q = 0; q < R; ++q) v[q] = zp[q << lns];
         RDft<T, R>::run(v);
-        const long row = freq[u * R];
+        const int low = freq[u * R];  // the last digit is 0
+        const bool twice = u * R >= lo && u * R < hi;
+        if (live)
 #pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const long off = (row + (long)k * M) * ss;
-            if (vec) {
-                if (la) *(cplx<T>*)(xa + off) = mk<T>(v[k].y * inv, v[k].x * inv);
-            } else {
-                if (la) xa[off] = v[k].y * inv;
-                if (lb) xb[off] = v[k].x * inv;
+            for (int k = 0; k < R; ++k) put_hat<T>(dst, tubes, n, low + k * M, twice, v[k]);
+    }
+}
+
+// First inverse pass over the blocks k1 <= r0 / 2 of length M = n / r0: word k2 of block
+// k1 is frequency f = k1 + r0 k2, the conjugate of n - f above n / 2 (blocks 0 and r0 / 2
+// read theirs twice), re and im swapped.  R = 1: a copy.
+template <typename T, int R, typename Note>
+__device__ __forceinline__ void pass_load_hat(cplx<T>* z, const cplx<T>* tw, int n, int r0, int M, int len, unsigned MR,
+                                              int lns, const cplx<T>* src, bool live, long tubes, Note note) {
+    const int p = threadIdx.x & ((1 << lns) - 1), ust = blockDim.x >> lns, items = len / R, Q = M / R;
+    constexpr int U = dft_batch(R);
+    for (int u0 = threadIdx.x >> lns; u0 < items; u0 += U * ust) {
+        cplx<T> v[U][R];
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            const int u = u0 + i * ust, k1 = (int)((u * MR) >> 20), j = u - k1 * Q;
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                const int f = k1 + r0 * (j + q * Q);
+                v[i][q] = live && u < items ? src[(long)(2 * f <= n ? f : n - f) * tubes] : mk<T>(0, 0);
             }
+        }
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            const int u = u0 + i * ust, k1 = (int)((u * MR) >> 20), j = u - k1 * Q;
+            if (u >= items) break;
+#pragma unroll
+            for (int q = 0; q < R; ++q) {
+                const int f = k1 + r0 * (j + q * Q);
+                if (f == 0 || 2 * f == n) v[i][q].y = 0;  // the imaginary parts of slices 0 and n / 2 are ignored
+                note(v[i][q]);
+                v[i][q] = mk<T>(2 * f <= n ? v[i][q].y : -v[i][q].y, v[i][q].x);
+            }
+            RDft<T, R>::run(v[i]);
+            cplx<T>* zp = z + ((size_t)(k1 * M + j) << lns) + p;
+            zp[0] = v[i][0];
+#pragma unroll
+            for (int k = 1; k < R; ++k) zp[(k * Q) << lns] = Q == 1 ? v[i][k] : cmul(v[i][k], tw[j * k * r0]);
         }
     }
 }
 
-// The direct part: DFTs of the n / D contiguous blocks of odd length D, whose
-// entries q and D - q first become e_q = x_q + x_{D-q} and o_q = x_q - x_{D-q}.
-// (direct_fold.)  A thread forms KB pairs (k, D - k) of two neighbouring sequences, so each
-// twiddle and each (e, o) read serves several products (about two thirds of
-// the issue slots are multiply-adds).  put(block, k, sequence, value).
-template <typename T>
-__device__ __forceinline__ void direct_fold(cplx<T>* z, int n, int D, int lns) {
-    typedef cplx<T> V;
-    const int H = D / 2, nb = n / D, ns = 1 << lns;
-    for (int e = threadIdx.x; e < nb * H * ns; e += blockDim.x) {
-        const int p = e & (ns - 1), bq = e >> lns, b = bq / H, q = bq - b * H + 1;
-        V* x = z + ((size_t)(b * D + q) << lns) + p;
-        V* y = z + ((size_t)(b * D + D - q) << lns) + p;
-        const V u = *x, v = *y;
-        *x = cadd(u, v);
-        *y = csub(u, v);
+// Last inverse pass: the blocks' entries at one position, times exp(2 pi i j k / n) (j
+// its time index), to the rows j + M q of the tube.
+template <typename T, int R>
+__device__ __forceinline__ void pass_store(const cplx<T>* z, const cplx<T>* tw, const unsigned short* time, int n, int lns,
+                                           T* x, bool live, long ss, T inv) {
+    const int p = threadIdx.x & ((1 << lns) - 1), M = n / R, ust = blockDim.x >> lns;
+    for (int u = threadIdx.x >> lns; u < M; u += ust) {
+        const cplx<T>* zp = z + ((size_t)u << lns) + p;
+        const int j = time[u];
+        T o[R];
+        cplx<T> a[R / 2 + 1];
+        a[0] = mk<T>(zp[0].y * inv, 0);
+#pragma unroll
+        for (int k = 1; k <= R / 2; ++k) {
+            const cplx<T> v = zp[(k * M) << lns], w = tw[j * k];  // (im, re); cos - i sin
+            const T g = 2 * k == R ? inv : 2 * inv;
+            a[k] = mk<T>((v.y * w.x + v.x * w.y) * g, (v.x * w.x - v.y * w.y) * g);
+        }
+        RealDft<T, R>::inverse(a, o);
+        if (live)
+#pragma unroll
+            for (int q = 0; q < R; ++q) x[(long)(j + q * M) * ss] = o[q];
     }
-    __syncthreads();
 }
+
+// The direct part: real DFTs of odd length D over the rows j, j + M, .. of each column
+// j < M, on pairs of tubes (a word holds an entry of tube 2 p and one of tube 2 p + 1, which
+// never meet: every sum is formed part by part).  The rows j + M q and j + M (D - q)
+// hold e_q and o_q; a thread forms KB pairs (k, D - k) of two neighbouring pairs of
+// tubes, so each twiddle and each (e, o) read serves several products (about two thirds of
+// the issue slots are multiply-adds).  put(j, k, pair, A, B) takes A = x_0 + sum e_q
+// cos(2 pi q k / D) and B = -sum o_q sin(2 pi q k / D).
 template <typename T, int KB, typename Put>
-__device__ __forceinline__ void direct_part(const cplx<T>* z, const cplx<T>* tw, int n, int D, int lns, Put put) {
+__device__ __forceinline__ void direct_sums(const cplx<T>* z, const cplx<T>* tw, int M, int D, int lnp, Put put) {
     typedef cplx<T> V;
-    const int H = D / 2, nb = n / D, ts = n / D;  // twiddles exp(-2 pi i m / D) = tw[m n / D]
-    const int lhs = lns - 1, sp = threadIdx.x & ((1 << lhs) - 1), gst = blockDim.x >> lhs;
+    const int H = D / 2;  // twiddles exp(-2 pi i m / D) = tw[m M]
+    const int lhs = lnp - 1, sp = threadIdx.x & ((1 << lhs) - 1), gst = blockDim.x >> lhs;
     const int ng = (H + KB) / KB;  // groups of KB values of k in 0 .. H
-    for (int it = threadIdx.x >> lhs; it < nb * ng; it += gst) {
-        const int b = it / ng, k0 = (it - b * ng) * KB;
-        const V* zb = z + ((size_t)(b * D) << lns) + 2 * sp;
+    const size_t row = (size_t)M << lnp;
+    for (int it = threadIdx.x >> lhs; it < M * ng; it += gst) {
+        const int j = it / ng, k0 = (it - j * ng) * KB;
+        const V* zj = z + ((size_t)j << lnp) + 2 * sp;
         V A[KB][2], B[KB][2];
         int idx[KB], kk[KB];
 #pragma unroll
         for (int t = 0; t < KB; ++t) {
             kk[t] = min(k0 + t, H);
             idx[t] = 0;
-            A[t][0] = zb[0];
-            A[t][1] = zb[1];
+            A[t][0] = zj[0];
+            A[t][1] = zj[1];
             B[t][0] = B[t][1] = mk<T>(0, 0);
         }
+        const V *ze = zj + row, *zo = zj + (D - 1) * row;
 #pragma unroll 2
-        for (int q = 1; q <= H; ++q) {
-            const V e0 = zb[(size_t)q << lns], e1 = zb[((size_t)q << lns) + 1];
-            const V o0 = zb[(size_t)(D - q) << lns], o1 = zb[((size_t)(D - q) << lns) + 1];
+        for (int q = 1; q <= H; ++q, ze += row, zo -= row) {
+            const V e0 = ze[0], e1 = ze[1], o0 = zo[0], o1 = zo[1];
 #pragma unroll
             for (int t = 0; t < KB; ++t) {
                 const unsigned nx = (unsigned)(idx[t] + kk[t]);
                 idx[t] = (int)min(nx, nx - (unsigned)D);  // (q k) mod D
-                const V w = tw[idx[t] * ts];
+                const V w = tw[idx[t] * M];
                 A[t][0].x = fma(e0.x, w.x, A[t][0].x);
                 A[t][0].y = fma(e0.y, w.x, A[t][0].y);
                 A[t][1].x = fma(e1.x, w.x, A[t][1].x);
@@ -570,91 +842,94 @@ __device__ __forceinline__ void direct_part(const cplx<T>* z, const cplx<T>* tw,
                 B[t][1].y = fma(o1.y, w.y, B[t][1].y);
             }
         }
-        // tw holds cos - i sin: X_k, X_{D-k} = A +- i B
 #pragma unroll
         for (int t = 0; t < KB; ++t) {
             const int k = k0 + t;
             if (k > H) break;
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const V a = A[t][c], bb = B[t][c];
-                put(b, k, 2 * sp + c, mk<T>(a.x - bb.y, a.y + bb.x));
-                if (k > 0) put(b, D - k, 2 * sp + c, mk<T>(a.x + bb.y, a.y - bb.x));
-            }
+            for (int c = 0; c < 2; ++c) put(j, k, 2 * sp + c, A[t][c], B[t][c]);
         }
     }
 }
-
-// Entries of two neighbouring tubes in one row of the spectrum.
-template <typename T>
-__device__ __forceinline__ void store_pair(cplx<T>* dst, cplx<T> a, cplx<T> b, bool lb, bool vec) {
-    if (sizeof(T) == 4 && vec) {
-        *(float4*)dst = make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
-    } else {
-        dst[0] = a;
-        if (lb) dst[1] = b;
-    }
+template <typename T, typename Put>
+__device__ __forceinline__ void direct_part(const DftPlan& P, const cplx<T>* z, const cplx<T>* tw, int lnp, Put put) {
+    if (P.kb == 2) direct_sums<T, 2>(z, tw, P.M, P.D, lnp, put);
+    else if (P.kb == 3) direct_sums<T, 3>(z, tw, P.M, P.D, lnp, put);
+    else if (P.kb == 4) direct_sums<T, 4>(z, tw, P.M, P.D, lnp, put);
+    else direct_sums<T, 6>(z, tw, P.M, P.D, lnp, put);
 }
+
+// Rows of a pair of tubes to shared memory as e and o (rows j of q = 0 as they are).
 template <typename T>
-__device__ __forceinline__ void load_pair(const cplx<T>* src, cplx<T>& a, cplx<T>& b, bool lb, bool vec) {
-    if (sizeof(T) == 4 && vec) {
-        const float4 v = *(const float4*)src;
-        a = mk<T>((T)v.x, (T)v.y);
-        b = mk<T>((T)v.z, (T)v.w);
-    } else {
-        a = src[0];
-        if (lb) b = src[1];
+__device__ __forceinline__ void direct_load(cplx<T>* z, int M, int D, unsigned FM, int lnp, const T* x, const T* y, bool la, bool lb,
+                                            long ss, T& acc) {
+    typedef cplx<T> V;
+    constexpr int U = 4;  // row pairs in flight per thread
+    const int p = threadIdx.x & ((1 << lnp) - 1), ust = blockDim.x >> lnp, items = M * (D / 2 + 1);
+    for (int u0 = threadIdx.x >> lnp; u0 < items; u0 += U * ust) {
+        V a[U], b[U];
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            const int u = u0 + i * ust, q = (int)((u * FM) >> 20), r = u - q * M + M * (q ? D - q : 0);  // rows u = j + M q and j + M (D - q)
+            const bool ok = u < items;
+            a[i] = mk<T>(ok && la ? __ldcs(x + (long)u * ss) : (T)0, ok && lb ? __ldcs(y + (long)u * ss) : (T)0);
+            b[i] = mk<T>(ok && la && q ? __ldcs(x + (long)r * ss) : (T)0, ok && lb && q ? __ldcs(y + (long)r * ss) : (T)0);
+        }
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            const int u = u0 + i * ust, q = (int)((u * FM) >> 20), r = u - q * M + M * (q ? D - q : 0);
+            if (u >= items) break;
+            acc = fma(a[i].x, a[i].x, fma(a[i].y, a[i].y, acc));
+            acc = fma(b[i].x, b[i].x, fma(b[i].y, b[i].y, acc));
+            z[((size_t)u << lnp) + p] = cadd(a[i], b[i]);
+            if (q) z[((size_t)r << lnp) + p] = csub(a[i], b[i]);
+        }
     }
 }
 
 template <typename T, int CLS>
 __global__ void __launch_bounds__(DFT_MAX_THREADS, sizeof(T) == 4 ? DFT_CTAS[CLS] : 1)
 k_rdft(const __grid_constant__ DftPlan P, const T* __restrict__ X, cplx<T>* __restrict__ Xh, long tubes, int cols,
-       long ld, long ss, int vin, int vout, double* sumsq, const int* skip) {
+       long ld, long ss, double* sumsq, const int* skip) {
     if (skip && *skip) return;
     typedef cplx<T> V;
+    constexpr bool ANY = CLS >= DFT_GENERAL;  // any sub-tile
     extern __shared__ __align__(16) unsigned char smraw[];
-    const int n = P.n, lns = CLS == 3 ? P.lns : 4, ns = 1 << lns, h = n / 2 + 1;
-    V* z = (V*)smraw;
-    V* z2 = CLS == 3 && P.D > 1 ? z + ((size_t)n << lns) : z;
-    V* tw = z2 + ((size_t)n << lns);
-    unsigned short* pos = (unsigned short*)(tw + n);
-    fill_tables<T>(P, tw, pos, false);
+    const int n = P.n, M = P.M, len = P.len, lns = ANY ? P.lns : 5, nts = 1 << lns, h = n / 2 + 1;
+    V* zp = (V*)smraw;  // DIRECT: the pairs of tubes
+    V* z = CLS == DFT_DIRECT ? zp + ((size_t)n << (lns - 1)) : zp;
+    V* tw = CLS == DFT_DIRECT && M == 1 ? z : z + ((size_t)len << lns);
+    unsigned short* freq = (unsigned short*)(tw + n);
+    fill_tables<T, true>(P, tw, freq);
     __syncthreads();
     T total = 0;
     // all sub-tiles of tile blockIdx.x, or (split) one
-    const int nsub = DFT_SEQ >> lns;
-    const long tile = CLS == 3 && P.split ? blockIdx.x / nsub : blockIdx.x;
-    const int sub0 = CLS == 3 && P.split ? (blockIdx.x % nsub) << lns : 0;
-    const int sub1 = CLS == 3 && P.split ? sub0 + ns : DFT_SEQ;
-    for (int sub = sub0; sub < sub1; sub += ns) {
-        const long t0 = tile * DFT_TILE + 2 * (sub + (threadIdx.x & (ns - 1)));
-        const bool la = t0 < tubes, lb = t0 + 1 < tubes;
-        const T* xa = X + (la ? tube_off(t0, cols, ld) : 0);
-        const T* xb = X + (lb ? tube_off(t0 + 1, cols, ld) : 0);
+    const int nsub = DFT_TILE >> lns;
+    const long tile = ANY && P.split ? blockIdx.x / nsub : blockIdx.x;
+    const int sub0 = ANY && P.split ? (blockIdx.x % nsub) << lns : 0;
+    const int sub1 = ANY && P.split ? sub0 + nts : DFT_TILE;
+    for (int sub = sub0; sub < sub1; sub += nts) {
+        const long f0 = tile * DFT_TILE + sub, t0 = f0 + (threadIdx.x & (nts - 1));
+        const bool live = t0 < tubes;
         T acc = 0;
-        int L = n, tstep = 1;
-        if (CLS < 3 || P.np > 0) {
-#define GO(R) pass_load<T, R>(z, tw, n, lns, xa, xb, la, lb, vin, ss, acc)
-            DFT_SWITCH(P.r[0], GO)
+        if constexpr (CLS == DFT_DIRECT) {
+            const long t = f0 + 2 * (threadIdx.x & ((nts >> 1) - 1));
+            const bool la = t < tubes, lb = t + 1 < tubes;
+            direct_load<T>(zp, M, P.D, P.fm, lns - 1, X + (la ? tube_off(t, cols, ld) : 0), X + (lb ? tube_off(t + 1, cols, ld) : 0), la,
+                           lb, ss, acc);
+        } else {
+            const T* x = X + (live ? tube_off(t0, cols, ld) : 0);
+#define GO(R) pass_load<T, R>(z, tw, n, lns, x, live, ss, acc)
+            DFT_SWITCH_FIRST(P.first, GO)
 #undef GO
-            tstep = P.r[0];
-            L = (int)((n * P.rr[0]) >> 20);
-        } else {  // n is all direct part: a plain copy
-            for (int k = threadIdx.x >> lns; k < n; k += blockDim.x >> lns) {
-                const V v = mk<T>(la ? __ldcs(xa + (long)k * ss) : (T)0, lb ? __ldcs(xb + (long)k * ss) : (T)0);
-                acc = fma(v.x, v.x, fma(v.y, v.y, acc));
-                z[((size_t)k << lns) + (threadIdx.x & (ns - 1))] = v;
-            }
         }
         const bool finite = !__syncthreads_or(!isfinite(acc));
         total += acc;
         if (!finite) {
             // the defining sum, tube by tube
-            const long f0 = tile * DFT_TILE + 2 * sub;
-            for (int e = threadIdx.x; e < h * 2 * ns; e += blockDim.x) {
-                const int s = e / (2 * ns), tt = e - s * 2 * ns;
-                const long t = f0 + tt;
+            for (int e = threadIdx.x; e < h * nts; e += blockDim.x) {
+                const int s = e >> lns;
+                const long t = f0 + (e & (nts - 1));
                 if (t >= tubes) continue;
                 const T* x = X + tube_off(t, cols, ld);
                 V o = mk<T>(0, 0);
@@ -671,45 +946,42 @@ k_rdft(const __grid_constant__ DftPlan P, const T* __restrict__ X, cplx<T>* __re
             __syncthreads();
             continue;
         }
-        for (int i = 1; i < P.np; ++i) {
-            if (L == P.r[i]) {
-#define GO(R) pass_smem<T, R, true>(z, tw, n, L, tstep, 0u, lns)
-                DFT_SWITCH(P.r[i], GO)
+        if constexpr (CLS == DFT_DIRECT) {
+            direct_part<T>(P, zp, tw, lns - 1, [&](int j, int k, int q, V a, V b) {
+                const V u = mk<T>(a.x, b.x), v = mk<T>(a.y, b.y);  // the two tubes
+                if (M == 1) {
+                    const long t = f0 + 2 * q;
+                    V* dst = Xh + (long)k * tubes + t;
+                    if (t < tubes) dst[0] = u;
+                    if (t + 1 < tubes) dst[1] = v;
+                } else {
+                    const V w = tw[j * k];
+                    V* dst = z + ((size_t)(k * M + j) << lns) + 2 * q;
+                    dst[0] = cmul(u, w);
+                    dst[1] = cmul(v, w);
+                }
+            });
+            if (M > 1) __syncthreads();
+        }
+        int L = M, tstep = P.first;
+        for (int i = 0; i < P.np - 1; ++i) {
+#define GO(R) pass_smem<T, R>(z, tw, len, L, tstep, P.rm[i], lns)
+            DFT_SWITCH(P.r[i], GO)
 #undef GO
-            } else {
-#define GO(R) pass_smem<T, R, false>(z, tw, n, L, tstep, P.rm[i], lns)
-                DFT_SWITCH(P.r[i], GO)
-#undef GO
-            }
             tstep *= P.r[i];
             L = (int)((L * P.rr[i]) >> 20);
             __syncthreads();
         }
-        if (CLS == 3 && P.D > 1) {
-            direct_fold<T>(z, n, P.D, lns);
-            auto put = [&](int b, int k, int q, V v) { z2[((size_t)(b * P.D + k) << lns) + q] = v; };
-            if (P.kb == 2) direct_part<T, 2>(z, tw, n, P.D, lns, put);
-            else if (P.kb == 3) direct_part<T, 3>(z, tw, n, P.D, lns, put);
-            else if (P.kb == 4) direct_part<T, 4>(z, tw, n, P.D, lns, put);
-            else direct_part<T, 6>(z, tw, n, P.D, lns, put);
-            __syncthreads();
+        const int lo = M, hi = (P.first + 1) / 2 * M;  // words of frequencies and of conjugates
+        V* dst = Xh + t0;
+        if (P.np > 0) {
+#define GO(R) pass_out<T, R>(z, freq, n, len, lns, lo, hi, dst, live, tubes)
+            DFT_SWITCH(P.r[P.np - 1], GO)
+#undef GO
+        } else if (CLS != DFT_DIRECT) {
+            pass_out<T, 1>(z, freq, n, len, lns, lo, hi, dst, live, tubes);
         }
-        // the two tubes of a sequence: (Z_s + conj Z_{n-s}) / 2 and (Z_s - conj Z_{n-s}) / 2i
-        const int p = threadIdx.x & (ns - 1);
-        if (la) {
-            const int hp = (n + 1) / 2, sst = blockDim.x >> lns;
-            V* dst = Xh + t0;
-            auto out = [&](int s, int m) {  // m: n - s, or s when they are the same slice
-                const V zs = z2[((size_t)pos[s] << lns) + p], zc = z2[((size_t)pos[m] << lns) + p];
-                const V a = mk<T>((zs.x + zc.x) * (T)0.5, (zs.y - zc.y) * (T)0.5);
-                const V b = mk<T>((zs.y + zc.y) * (T)0.5, (zc.x - zs.x) * (T)0.5);
-                store_pair<T>(dst + (long)s * tubes, a, b, lb, vout);
-            };
-#pragma unroll 2
-            for (int s = threadIdx.x >> lns; s < hp; s += sst) out(s, s ? n - s : 0);
-            if (2 * hp == n && (int)(threadIdx.x >> lns) == sst - 1) out(hp, hp);
-        }
-        if (ns < DFT_SEQ) __syncthreads();
+        if (nts < DFT_TILE) __syncthreads();
     }
     if (sumsq) store_partial<T>(total, sumsq);
 }
@@ -717,60 +989,56 @@ k_rdft(const __grid_constant__ DftPlan P, const T* __restrict__ X, cplx<T>* __re
 template <typename T, int CLS>
 __global__ void __launch_bounds__(DFT_MAX_THREADS, sizeof(T) == 4 ? DFT_CTAS[CLS] : 1)
 k_irdft(const __grid_constant__ DftPlan P, const cplx<T>* __restrict__ Xh, T* __restrict__ X, long tubes, int cols,
-        long ld, long ss, int vin, int vout, const int* skip) {
+        long ld, long ss, const int* skip) {
     if (skip && *skip) return;
     typedef cplx<T> V;
+    constexpr bool ANY = CLS >= DFT_GENERAL;
     extern __shared__ __align__(16) unsigned char smraw[];
-    const int n = P.n, lns = CLS == 3 ? P.lns : 4, ns = 1 << lns, h = n / 2 + 1;
-    V* z = (V*)smraw;
-    V* tw = z + ((size_t)n << lns);
-    unsigned short* freq = (unsigned short*)(tw + n);
-    fill_tables<T>(P, tw, freq, true);
-    const int nsub = DFT_SEQ >> lns;
-    const long tile = CLS == 3 && P.split ? blockIdx.x / nsub : blockIdx.x;
-    const int sub0 = CLS == 3 && P.split ? (blockIdx.x % nsub) << lns : 0;
-    const int sub1 = CLS == 3 && P.split ? sub0 + ns : DFT_SEQ;
-    for (int sub = sub0; sub < sub1; sub += ns) {
-        const int p = threadIdx.x & (ns - 1), sst = blockDim.x >> lns;
-        const long t0 = tile * DFT_TILE + 2 * (sub + p);
-        const bool la = t0 < tubes, lb = t0 + 1 < tubes;
-        T* xa = X + (la ? tube_off(t0, cols, ld) : 0);
-        T* xb = X + (lb ? tube_off(t0 + 1, cols, ld) : 0);
-        T bad = 0;  // stays 0 for finite data
-        constexpr int LB = sizeof(T) == 4 ? 8 : 4;  // pairs of spectrum entries in flight per thread
-        const int hp = (n + 1) / 2;  // slices 0 .. hp - 1, then slice n / 2 of an even n
-        auto put = [&](int s, V x, V y, bool self) {
-            if (self) x.y = y.y = 0;  // the imaginary parts of slices 0 and n / 2 are ignored
-            bad = fma(x.x, (T)0, fma(x.y, (T)0, fma(y.x, (T)0, fma(y.y, (T)0, bad))));
-            // Z_s = x + i y and Z_{n-s} = conj(x) + i conj(y), re and im swapped
-            z[((size_t)s << lns) + p] = mk<T>(x.y + y.x, x.x - y.y);
-            if (!self) z[((size_t)(n - s) << lns) + p] = mk<T>(y.x - x.y, x.x + y.y);
-        };
+    const int n = P.n, M = P.M, len = P.len, lns = ANY ? P.lns : 5, nts = 1 << lns, h = n / 2 + 1;
+    V* zp = (V*)smraw;
+    V* z = CLS == DFT_DIRECT ? zp + ((size_t)n << (lns - 1)) : zp;
+    V* tw = CLS == DFT_DIRECT && M == 1 ? z : z + ((size_t)len << lns);
+    unsigned short* time = (unsigned short*)(tw + n);
+    fill_tables<T, false>(P, tw, time);
+    __syncthreads();
+    const T inv = (T)1 / (T)n;
+    const int nsub = DFT_TILE >> lns;
+    const long tile = ANY && P.split ? blockIdx.x / nsub : blockIdx.x;
+    const int sub0 = ANY && P.split ? (blockIdx.x % nsub) << lns : 0;
+    const int sub1 = ANY && P.split ? sub0 + nts : DFT_TILE;
+    for (int sub = sub0; sub < sub1; sub += nts) {
+        const long f0 = tile * DFT_TILE + sub, t0 = f0 + (threadIdx.x & (nts - 1));
+        const bool live = t0 < tubes;
         const V* src = Xh + t0;
-        for (int s0 = threadIdx.x >> lns; s0 < hp; s0 += LB * sst) {
-            V a[LB], b[LB];
-#pragma unroll
-            for (int u = 0; u < LB; ++u) {
-                a[u] = b[u] = mk<T>(0, 0);
-                if (la && s0 + u * sst < hp) load_pair<T>(src + (long)(s0 + u * sst) * tubes, a[u], b[u], lb, vin);
+        T bad = 0;  // stays 0 for finite data
+        auto note = [&](V v) { bad = fma(v.x, (T)0, fma(v.y, (T)0, bad)); };
+        if (P.np > 0) {
+#define GO(R) pass_load_hat<T, R>(z, tw, n, P.first, M, len, P.rm[0], lns, src, live, tubes, note)
+            DFT_SWITCH(P.r[0], GO)
+#undef GO
+        } else if constexpr (CLS == DFT_DIRECT) {
+            // straight to the pairs of tubes: e = 2 Re X_s, o = 2 Im X_s
+            const int np = nts >> 1, p = threadIdx.x & (np - 1);
+            const long t = f0 + 2 * p;
+            for (int s = threadIdx.x >> (lns - 1); s < h; s += blockDim.x >> (lns - 1)) {
+                const V* x = Xh + (long)s * tubes + t;
+                V a = t < tubes ? x[0] : mk<T>(0, 0), b = t + 1 < tubes ? x[1] : mk<T>(0, 0);
+                if (s == 0) a.y = b.y = 0;  // the imaginary part of slice 0 is ignored
+                note(a);
+                note(b);
+                const T g = s ? (T)2 : (T)1;
+                zp[s * np + p] = mk<T>(g * a.x, g * b.x);
+                if (s) zp[(n - s) * np + p] = mk<T>(g * a.y, g * b.y);
             }
-#pragma unroll
-            for (int u = 0; u < LB; ++u)
-                if (s0 + u * sst < hp) put(s0 + u * sst, a[u], b[u], s0 + u * sst == 0);
-        }
-        if (2 * hp == n && (int)(threadIdx.x >> lns) == sst - 1) {
-            V a = mk<T>(0, 0), b = mk<T>(0, 0);
-            if (la) load_pair<T>(src + (long)hp * tubes, a, b, lb, vin);
-            put(hp, a, b, true);
+        } else {
+            pass_load_hat<T, 1>(z, tw, n, P.first, M, len, P.fm, lns, src, live, tubes, note);
         }
         const bool finite = !__syncthreads_or(bad != (T)0 || isnan(bad));
         if (!finite) {
             // the defining sum, tube by tube
-            const long f0 = tile * DFT_TILE + 2 * sub;
-            const T inv = (T)1 / (T)n;
-            for (int e = threadIdx.x; e < n * 2 * ns; e += blockDim.x) {
-                const int k = e / (2 * ns), tt = e - k * 2 * ns;
-                const long t = f0 + tt;
+            for (int e = threadIdx.x; e < n * nts; e += blockDim.x) {
+                const int k = e >> lns;
+                const long t = f0 + (e & (nts - 1));
                 if (t >= tubes) continue;
                 T acc = Xh[t].x;
                 int idx = k;
@@ -787,64 +1055,64 @@ k_irdft(const __grid_constant__ DftPlan P, const cplx<T>* __restrict__ Xh, T* __
             __syncthreads();
             continue;
         }
-        int L = n, tstep = 1;
-        const int last = P.D > 1 ? P.np : P.np - 1;
-        for (int i = 0; i < last; ++i) {
-            if (L == P.r[i]) {
-#define GO(R) pass_smem<T, R, true>(z, tw, n, L, tstep, 0u, lns)
+        int L = M, tstep = P.first;
+        for (int i = 0; i < P.np; ++i) {
+            if (i > 0) {
+#define GO(R) pass_smem<T, R>(z, tw, len, L, tstep, P.rm[i], lns)
                 DFT_SWITCH(P.r[i], GO)
 #undef GO
-            } else {
-#define GO(R) pass_smem<T, R, false>(z, tw, n, L, tstep, P.rm[i], lns)
-                DFT_SWITCH(P.r[i], GO)
-#undef GO
+                __syncthreads();
             }
             tstep *= P.r[i];
             L = (int)((L * P.rr[i]) >> 20);
-            __syncthreads();
         }
-        if (CLS == 3 && P.D > 1) {
-            const T inv = (T)1 / (T)n;
-            const int nb = n / P.D;
-            const long f0 = tile * DFT_TILE + 2 * sub;
-            direct_fold<T>(z, n, P.D, lns);
-            auto put = [&](int b, int k, int q, V v) {
-                const long t = f0 + 2 * q, off = (long)(freq[b * P.D] + nb * k) * ss;
-                if (t < tubes) X[tube_off(t, cols, ld) + off] = v.y * inv;
-                if (t + 1 < tubes) X[tube_off(t + 1, cols, ld) + off] = v.x * inv;
-            };
-            if (P.kb == 2) direct_part<T, 2>(z, tw, n, P.D, lns, put);
-            else if (P.kb == 3) direct_part<T, 3>(z, tw, n, P.D, lns, put);
-            else if (P.kb == 4) direct_part<T, 4>(z, tw, n, P.D, lns, put);
-            else direct_part<T, 6>(z, tw, n, P.D, lns, put);
+        if constexpr (CLS == DFT_DIRECT) {
+            if (M > 1) {
+                // the blocks' entries at a position, times exp(2 pi i j k / n): e = 2 Re, o = 2 Im at row j + M k of the pairs
+                T* zr = (T*)zp;
+                for (int e = threadIdx.x >> lns; e < len; e += blockDim.x >> lns) {
+                    const int k = (int)((e * P.fm) >> 20), j = time[e - k * M], t = threadIdx.x & (nts - 1);
+                    const V v = z[((size_t)e << lns) + t], w = tw[j * k];  // (im, re); cos - i sin
+                    const T g = k ? (T)2 : (T)1;
+                    zr[((size_t)(j + M * k) << lns) + t] = (v.y * w.x + v.x * w.y) * g;
+                    if (k) zr[((size_t)(j + M * (P.D - k)) << lns) + t] = (v.x * w.x - v.y * w.y) * g;
+                }
+                __syncthreads();
+            }
+            direct_part<T>(P, zp, tw, lns - 1, [&](int j, int k, int q, V a, V b) {
+                const long t = f0 + 2 * q, up = (long)(j + M * k) * ss, down = (long)(j + M * (P.D - k)) * ss;
+                if (t < tubes) {
+                    T* o = X + tube_off(t, cols, ld);
+                    o[up] = (a.x + b.x) * inv;
+                    if (k > 0) o[down] = (a.x - b.x) * inv;
+                }
+                if (t + 1 < tubes) {
+                    T* o = X + tube_off(t + 1, cols, ld);
+                    o[up] = (a.y + b.y) * inv;
+                    if (k > 0) o[down] = (a.y - b.y) * inv;
+                }
+            });
         } else {
-#define GO(R) pass_store<T, R>(z, freq, n, lns, xa, xb, la, lb, vout, ss)
-            DFT_SWITCH(P.r[last], GO)
+            T* x = X + (live ? tube_off(t0, cols, ld) : 0);
+#define GO(R) pass_store<T, R>(z, tw, time, n, lns, x, live, ss, inv)
+            DFT_SWITCH_FIRST(P.first, GO)
 #undef GO
         }
-        if (ns < DFT_SEQ) __syncthreads();
+        if (nts < DFT_TILE) __syncthreads();
     }
 }
 
 int rdft_parts(int rows, int cols) { return (int)(((long)rows * cols + DFT_TILE - 1) / DFT_TILE); }
 
-// Tubes t and t + 1 (t even) are neighbours in every slice and 2-element
-// aligned: one load or store serves both.
-template <typename T> static int pair_ok(const void* X, long tubes, int cols, long ld, long ss) {
-    return ld == cols && (ss & 1) == 0 && (tubes & 1) == 0 && ((size_t)X & (2 * sizeof(T) - 1)) == 0;
-}
-// the same for the spectrum's (h, tubes) rows, 16 bytes a store in float32
-template <typename T> static int hat_pair_ok(const void* Xh, long tubes) {
-    return (tubes & 1) == 0 && ((size_t)Xh & 15) == 0;
-}
-
 // Float64 transforms of few tubes take a CTA per sub-tile: the time is that of
-// one SM's float64 units on its 16 sequences (n = 73, 1600 tubes in 50 tiles:
+// one SM's float64 units on its tile (n = 73, 1600 tubes in 50 tiles:
 // 41 -> 31 us), and most SMs would be idle.  Not where the norm
 // partials are wanted, which are one per tile.
 template <typename T> static bool dft_split(unsigned tiles, const double* sumsq) {
     return sizeof(T) == 8 && !sumsq && tiles <= 76;
 }
+
+static unsigned dft_grid(const DftPlan& P, unsigned tiles) { return P.split ? tiles * (unsigned)(DFT_TILE >> P.lns) : tiles; }
 
 template <typename T>
 tp_status rdft(const T* X, void* Xh, int n, int rows, int cols, long ld, long ss, double* sumsq,
@@ -852,13 +1120,13 @@ tp_status rdft(const T* X, void* Xh, int n, int rows, int cols, long ld, long ss
     const long tubes = (long)rows * cols;
     if (tubes == 0) return TP_OK;
     const unsigned tiles = (unsigned)((tubes + DFT_TILE - 1) / DFT_TILE);
-    const DftPlan& P = dft_plan(n, sizeof(T), true, dft_split<T>(tiles, sumsq));
-    auto kern = P.cls == 0 ? k_rdft<T, 0> : (P.cls == 1 ? k_rdft<T, 1> : (P.cls == 2 ? k_rdft<T, 2> : k_rdft<T, 3>));
+    const DftPlan& P = dft_plan(n, sizeof(T), dft_split<T>(tiles, sumsq), tiles >= DFT_FULL);
+    static constexpr decltype(&k_rdft<T, 0>) forms[DFT_CLASSES] = {k_rdft<T, 0>, k_rdft<T, 1>, k_rdft<T, 2>, k_rdft<T, 3>,
+                                                                   k_rdft<T, 4>};
+    const auto kern = forms[P.cls];
     if (smem_optin((const void*)kern, P.smem) != TP_OK) return TP_ERR_CUDA;
     prof_begin(TP_KC_DFT, st);
-    kern<<<tiles * (P.split ? DFT_SEQ >> P.lns : 1), P.nt, P.smem, st>>>(
-        P, X, (cplx<T>*)Xh, tubes, cols, ld, ss, pair_ok<T>(X, tubes, cols, ld, ss), hat_pair_ok<T>(Xh, tubes), sumsq,
-        skip);
+    kern<<<dft_grid(P, tiles), P.nt, P.smem, st>>>(P, X, (cplx<T>*)Xh, tubes, cols, ld, ss, sumsq, skip);
     return launched(TP_KC_DFT, st);
 }
 
@@ -868,14 +1136,13 @@ tp_status irdft(const void* Xh, T* X, int n, int rows, int cols, long ld, long s
     const long tubes = (long)rows * cols;
     if (tubes == 0) return TP_OK;
     const unsigned tiles = (unsigned)((tubes + DFT_TILE - 1) / DFT_TILE);
-    const DftPlan& P = dft_plan(n, sizeof(T), false, dft_split<T>(tiles, nullptr));
-    auto kern =
-        P.cls == 0 ? k_irdft<T, 0> : (P.cls == 1 ? k_irdft<T, 1> : (P.cls == 2 ? k_irdft<T, 2> : k_irdft<T, 3>));
+    const DftPlan& P = dft_plan(n, sizeof(T), dft_split<T>(tiles, nullptr), tiles >= DFT_FULL);
+    static constexpr decltype(&k_irdft<T, 0>) forms[DFT_CLASSES] = {k_irdft<T, 0>, k_irdft<T, 1>, k_irdft<T, 2>,
+                                                                    k_irdft<T, 3>, k_irdft<T, 4>};
+    const auto kern = forms[P.cls];
     if (smem_optin((const void*)kern, P.smem) != TP_OK) return TP_ERR_CUDA;
     prof_begin(TP_KC_DFT, st);
-    kern<<<tiles * (P.split ? DFT_SEQ >> P.lns : 1), P.nt, P.smem, st>>>(
-        P, (const cplx<T>*)Xh, X, tubes, cols, ld, ss, hat_pair_ok<T>(Xh, tubes), pair_ok<T>(X, tubes, cols, ld, ss),
-        skip);
+    kern<<<dft_grid(P, tiles), P.nt, P.smem, st>>>(P, (const cplx<T>*)Xh, X, tubes, cols, ld, ss, skip);
     return launched(TP_KC_DFT, st);
 }
 
