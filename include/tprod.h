@@ -109,7 +109,9 @@ tp_status tprod_ifft(const void* Xhat, int l, int m, int n, void* X, int prec, v
 
 /* ---------------------------------------------------------- t-product -----
  * tprod_gemm: C = op(A) * op(B), the t-product of Definition 2.1 computed as
- * mode-3 DFT, one complex matrix product per Fourier slice, inverse DFT.
+ * mode-3 DFT, one complex matrix product per Fourier slice, inverse DFT (small
+ * float32 products: as the circular convolution itself, in one launch; the
+ * workspace is asked for in either case).
  * op(X) = X^T is the t-transpose of Section 2 (each frontal slice transposed,
  * slices 2..n reversed), the adjoint of the t-product: for C = A * B,
  * dL/dA = G * B^T and dL/dB = A^T * G.  trans bit 0 selects op(A), bit 1

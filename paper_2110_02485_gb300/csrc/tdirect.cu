@@ -15,10 +15,14 @@
 // Float32 only: the sums are as exact as the Fourier form's there (1.2e-7 to
 // 1.8e-7 relative against 1.0e-7 to 1e-6 over the sizes below), in float64 they
 // would be up to twice as far off (3e-16).  The limit on l kk m n^2: at 8e6
-// multiply-adds the kernel takes at most 10 us against 15 to 23 us of the four
-// launches (32 x 32 x 32 by one column, 1e6: 4.3 against 13 us on the device, 19
-// against 27 us a call); from 1.7e7 on it is no longer always the faster one
-// (n = 128, 32 x 32 by 1: 30 against 20 us).
+// multiply-adds in CTAs of some size the kernel takes at most 10 us against 15 to 23 us
+// of the four launches (32 x 32 x 32 by one column, 1e6: 4.3 against 13 us on the device,
+// 19 against 27 us a call); from 1.7e7 on it is no longer always the faster one (n =
+// 128, 32 x 32 by 1: 30 against 20 us).  The limit on the CTAs: one costs 2 ns whatever
+// it does, so many rows or columns of short tubes belong to the Fourier form, 32 tubes
+// a CTA there (n = 2: 1,216 CTAs 5.1 against 10.3 us, 5,000 13.6 against 10.8, 60,000
+// 124 against 45; n = 8: 5,000 11.5 against 13.5; n = 32: 7,000 18 against 47).  It also
+// keeps both dimensions of the grid in range.
 #include <algorithm>
 
 #include "common.cuh"
@@ -92,8 +96,8 @@ static size_t td_smem(int kk, int n) {
 }
 
 bool tprod_direct_fits(int l, int kk, int m, int n) {
-    const double work = (double)l * kk * m * n * n;
-    return n <= TD_MAX_N && work <= 8e6 && td_smem(kk, n) <= 100 * 1024;
+    const double work = (double)l * kk * m * n * n, ctas = (double)l * ((m + TD_COLS - 1) / TD_COLS);
+    return n <= TD_MAX_N && work <= 8e6 && ctas <= 608.0 * (n + 1) && td_smem(kk, n) <= 100 * 1024;
 }
 
 tp_status tprod_direct(const float* A, const float* B, float* C, int l, int kk, int m, int n, int trans,
