@@ -118,7 +118,7 @@ tp_status tprod_ifft(const void* Xhat, int l, int m, int n, void* X, int prec, v
  * op(B):
  *   bit 0 clear: A is l x kk x n, array (n, l, kk);  set: A is kk x l x n, (n, kk, l)
  *   bit 1 clear: B is kk x m x n, array (n, kk, m);  set: B is m x kk x n, (n, m, kk)
- *   C : real (n, l, m)
+ *   C : real (n, l, m); it may overlap A or B
  * Workspace: tprod_gemm_workspace_bytes(l, kk, m, n, prec).
  */
 size_t tprod_gemm_workspace_bytes(int l, int kk, int m, int n, int prec);

@@ -159,10 +159,17 @@ static size_t gemm_ws(int l, int kk, int m, int n, size_t c) {
     return align256(h * l * kk * c) + align256(h * kk * m * c) + align256(h * l * m * c);
 }
 
+static bool disjoint(const void* a, size_t na, const void* b, size_t nb) {
+    return (const char*)a + na <= (const char*)b || (const char*)b + nb <= (const char*)a;
+}
+
 template <typename T>
 static tp_status gemm_t(const void* A, const void* B, void* C, int l, int kk, int m, int n, int trans, void* ws,
                         cudaStream_t st, int tc_passes = 3) {
-    if (sizeof(T) == 4 && tc_passes == 3 && tprod_direct_fits(l, kk, m, n))
+    // the one-launch form writes C while it reads A and B; the others have read them by then
+    const size_t nA = sizeof(T) * n * l * kk, nB = sizeof(T) * n * kk * m, nC = sizeof(T) * n * l * m;
+    if (sizeof(T) == 4 && tc_passes == 3 && tprod_direct_fits(l, kk, m, n) && disjoint(C, nC, A, nA) &&
+        disjoint(C, nC, B, nB))
         return tprod_direct((const float*)A, (const float*)B, (float*)C, l, kk, m, n, trans, st);
     const int h = n / 2 + 1;
     const size_t c = 2 * sizeof(T);

@@ -39,3 +39,24 @@ def test_many_rows_or_columns(tp, n, l, kk, m):
     C = tp.tprod(A, B).double()
     ref = reference(A, B)
     assert float((C - ref).norm() / ref.norm()) <= tolerance(n, kk)
+
+
+@pytest.mark.parametrize("n,l,m", [(1, 4, 4), (8, 6, 5), (32, 32, 1), (33, 16, 9), (64, 12, 12), (240, 24, 6)])
+@pytest.mark.parametrize("over", ["A", "B", "shifted"])
+def test_result_over_an_operand(tp, n, l, m, over):
+    """tprod_gemm with C at A, at B, or a slice past the start of B: small products and one of the Fourier form."""
+    g = torch.Generator(device="cuda").manual_seed(n)
+    if over == "A":
+        m = l
+    A = torch.randn((n, l, l), generator=g, device="cuda")
+    buf = torch.randn((n + 1, l, m), generator=g, device="cuda")
+    B = buf[:n]
+    ref = reference(A, B)
+    C = A if over == "A" else (B if over == "B" else buf[1:])
+    L = tp.load()
+    ws = torch.empty(L.tprod_gemm_workspace_bytes(l, l, m, n, 0) + 256, dtype=torch.uint8, device="cuda")
+    wp = -(-ws.data_ptr() // 256) * 256
+    st = L.tprod_gemm(A.data_ptr(), B.data_ptr(), C.data_ptr(), l, l, m, n, 0, 0, wp, ws.data_ptr() + ws.numel() - wp,
+                      torch.cuda.current_stream().cuda_stream)
+    assert st == 0
+    assert float((C.double() - ref).norm() / ref.norm()) <= tolerance(n, l)
