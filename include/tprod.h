@@ -235,10 +235,10 @@ tp_status rtsvd_adjoint(const void* G, int l, int m, int n, int p, const tp_rtsv
  * ttsvd_solve: the T-tSVD method (Section 4.1, Eqs. (11)-(14)): the full tSVD
  * of A and X_s = sum_{i<=s} V_i * s_i^{-1} * U_i^T * B with the smallest s
  * whose residual ||B - A*X_s||_F <= tau*delta (Eq. (disp); else s = the last
- * index and TP_ERR_NOT_CONVERGED).  Computed by the RT-tSVD path with the
- * t-identity as the sketching tensor and r = min(l, m) (the sketch then spans
- * the whole range of A, and B-tilde has A's singular values), no power
- * iterations, the scan of Eq. (disp) from s = 1.  Singular values at or below
+ * index and TP_ERR_NOT_CONVERGED).  Computed by the RT-tSVD path with r =
+ * min(l, m) and a basis that spans the whole range of A (its columns,
+ * orthonormalised, or the t-identity where l < m), so that B-tilde has A's
+ * singular values, no power iterations, the scan of Eq. (disp) from s = 1.  Singular values at or below
  * max(l,m)*eps*sigma_max are treated as zero.  B (n, l, p), X (n, m, p); p > 1
  * slices share one s (as rtsvd_truncated_solve).
  * Limits: min(l, m) <= 256, and as rtsvd_truncated_solve (with r_max = min(l, m)).

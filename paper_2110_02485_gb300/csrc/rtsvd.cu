@@ -1936,7 +1936,7 @@ __global__ void k_dp_reduce(const double* out, long so, int h, int np, int n, St
 }
 
 // Columns col[0 .. b-1] of every A-hat slice (l x m) as the block Y (l x b): the
-// sketch of the T-tSVD (tt_solve), whose sketching slices are unit vectors.
+// sketch of the T-tSVD of l >= m (tt_solve), whose sketching slices are unit vectors.
 struct ColList {
     int col[MAX_BLOCK];
 };
@@ -1948,6 +1948,20 @@ __global__ void __launch_bounds__(256) k_take_cols(const cplx<T>* __restrict__ A
     if (e >= l * b) return;
     const int i = e / b, c = e - i * b;
     Y[s * l * b + e] = A[(s * l + i) * m + list.col[c]];
+}
+
+// Unit vectors e_col[c] as the block Y and as the basis rows r0 + c of Q (vectors of
+// length l, sQ entries per slice): T-tSVD of operators with fewer rows than columns.
+template <typename T>
+__global__ void __launch_bounds__(256) k_unit_cols(int l, int b, const __grid_constant__ ColList list,
+                                                   cplx<T>* __restrict__ Y, cplx<T>* __restrict__ Q, long sQ, int r0) {
+    const long s = blockIdx.y;
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= l * b) return;
+    const int i = e / b, c = e - i * b;
+    const cplx<T> v = mk<T>(i == list.col[c] ? (T)1 : (T)0, 0);
+    Y[s * l * b + e] = v;
+    Q[s * sQ + (long)(r0 + c) * l + i] = v;
 }
 
 // ---------------------------------------------------------------------------
@@ -2129,7 +2143,7 @@ static tp_status rt_solve_impl(const T* A, const T* B, const T* Om, int l, int m
                                      st);
         return e == TP_ERR_UNSUPPORTED ? TP_ERR_ARG : e;
     };
-    // T-tSVD: the columns 0 .. r_max - 1 in bit-reversed order (see tt_solve)
+    // T-tSVD: the columns (or, l < m, the rows) 0 .. r_max - 1 in bit-reversed order (see tt_solve)
     int spread[RT_MAX_RANK], nspread = 0;
     for (int i = 0; full && nspread < r_max; ++i) {
         int rev = 0;
@@ -2143,16 +2157,18 @@ static tp_status rt_solve_impl(const T* A, const T* B, const T* Om, int l, int m
         if (full) {
             ColList list;
             for (int c = 0; c < bb; ++c) list.col[c] = spread[r0 + c];
+            const dim3 grid((unsigned)((l * bb + 255) / 256), (unsigned)h);
             prof_begin(TP_KC_GEMM, st);
-            k_take_cols<T><<<dim3((unsigned)((l * bb + 255) / 256), (unsigned)h), 256, 0, st>>>(w.Ahat, l, m, bb, list,
-                                                                                                w.Y);
+            if (l < m) k_unit_cols<T><<<grid, 256, 0, st>>>(l, bb, list, w.Y, w.Q, (long)r_max * l, r0);
+            else k_take_cols<T><<<grid, 256, 0, st>>>(w.Ahat, l, m, bb, list, w.Y);
             TRY(launched(TP_KC_GEMM, st));
         } else {
             TRY(sketch(l, bb, m, w.Ahat, w.Abf, m, OP_N, w.G + r0, r_max, (long)m * r_max, w.Y, bb, (long)l * bb));
         }
         const bool last_y = (P->q_power == 0);
-        TRY(orth<T>(h, w.Y, (long)l * bb, l, bb, w.Q, (long)r_max * l, r0, last_y ? w.Q : nullptr, nullptr, 0, 0, 0,
-                    nullptr, done, st));
+        if (!full || l >= m)
+            TRY(orth<T>(h, w.Y, (long)l * bb, l, bb, w.Q, (long)r_max * l, r0, last_y ? w.Q : nullptr, nullptr, 0, 0,
+                        0, nullptr, done, st));
         for (int it = 0; it < P->q_power; ++it) {
             TRY(sketch(m, bb, l, AH, w.ATbf, ldah, op_h, w.Y, bb, (long)l * bb, w.Z, bb, (long)m * bb));
             TRY(orth<T>(h, w.Z, (long)m * bb, m, bb, nullptr, 0, 0, nullptr, nullptr, 0, 0, 0, nullptr, done, st));
@@ -2263,12 +2279,14 @@ tp_status rt_adjoint(const T* G, int l, int m, int n, int p, const tp_rtsvd_para
 }
 
 // ---------------------------------------------------------------------------
-// T-tSVD method (Section 4.1, Eqs. (11)-(14)) through the RT-tSVD path: with
-// the t-identity's lateral slices as the sketching tensor and r = min(l, m),
-// the block sketch spans the whole range of every A-hat slice, B-tilde =
-// Q^H A-hat has the singular values of A-hat, and the discrepancy scan from
-// k = 1 (p = r in Eq. (kinit)) is Eq. (14)'s choice of s.  No power iterations;
-// a block's product with A-hat is a copy of its columns.
+// T-tSVD method (Section 4.1, Eqs. (11)-(14)) through the RT-tSVD path with r =
+// min(l, m) and a basis Q that holds the whole range of every A-hat slice, so that
+// B-tilde = Q^H A-hat has the singular values of A-hat, and the discrepancy scan
+// from k = 1 (p = r in Eq. (kinit)) is Eq. (14)'s choice of s.  No power iterations.
+//   l >= m: the sketching slices are the t-identity's, all m of them: a block's product with
+//     A-hat is a copy of its columns, which are then orthonormalised.
+//   l < m: l of the columns need not span the range (the leading ones may be zero or
+//     repeated); the unit vectors of the l rows do, and B-tilde is A-hat itself.
 //
 // The columns come in bit-reversed order.  Any order gives the same subspace;
 // this one takes widely spaced columns first, which for operators whose
