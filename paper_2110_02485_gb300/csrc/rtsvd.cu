@@ -54,17 +54,7 @@ template <> __device__ __forceinline__ float rsqrt_t<float>(float x) {
     const float y = rsqrtf(x);
     return y * fmaf(-0.5f * x * y, y, 1.5f);
 }
-// 1/sqrt(x), x positive and normal: two Newton steps on the hardware's
-// approximation (its relative error is below 2^-20, theirs below 2^-52)
-__device__ __forceinline__ double rsqrt_nr64(double x) {
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    y = y * fma(-0.5 * x * y, y, 1.5);
-    return y * fma(-0.5 * x * y, y, 1.5);
-}
-template <> __device__ __forceinline__ double rsqrt_t<double>(double x) {
-    return x > 1e-290 && x < 1e290 ? rsqrt_nr64(x) : 1.0 / sqrt(x);
-}
+template <> __device__ __forceinline__ double rsqrt_t<double>(double x) { return 1.0 / sqrt(x); }
 
 // Cholesky factor of a 16 x 16 Hermitian Gram matrix (upper triangle of G in
 // shared memory) by the first 160 threads (warps 0-4, named barrier 1): thread
@@ -1023,8 +1013,7 @@ __device__ int jacobi_sweeps_smem(cplx<T>* Rs, cplx<T>* dp, int np, int r, int m
 // so a round (r / 2 disjoint pairs) runs in three phases that keep the count
 // down: 16 lanes per pair form g = x^H y alone (4 multiply-adds per entry; the
 // squared norms are carried through the rotations as in the float32 form);
-// one lane per pair works out the rotations, 32 pairs to a warp, with
-// Newton-refined reciprocals instead of divisions and square roots; 16 lanes
+// one lane per pair works out the rotations, 32 pairs to a warp; 16 lanes
 // per pair apply them at 8 multiply-adds per entry (the cosines are kept as
 // scales of the columns, folded in at every sweep's start).  The form before
 // had every lane of a pair do the scalar work and form both norms in every
@@ -1036,14 +1025,6 @@ struct JacPair64 {
     double c;
 };
 constexpr int JAC64_PAIRS = RT_MAX_RANK / 2;
-
-// 1/x, x positive and normal, in the same way as rsqrt_nr64
-__device__ __forceinline__ double rcp_nr64(double x) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    y = fma(y, fma(-x, y, 1.0), y);
-    return fma(y, fma(-x, y, 1.0), y);
-}
 
 // cn, cd: squared norms and scales of the columns (r entries each).
 __device__ int jacobi_sweeps_f64(double2* Rs, double2* dp, int np, int r, int max_sweeps, double tol, double* cn,
@@ -1100,16 +1081,16 @@ __device__ int jacobi_sweeps_f64(double2* Rs, double2* dp, int np, int r, int ma
                     const double dx = cd[p], dy = cd[q], a = cn[p], b = cn[q], dd = dx * dy;
                     const double2 g = cscale(pr[tid].g, dd);
                     const double ag2 = fma(g.x, g.x, g.y * g.y), ab = a * b;
-                    if (ab > 0.0) atomicMax(max_off, __float_as_int((float)(ag2 * rcp_nr64(fmax(ab, 1e-300)))));
                     if (a > 0.0 && b > 0.0 && ag2 > 1e-290 && ag2 > tol2 * ab) {
-                        const double rg = rsqrt_nr64(ag2);  // 1/|g|
+                        atomicMax(max_off, __float_as_int((float)(ag2 / fmax(ab, 1e-300))));  // (the others are below tol)
+                        const double rg = rsqrt(ag2);  // 1/|g|
                         const double2 e = cscale(g, rg);
                         // zeta = (b - a) / (2 |g|); beyond 1e100 its square would overflow and t is 0 to rounding anyway
                         const double zeta = fmin(fmax((b - a) * 0.5 * rg, -1e100), 1e100);
                         const double w = fma(zeta, zeta, 1.0);
-                        const double tt = copysign(rcp_nr64(fabs(zeta) + w * rsqrt_nr64(w)), zeta);
-                        const double c = rsqrt_nr64(fma(tt, tt, 1.0));
-                        const double tg = tt * (ag2 * rg), q1 = tt * dy * rcp_nr64(dx), q2 = tt * dx * rcp_nr64(dy);
+                        const double tt = copysign(1.0 / (fabs(zeta) + sqrt(w)), zeta);
+                        const double c = rsqrt(fma(tt, tt, 1.0));
+                        const double tg = tt * (ag2 * rg), sc = tt / dd, q1 = sc * dy * dy, q2 = sc * dx * dx;
                         o.g = make_double2(e.x * q1, -e.y * q1);
                         o.f2 = cscale(e, q2);
                         o.se = cscale(e, c * tt);
