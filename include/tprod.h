@@ -168,10 +168,14 @@ tp_status tprod_gemm_noalloc(const void* A, const void* B, void* C, int l, int k
  *   Omega : real (n, m, r_max)   (Gaussian test slices, supplied by the caller)
  * Limits: 1 <= block <= 32; r_max <= min(l, m) and r_max <= 256; l, m <=
  * 1024; 1 <= p <= 64.  The small SVD keeps R's working copy in shared memory
- * while (r_max^2 + r_max p) complex entries fit in 227 KB, else in the
- * workspace (global memory, L2-resident); its r_max p right-hand sides must
- * fit in shared memory in either case; and the block orthonormalisation's
- * working set (about (l + 1) b + 2 r_max b complex entries) must fit too.
+ * while about (r_max^2 + r_max p) complex entries fit in 224 KB (float32) or 215
+ * KB (float64), else in the workspace (global memory, L2-resident); its r_max p
+ * right-hand sides must fit in 227 KB in either case.  The block
+ * orthonormalisation's working set must fit in shared memory too, which for
+ * blocks of up to 16 (up to 32) columns means
+ *   max(l, m) + 2 r_max <= 1399 (762) in float32, 811 (308) in float64;
+ * float64 blocks of up to 4 columns take every size.  Other sizes are refused
+ * with TP_ERR_ARG.
  * Float32 range: the small SVD forms squared inner products of the factor
  * (fourth powers of the data's magnitude), so float32 data far from unit
  * scale (entries of A near 1e-13, say) can end in TP_ERR_NOT_CONVERGED;
