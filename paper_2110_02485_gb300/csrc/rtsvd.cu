@@ -437,11 +437,9 @@ __device__ void orth_update_h16(const float2* __restrict__ Q, float2* Ys, int L,
 }
 
 // Shared-memory extents of k_orth beyond its matrices: the partial tiles of
-// the tensor-core products (float32, 16 columns), and the Gram partials (one
-// per thread, at least one per upper-triangle entry; none in the TC kernel).
-template <typename T, int BB> constexpr size_t orth_part_bytes() {
-    return (sizeof(T) == 4 && BB == 16) ? (size_t)PART_TILES * 2048 : 0;
-}
+// the tensor-core products (TC), or the Gram partials (one per thread, at least one
+// per upper-triangle entry).
+constexpr size_t ORTH_PART_BYTES = (size_t)PART_TILES * 2048;
 template <typename T, int BB> constexpr size_t orth_gram_elems() {
     return (size_t)(BB * (BB + 1) / 2 > OrthThreads<T, BB>::v ? BB * (BB + 1) / 2 : OrthThreads<T, BB>::v);
 }
@@ -473,7 +471,7 @@ k_orth(cplx<T>* Y, long sY, int L, int b, const cplx<T>* Qb, long sQ, int r_prev
     V* G = Cp + (size_t)r_prev * BB;        // BB x BB Gram / Cholesky work
     V* Rk = G + BB * BB;                    // this pass's R
     float* part = (float*)(Rk + BB * BB);   // partial coefficient tiles
-    constexpr size_t GRAM = TC ? 0 : orth_gram_elems<T, BB>(), PART = orth_part_bytes<T, BB>();
+    constexpr size_t GRAM = TC ? 0 : orth_gram_elems<T, BB>(), PART = TC ? ORTH_PART_BYTES : 0;
     V* gpart = (V*)((unsigned char*)part + PART);  // Gram partials
     V* Rt = gpart + GRAM;                   // copy of G (SIMT Cholesky), scratch for the product Rk Ra
     V* Ra = Rt + BB * BB;                   // accumulated in-block R (R an output)
@@ -630,9 +628,9 @@ k_orth(cplx<T>* Y, long sY, int L, int b, const cplx<T>* Qb, long sQ, int r_prev
         // coefficient product with the block's own columns as the basis, the
         // full 16 x 16, 3xTF32); otherwise the upper triangle incl. diagonal by
         // a thread per (entry, chunk of rows), the chunk sums meeting in gpart
-        if (TC || (sizeof(T) == 4 && BB == 16 && (L & 15) == 0)) {
+        if constexpr (TC) {
             orth_coef_mma<false>((const float2*)Ys, LP, (const float2*)Ys, L, LP, 16, (float2*)G, part);
-        } else if constexpr (!TC) {
+        } else {
             constexpr int NE = BB * (BB + 1) / 2;
             // chunks of at least four rows, at most 32 (their sums are added one after another)
             const int nch = max(1, min((int)blockDim.x / NE, min(32, L / 4)));
@@ -823,28 +821,23 @@ template <typename T> static bool orth_tc(int L, int b, int r_prev) {
     return sizeof(T) == 4 && b <= 16 && (L & 15) == 0 && r_prev <= 256;
 }
 
-template <typename T> static void orth_extents(int BB, size_t& part, size_t& gram) {
-    part = BB == 16 ? orth_part_bytes<T, 16>() : 0;
-    gram = BB == 1 ? orth_gram_elems<T, 1>() : (BB == 4 ? orth_gram_elems<T, 4>() :
+template <typename T> static size_t orth_gram(int BB) {
+    return BB == 1 ? orth_gram_elems<T, 1>() : (BB == 4 ? orth_gram_elems<T, 4>() :
            (BB == 16 ? orth_gram_elems<T, 16>() : orth_gram_elems<T, 32>()));
 }
 template <typename T> static size_t orth_smem(int L, int b, int r_prev, bool has_r) {
     const int BB = orth_cols<T>(b);
     const bool tc = orth_tc<T>(L, b, r_prev);
-    size_t part, gram;
-    orth_extents<T>(BB, part, gram);
-    size_t e = (size_t)BB * (L + 1) + (size_t)r_prev * BB + 2 * BB * BB + (tc ? 0 : gram + BB * BB);
+    size_t e = (size_t)BB * (L + 1) + (size_t)r_prev * BB + 2 * BB * BB + (tc ? 0 : orth_gram<T>(BB) + BB * BB);
     if (has_r) e += (tc ? 2 : 1) * BB * BB;
-    return e * sizeof(cplx<T>) + part;
+    return e * sizeof(cplx<T>) + (tc ? ORTH_PART_BYTES : 0);
 }
 // The sizes a solve takes: with 40 KB for the tensor-core partials and both
 // coefficient blocks the largest launch stays within 227 KB (orth_smem is less).
 template <typename T> static bool orth_fits(int L, int b, int r) {
     const int BB = orth_cols<T>(b);
-    size_t part, gram;
-    orth_extents<T>(BB, part, gram);
-    const size_t e = (size_t)BB * (L + 1) + 2 * (size_t)r * BB + 4 * BB * BB + gram;
-    return e * sizeof(cplx<T>) + (part ? 40960 : 0) <= 227 * 1024;
+    const size_t e = (size_t)BB * (L + 1) + 2 * (size_t)r * BB + 4 * BB * BB + orth_gram<T>(BB);
+    return e * sizeof(cplx<T>) + (sizeof(T) == 4 && BB == 16 ? 40960 : 0) <= 227 * 1024;
 }
 
 template <typename T>
@@ -1549,8 +1542,10 @@ static tp_status jacobi_launch(int h, const cplx<T>* R, long ldr, long sR, const
     // a working set that leaves no room for the sweeps' scratch takes the sweeps without it
     if (smem > jac_smem_limit(sizeof(T))) {
         smem = jacobi_smem(r_max, sizeof(cplx<T>), np, gR != nullptr, false);
-        if (smem > 227 * 1024) return TP_ERR_UNSUPPORTED;
-        kern = gR ? k_jacobi<T, false, true> : k_jacobi<T, false, false>;
+        if (smem > 227 * 1024 || (gR && sizeof(T) == 4)) return TP_ERR_UNSUPPORTED;
+        kern = k_jacobi<T, false, false>;
+        if constexpr (sizeof(T) == 8)  // float32 right-hand sides alone (64 at rank 256: 134 KB) never fill it
+            if (gR) kern = k_jacobi<T, false, true>;
         nt = jac_threads<T>(false);
     }
     if (smem_optin((const void*)kern, smem) != TP_OK) return TP_ERR_CUDA;
