@@ -54,7 +54,7 @@ template <> __device__ __forceinline__ float rsqrt_t<float>(float x) {
     const float y = rsqrtf(x);
     return y * fmaf(-0.5f * x * y, y, 1.5f);
 }
-template <> __device__ __forceinline__ double rsqrt_t<double>(double x) { return 1.0 / sqrt(x); }
+template <> __device__ __forceinline__ double rsqrt_t<double>(double x) { return rsqrt(x); }
 
 // Cholesky factor of a 16 x 16 Hermitian Gram matrix (upper triangle of G in
 // shared memory) by the first 160 threads (warps 0-4, named barrier 1): thread
