@@ -164,11 +164,8 @@ __device__ void mvn_multi(const cplx<T>* __restrict__ A, int l, int m, const cpl
 // times (coefficients and update of both passes) with ordinary loads: the group's
 // bases (PB cnt vectors, 123 KB at 256 entries and the mean cnt of 7.5) stay in
 // the L1 beside this kernel's 52 KB of shared memory, and A, whose loads bypass
-// it, does not evict them.  (Bypassing L1 here too: 18.1k + 22.5k cycles per
-// step on the two sides, now 16.2k + 19.9k.  Measured and not kept, both on 512
-// threads of 128 registers: four columns or rows of A per lane in the products,
-// 49k + 43k against 38k + 44k cycles, and 16 basis loads in flight here, 24k +
-// 25k.)
+// it, does not evict them (bypassing L1 here too: 18.1k + 22.5k cycles per step on
+// the two sides, now 16.2k + 19.9k).
 template <typename T, int PB>
 __device__ void reorth_multi(cplx<T>* u, int lu, int len, const cplx<T>* gb, long bsj, int cnt, const int* act,
                              cplx<T>* cf, int cfs) {

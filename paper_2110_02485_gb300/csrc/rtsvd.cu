@@ -28,7 +28,8 @@ constexpr int MAX_BLOCK = 32;
 
 // ---------------------------------------------------------------------------
 // Block orthonormalisation (Algorithm 3, Normalize + reorthogonalisation, in
-// block form), one CTA of 1024 threads per Fourier slice:
+// block form), one CTA of 512 threads (256 for float64 blocks of more than 16
+// columns) per Fourier slice:
 //   1. Y <- Y - Q (Q^H Y), twice (classical Gram-Schmidt against the basis);
 //   2. Y = Q_new R by shifted Cholesky-QR3 (Fukaya et al., 2020): one Cholesky
 //      QR of the Gram matrix shifted by 11 (L b + b(b+1)) u ||Y||_F^2, then two
@@ -893,16 +894,16 @@ __global__ void k_rt_init(State* st, const double* partsA, int nA, const double*
 
 // ---------------------------------------------------------------------------
 // One-sided Jacobi SVD of R (r x r) per slice, rotations from the right
-// (cyclic round-robin ordering, r/2 disjoint pairs per round, a group of
-// lanes per pair: 8 in the float32 register form, 16 in the shared-memory
-// form).  Tracks d' = J^H d.  Outputs, sorted by decreasing sigma:
+// (cyclic round-robin ordering over columns, 16 lanes per pair, or in float32
+// over blocks of four columns, 16 or 32 lanes per pair of blocks).  Tracks
+// d' = J^H d.  Outputs, sorted by decreasing sigma:
 // sigma (r), U_R (r x r row-major, columns normalised), d'.
 //
 // A pair (p, q) with Gram entries a = |x|^2, b = |y|^2, g = x^H y is rotated
 // when |g| > tol sqrt(a b) (tol = 4 sqrt(r) u): with e = g/|g|,
 // zeta = (b - a) / (2|g|), t = sign(zeta) / (|zeta| + sqrt(1 + zeta^2)),
 // c = 1/sqrt(1 + t^2), s = c t, the columns become x' = c x - s conj(e) y and
-// y' = s x + c conj(e) y, which makes them orthogonal.
+// y' = s e x + c y (or conj(e) times that), which makes them orthogonal.
 // Convergence is quadratic once the columns are nearly orthogonal: a sweep
 // whose largest relative off-diagonal |g|/sqrt(a b) is below sqrt(tol) leaves
 // residues below tol, so the sweep after it (which would only confirm) is
@@ -2264,15 +2265,16 @@ tp_status rt_adjoint(const T* G, int l, int m, int n, int p, const tp_rtsvd_para
 //   l < m: l of the columns need not span the range (the leading ones may be zero or
 //     repeated); the unit vectors of the l rows do, and B-tilde is A-hat itself.
 //
-// The columns come in bit-reversed order.  Any order gives the same subspace;
-// this one takes widely spaced columns first, which for operators whose
-// neighbouring columns are alike (blurs) does what column pivoting does: R
-// comes out graded, and the Jacobi SVD needs 8 sweeps where the natural order
-// needs 13 to 16 (float32 emulation and runs at 192 and 256; true column
-// pivoting: 7 to 8; a random order: 9 to 12).  The
-// 256^3 solve: 64.8 -> 22.1 ms, of which the SVD 57.6 -> 15.2.  Measured and
-// not kept: random slices with a power iteration (6 sweeps, but up to
-// 10 times the float32 error on ill-conditioned slices).
+// The columns (rows) come in bit-reversed order.  Any order gives the same
+// subspace; this one takes widely spaced columns first, as column pivoting would for
+// operators whose neighbouring columns are alike (blurs), and the Jacobi SVD of the
+// 256^3 image problem takes 8 or 9 sweeps.  In the natural order it took 18 there
+// (float32 emulation at 192 and 256: natural 13 to 16, random 9 to 12, true column
+// pivoting 7 to 8).  The
+// 256^3 solve takes 18.9 ms, of which the SVD 13.1 (64.8 and 57.6 in the natural order
+// with the kernel of one column pair per eight lanes).  Measured and not kept: random
+// slices with a power iteration (6 sweeps, but up to 10 times the float32 error on
+// ill-conditioned slices).
 // ---------------------------------------------------------------------------
 template <typename T>
 static tp_rtsvd_params tt_params(int l, int m, const tp_ttsvd_params* P) {
