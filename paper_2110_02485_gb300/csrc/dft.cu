@@ -32,12 +32,12 @@
 // that every n but the powers of two took (1), a radix-2 kernel for those and
 // 16 x 16 and 16 x 32 forms for n = 256 and 512, and two tubes as one complex sequence (2):
 //   n     now                      (1)              (2)
-//   96    16.0 / 14.8 us           111 / 135        14.6 / 15.0
-//   128   14.7 / 16.6 us           49 / 32          14.2 / 16.6
-//   256   30.7 / 32.8 us (4.4 TB/s) 31 / 37         29.9 / 34.1
-//   331   280 / 268 us             1166 / 1480      324 / 283   (prime)
-//   384   48.9 / 50.0 us (4.1 TB/s) 1571 / 1980     53.5 / 55.2
-//   512   62.7 / 67.1 us (4.3 TB/s) 73 / 123        73.0 / 77.8
+//   96    15.2 / 16.3 us           111 / 135        14.6 / 15.0
+//   128   14.2 / 16.5 us           49 / 32          14.2 / 16.6
+//   256   29.7 / 32.8 us (4.5 TB/s) 31 / 37         29.9 / 34.1
+//   331   280 / 267 us             1166 / 1480      324 / 283   (prime)
+//   384   49.0 / 49.9 us (4.1 TB/s) 1571 / 1980     53.5 / 55.2
+//   512   62.0 / 67.3 us (4.3 TB/s) 73 / 123        73.0 / 77.8
 //   1000  210 / 182 us             18651 / 19087    215 / 178
 // The forward's root mean square error at 256 and 384 is 0.90e-7 and 0.95e-7 (0.99e-7 and
 // 1.19e-7 in the form (2)): the first sums and differences are taken on exact data.
@@ -453,8 +453,8 @@ static DftPlan make_plan(int n, size_t elem, bool split, bool full) {
         P.np = DFT_MAX_PASS;
         best_radices(m, 0, 0, 0, cur, P.r, &P.np, &sum);
     } else {
-        // Fewest passes, then the least arithmetic, about W words times the radix of a complex pass and n / 3 times the
-        // real one (float32 radices above 10 take more registers: a tenth more).  A single pass of a wide radix counts as
+        // Fewest passes, then the least arithmetic, about W words times the radix of a complex pass and 0.3 n times the
+        // real one (fitted to n = 96 .. 384; float32 radices above 10 take more registers: a tenth more).  A single pass of a wide radix counts as
         // two: most lanes of a small tile would idle (n = 32 in float64, one pass of 32 and 8 x 4: 15.8 and 6.7 us for
         // 32 x 32 tubes; n = 24 in float32, 256 x 256 tubes: 8.2 and 5.3 us).
         int passes = INT_MAX;
@@ -465,7 +465,7 @@ static DftPlan make_plan(int n, size_t elem, bool split, bool full) {
             int r[DFT_MAX_PASS], np = DFT_MAX_PASS, sum = INT_MAX;
             best_radices(rest, 0, 0, 0, cur, r, &np, &sum);
             const int total = np + 1 + (np == 0 && f >= 8 ? 1 : 0);
-            double c = (double)(f / 2 + 1) * rest * (np ? sum : 0) + n * f / 3.0;
+            double c = (double)(f / 2 + 1) * rest * (np ? sum : 0) + 0.3 * n * f;
             if (elem == 4 && (f > 10 || (np && r[0] > 10)) && (n & (n - 1))) c *= 1.1;
             if (total < passes || (total == passes && c < cost)) {
                 passes = total;
@@ -495,10 +495,12 @@ static DftPlan make_plan(int n, size_t elem, bool split, bool full) {
     // a thread per item of the first pass
     const int items = P.M << P.lns;
     P.nt = std::min(DFT_MAX_THREADS, std::max(64, (items + 31) & ~31));
-    // where tiles fill the SMs, about 24 words a thread: fewer threads keep more tiles (and loads) in flight (n = 128,
-    // 256 x 256 tubes, 256 and 128 threads: 18.0 and 14.4 us; with 200 tiles in all 4.1 and 4.3 us)
+    // where tiles fill the SMs, fewer threads keep more tiles (and loads) in flight (n = 128, 256 x 256 tubes, 256 and
+    // 128 threads: 18.0 and 14.4 us; with 200 tiles in all 4.1 and 4.3 us), more so beside three CTAs of 256 than four
+    // (n = 240: 34.3 and 30.7 us; n = 256: 30.5 and 33.9)
     const int want = (P.len << P.lns) / 24;
-    if (full) P.nt = std::min(P.nt, want <= 64 ? 64 : (want <= 144 ? 128 : DFT_MAX_THREADS));
+    if (full && P.cls < 2) P.nt = std::min(P.nt, want <= 64 ? 64 : (want <= 144 ? 128 : DFT_MAX_THREADS));
+    if (full && P.cls >= 2) P.nt = std::min(P.nt, want <= 64 ? 64 : (want <= 224 ? 128 : (want <= 250 ? 192 : DFT_MAX_THREADS)));
     // The direct part: M columns of groups of kb pairs on a quarter as many lanes as tubes, about 12 kb + 4 instructions
     // per entry.  Up to about 370 points one round of some width does (17 .. 61 points on 64 or 128 threads, 331 on
     // 256): the cheapest of those, counting no fewer than three warps (fewer leave the SM waiting).  Beyond, 256 threads
@@ -527,15 +529,16 @@ static DftPlan make_plan(int n, size_t elem, bool split, bool full) {
     return P;
 }
 
-// The plans of the last lengths that a thread used (the search takes about a
-// microsecond, which a small transform would notice).
+// The plans of the last lengths that a thread used (the search takes some
+// microseconds, which a small transform would notice).  A solve uses one length with
+// few and with many tiles, split and not: a slot for each.
 static const DftPlan& dft_plan(int n, size_t elem, bool split, bool full) {
     struct Slot {
         DftPlan P;
         size_t elem = 0;
     };
-    thread_local Slot slots[16];
-    Slot& s = slots[((n * 2) ^ (elem == 4 ? 1 : 0)) & 15];
+    thread_local Slot slots[64];
+    Slot& s = slots[((n << 3) | (elem == 4 ? 4 : 0) | (split ? 2 : 0) | (full ? 1 : 0)) & 63];
     if (s.elem != elem || s.P.n != n || s.P.split != split || s.P.full != full) {
         s.P = make_plan(n, elem, split, full);
         s.elem = elem;
@@ -676,7 +679,7 @@ constexpr int dft_batch(int R) { return R >= 12 ? 1 : (R >= 6 ? 2 : (R > 1 ? 4 :
 template <typename T, int R>
 __device__ __forceinline__ void pass_load(cplx<T>* z, const cplx<T>* tw, int n, int lns, const T* x, bool live, long ss,
                                           T& acc) {
-    constexpr int U = dft_batch(R);
+    constexpr int U = (R == 16 || R == 8 ? 2 : 1) * dft_batch(R);  // powers of two: 32 loads (30.5 -> 29.7 us at n = 256)
     const int p = threadIdx.x & ((1 << lns) - 1), M = n / R, ust = blockDim.x >> lns;
     for (int j0 = threadIdx.x >> lns; j0 < M; j0 += U * ust) {
         T a[U][R];
