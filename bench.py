@@ -45,20 +45,20 @@ FP32_SIMT_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 _SRC = "paper_2110_02485_gb300/csrc/"
 _SHA = {"zgemm_tc.cu": "4f198436354ce99befa630db5c8f7430aed52afddb33c65deea71d7af335262b",
         "cgemm.cu": "8b4cf3173196c2b8142d78471b918fb0ba5edbbbc9a3e09996063edc4883a3ab",
-        "rtsvd.cu": "61e61b8c7b57b18d0d3416339cd34dc442be0b189164623a0d3f15ccbec2c887",
+        "rtsvd.cu": "575508f39d5c2290abab07529a308a1ae7ca0badce547c8593552997649f7325",
         "gkb.cu": "fd3a4bc662f251cde3dce1b2b5eff906b7b590f91a142f5a30352c37dedb855e",
-        "dft.cu": "af6a94d0c8570c6af241d4b07bf3480d190a19bc297f3d4c60334a6e83210c18"}
+        "dft.cu": "a3306f11ff69eb39ca8c4ba3905c379b1da74129f82d2c828846d5f7f314d354"}
 # DRAM bytes (read + write) per launch of each kernel class, averaged over the class's launches in one plain
 # step of the n256 workload (ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum over the whole step,
 # profiles/launches_n256_bench_step.md), with the sha256 of every source the class's kernels come from: a record
 # whose sources changed since the capture reads as null.
 NCU_TRAFFIC = {
-    "gemm": {"bytes": 43.68e6, "sources": ["zgemm_tc.cu", "cgemm.cu", "rtsvd.cu"],
+    "gemm": {"bytes": 43.69e6, "sources": ["zgemm_tc.cu", "cgemm.cu", "rtsvd.cu"],
              "profile": "profiles/k_zgemm_tc_n256.md"},
-    "gkb": {"bytes": 68.60e6, "sources": ["gkb.cu"], "profile": "profiles/k_gkb_n256.md"},
-    "orth": {"bytes": 7.36e6, "sources": ["rtsvd.cu"], "profile": "profiles/k_orth_n256.md"},
-    "svd": {"bytes": 9.76e6, "sources": ["rtsvd.cu"], "profile": "profiles/k_jacobi_n256.md"},
-    "dft": {"bytes": 27.14e6, "sources": ["dft.cu"], "profile": "profiles/k_rdft_n256_n384.md"},
+    "gkb": {"bytes": 68.67e6, "sources": ["gkb.cu"], "profile": "profiles/k_gkb_n256.md"},
+    "orth": {"bytes": 7.35e6, "sources": ["rtsvd.cu"], "profile": "profiles/k_orth_n256.md"},
+    "svd": {"bytes": 9.77e6, "sources": ["rtsvd.cu"], "profile": "profiles/k_jacobi_n256.md"},
+    "dft": {"bytes": 26.83e6, "sources": ["dft.cu"], "profile": "profiles/k_rdft_n256_n384.md"},
     "dp": {"bytes": 17.68e6, "sources": ["rtsvd.cu"], "profile": "profiles/launches_n256_bench_step.md"},
 }
 
